@@ -46,7 +46,9 @@ struct fm_ctx {
     int hist_gen = 0;      // bumped when the history buffers move (captured graphs hold them)
     int* istate = nullptr;
     int* icint = nullptr;  // IC sweeps: [0] forward ticket, [1] back-substitution ticket, [2] its done count, [3] pad
-    int* order = nullptr;
+    int* order = nullptr;      // claim orders of all tiles: forward, then the back substitution's
+    int* order_act = nullptr;  // the same without the tiles the mask leaves empty
+    int* tile_rng = nullptr;   // per tile: hyperplanes that hold a mask voxel
     int ntx = 0, nty = 0, ntz = 0, ntiles = 0;
     int ic_wxy = 2, ic_wz = 1;  // forward tile claim order weights
     int nsm = 0, grid_data = 0, grid_ls = 0, grid_ic = 0, grid_icb = 0;  // grid_icb: backward IC sweep
@@ -129,7 +131,7 @@ void free_all(fm_ctx* c) {
                 if (e) cudaEventDestroy(e);
     void* bufs[] = {c->pairs, c->coils, c->w0, c->nb, c->vlist, c->chunk_off, c->w[0], c->w[1], c->z[0], c->z[1], c->g[0],
                     c->g[1], c->d, c->p, c->v, c->ip, c->scal, c->partials, c->face, c->tile_part, c->rho,
-                    c->hist_cost, c->hist_alpha, c->hist_mu, c->istate, c->icint, c->order, c->ict_L,
+                    c->hist_cost, c->hist_alpha, c->hist_mu, c->istate, c->icint, c->order, c->order_act, c->tile_rng, c->ict_L,
                     c->st_y[0], c->st_y[1], c->st_s[0], c->st_s[1], c->st_m[0], c->st_m[1], c->w_io, c->ip_lo,
                     c->ict_tab, c->ict_qflags, c->ict_w0};
     for (void* b : bufs)
@@ -219,7 +221,8 @@ IcArgs ic_args(fm_ctx* c) {
     a.nty = c->nty;
     a.ntz = c->ntz;
     a.ntiles = c->ntiles;
-    a.order = c->order;
+    a.order = c->order_act;
+    a.range = c->tile_rng;
     a.beta = c->beta;
     a.nb = c->nb;
     a.face = c->face;
@@ -269,7 +272,7 @@ cudaError_t run_ic0(fm_ctx* c, const void* d, const void* g, void* p, const void
     IcArgs b = ic_args(c);
     b.ticket = c->icint + 1;
     b.done = c->icint + 2;
-    b.order = c->order + c->ntiles;
+    b.order = c->order_act + c->ntiles;
     b.vin = c->v;
     b.ipb = c->ip;
     b.p = p;
@@ -822,7 +825,7 @@ int implicit_t(fm_ctx* c, const void* y, const void* smap, const void* w_hat, co
 // predecessors and 14 steps plus one hand-off behind its z predecessor, so the forward order
 // takes wxy : wz (default 2 : 1) and the back substitution walks FM_IC_BXY : FM_IC_BZ
 // (2 : 1; measured on the 256 x 256 x 128 volume against 1 : 1 and 3 : 2) backwards.
-// Uploads both orders synchronously.
+// Uploads both orders synchronously and relists the tiles of the current mask.
 bool set_ic_order(fm_ctx* c, int wxy, int wz) {
     std::vector<int> ord(2 * (size_t)c->ntiles);
     const int ntx = c->ntx, nty = c->nty;
@@ -838,7 +841,9 @@ bool set_ic_order(fm_ctx* c, int wxy, int wz) {
     }
     c->ic_wxy = wxy;
     c->ic_wz = wz;
-    return cudaMemcpy(c->order, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
+    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;  // launches that read the order are done
+    if (cudaMemcpy(c->order, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return false;
+    return !c->have_data || launch_ic_order(c->order, c->tile_rng, c->ntiles, c->order_act, c->istate, c->stream) == cudaSuccess;
 }
 
 // Cooperative line-search grid: every block must be co-resident, so the grid follows the
@@ -1020,7 +1025,9 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     A(&c->tile_part, 2 * (size_t)c->ntiles * sizeof(double));
     A(&c->istate, I_NISTATE * sizeof(int));
     A(&c->icint, 4 * sizeof(int));
-    A(&c->order, 2 * (size_t)c->ntiles * sizeof(int));  // forward order, then the back substitution's
+    A(&c->order, 2 * (size_t)c->ntiles * sizeof(int));
+    A(&c->order_act, 2 * (size_t)c->ntiles * sizeof(int));
+    A(&c->tile_rng, (size_t)c->ntiles * sizeof(int));
 
     if (!ok) { cudaGetLastError(); return bail(FM_ERR_OOM); }
 #ifndef FM_IC_WXY
@@ -1150,7 +1157,11 @@ int fm_set_data(fm_ctx* c, const void* y, const void* smap, const double* te, co
     a.istate = c->istate;
     cudaError_t e = c->o.precision == FM_FP64 ? launch_setup<double>(a, c->stream)
                                               : launch_setup<float>(a, c->stream);
+    if (e == cudaSuccess) e = launch_ic_ranges(a.geo, c->ntx, c->nty, c->ntiles, c->nb, c->tile_rng, c->stream);
+    if (e == cudaSuccess) e = launch_ic_order(c->order, c->tile_rng, c->ntiles, c->order_act, c->istate, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "setup kernel");
+    // the IC sweeps leave out tiles outside the mask: their inverse pivots are 0
+    FM_CK(cudaMemsetAsync(c->ip, 0, (size_t)c->nv * c->ts, c->stream), "clear pivots");
     // rows outside the new mask must read as empty in the drop-tolerance factor
     if (c->ict_L)
         FM_CK(cudaMemsetAsync(c->ict_L, 0, (size_t)c->ict_nplanes * c->nv * sizeof(double), c->stream), "clear factor");
@@ -1305,6 +1316,8 @@ int fm_ic_apply(fm_ctx* c, const void* g, void* p) {
         if (e == cudaSuccess)
             e = f64 ? launch_rb_red<double>(a, c->grid_data, c->stream) : launch_rb_red<float>(a, c->grid_data, c->stream);
     } else {
+        // the sweeps leave out tiles outside the mask
+        if (c->o.precond != FM_PC_ICT) FM_CK(cudaMemsetAsync(p, 0, (size_t)c->nv * c->ts, c->stream), "clear");
         e = c->o.precision == FM_FP64 ? run_ic<double>(c, nullptr, g, p, nullptr, nullptr)
                                       : run_ic<float>(c, nullptr, g, p, nullptr, nullptr);
     }

@@ -43,6 +43,7 @@ enum Scal {
 enum IState {
     I_ERR = 0, I_ITER, I_DONE0, I_DONE1, I_BAR_COUNT, I_BAR_GEN, I_NMASK, I_CG_IT, I_CG_DONE,
     I_ICT_BAD,  // drop-tolerance IC: a pivot <= 0 on the held pattern (reported after the fill check)
+    I_NTILE,    // IC tiles that hold a mask voxel
     I_NISTATE
 };
 
@@ -259,7 +260,8 @@ struct DataArgs {
 struct IcArgs {
     Geo geo;
     int ntx, nty, ntz, ntiles;
-    const int* order;      // [ntiles] tiles in a dependency-respecting order
+    const int* order;      // [istate[I_NTILE]] tiles that hold a mask voxel, in a dependency-respecting order
+    const int* range;      // [ntiles] local hyperplanes that hold a mask voxel (tile_range)
     int* ticket;           // claim counter
     int* done;             // finished-tile counter
     double beta;
@@ -373,6 +375,9 @@ template <typename T> cudaError_t launch_pdiag(const DataArgs& a, int mode, int 
 template <typename T> int ls_max_blocks_per_sm(const DataArgs& a);
 template <typename T> cudaError_t launch_rb_black(const DataArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_rb_red(const DataArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, int* range,
+                             cudaStream_t s);
+cudaError_t launch_ic_order(const int* order, const int* range, int ntiles, int* out, int* istate, cudaStream_t s);
 template <typename T> cudaError_t launch_ic_fwd(const IcArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_ic_bwd(const IcArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_inv_pivot64(const float* hi, const float* lo, double* out, long long nv, int grid, cudaStream_t s);

@@ -26,6 +26,16 @@
 // of waiting for them to finish.  The row-coalesced write-back of the whole tile follows the
 // sweep.
 //
+// Support mask.  A voxel outside the mask has 1/pi = v = p = 0 whatever its neighbours hold, so
+// the sweeps leave out what the mask leaves empty.  fm_set_data records, per tile, the first
+// and last local hyperplane that holds a mask voxel (k_ic_range) and lists the tiles that hold
+// any (k_ic_order).  Only listed tiles are claimed, a tile sweeps its own hyperplanes only, and
+// a face entry is handed over only where the producer's and the consumer's hyperplanes both
+// reach it (both sides evaluate the same test); every other incoming entry is 0.  An ellipsoid
+// mask fills a quarter of its grid, and the chain through it is about half as long as the
+// grid's: 256 x 256 x 128 voxels, forward 271 -> 128 us, back substitution 194 -> 118 us.
+// Without a mask every tile keeps its 70 hyperplanes and nothing changes.
+//
 // Pivot arithmetic.  FP64 mode uses IEEE double.  FP32 mode carries each inverse pivot as
 // an unevaluated pair a + b of floats (about 46 significant bits, like double-float), but
 // arranged so that the hi part a is exactly the float recurrence a_j = 1/fl(H - beta^2 sum a_k)
@@ -267,6 +277,79 @@ __device__ __forceinline__ int out_face_vox(int i, bool fwd) {
     return vox(k & 31, k >> 5, fwd ? kTZ - 1 : 0);
 }
 
+// Hyperplanes of a tile that hold a mask voxel, first | last << 8 (an empty tile: 255, none
+// after it), as the sweeps read them.
+struct Range {
+    int lo, hi;
+    __device__ __forceinline__ bool has(int s) const { return s >= lo && s <= hi; }
+};
+__device__ __forceinline__ Range tile_range(const int* range, int tile) {
+    if (tile < 0) return {255, 0};
+    const int r = range[tile];
+    return {r & 255, r >> 8};
+}
+
+// One block per tile, one thread per (y, z) row.
+__global__ void __launch_bounds__(kCompute) k_ic_range(Geo geo, int ntx, int nty, const uint8_t* nb, int* range) {
+    const int tile = blockIdx.x, X = tile % ntx, Y = (tile / ntx) % nty, Z = tile / (ntx * nty);
+    const int ly = threadIdx.x & 31, lz = threadIdx.x >> 5;
+    const int y = Y * 32 + ly, z = Z * kTZ + lz, x0 = X * 32;
+    int lo = 255, hi = 0;
+    if (y < geo.ny && z < geo.nz) {
+        const uint8_t* row = nb + ((long long)z * geo.ny + y) * geo.nx + x0;
+        const int n = min(32, geo.nx - x0);
+        for (int i = 0; i < n; ++i)
+            if (row[i] & NB_IN) {
+                lo = min(lo, i + ly + lz);
+                hi = i + ly + lz;
+            }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    __shared__ int s_lo[kTZ], s_hi[kTZ];
+    if (ly == 0) {
+        s_lo[lz] = lo;
+        s_hi[lz] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kTZ; ++w) {
+            lo = min(lo, s_lo[w]);
+            hi = max(hi, s_hi[w]);
+        }
+        range[tile] = lo | hi << 8;
+    }
+}
+
+// The non-empty tiles of both claim orders (order[0..ntiles) forward, order[ntiles..) for the
+// back substitution), kept in order: one block per claim order.
+__global__ void __launch_bounds__(1024) k_ic_order(const int* order, const int* range, int ntiles, int* out,
+                                                   int* istate) {
+    __shared__ int s_warp[32], s_base;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const size_t off = (size_t)blockIdx.x * ntiles;
+    if (threadIdx.x == 0) s_base = 0;
+    __syncthreads();
+    for (int b = 0; b < ntiles; b += 1024) {
+        const int i = b + threadIdx.x;
+        const int t = i < ntiles ? order[off + i] : -1;
+        const bool keep = t >= 0 && (range[t] & 255) != 255;
+        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+        if (lane == 0) s_warp[wid] = __popc(bal);
+        __syncthreads();
+        int at = s_base, tot = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < wid) at += s_warp[w];
+            tot += s_warp[w];
+        }
+        if (keep) out[off + at + __popc(bal & ((1u << lane) - 1u))] = t;
+        __syncthreads();
+        if (threadIdx.x == 0) s_base += tot;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) istate[I_NTILE] = s_base;
+}
+
 // ------------------------------------------------------------------ streamed faces
 //
 // A forward tile's sweep does not wait for its predecessor tiles to finish: every voxel of a
@@ -457,42 +540,46 @@ __global__ void __launch_bounds__(kThreadsIC) k_ic_fwd(IcArgs a, PivScal pc) {
 
     if (tid == 0)
         for (int c = 0; c < kNch; ++c) mbar_init(&s_mbar[c], 1);
-    unsigned par = 0;  // phase parity of this CTA's current tile
+    const int ntile = a.istate[I_NTILE];
+    unsigned par = 0;  // bit c: phase parity of chunk c's barrier (one phase per tile that has the chunk)
     for (;;) {
         if (tid == 0) {
             const int t = atomicAdd(a.ticket, 1);
-            s_tile = t < a.ntiles ? a.order[t] : -1;
+            s_tile = t < ntile ? a.order[t] : -1;
         }
         __syncthreads();
         const int tile = s_tile;
         if (tile < 0) break;
         const int X = tile % a.ntx, Y = (tile / a.ntx) % a.nty, Z = tile / (a.ntx * a.nty);
         const int x0 = X * 32, y0 = Y * 32, z0 = Z * kTZ;
+        const Range rg = tile_range(a.range, tile);
+        const int nch = (rg.hi - rg.lo) / kCS + 1;
 
         if (wz >= kTZ) {
             // fetch warps: the -x, -y, -z neighbours' outgoing +x, +y, +z faces, alternate chunks each
             const int sx = X > 0 ? tile - 1 : -1, sy = Y > 0 ? tile - a.ntx : -1;
             const int sz = Z > 0 ? tile - a.ntx * a.nty : -1;
+            const Range rx = tile_range(a.range, sx), ry = tile_range(a.range, sy), rz = tile_range(a.range, sz);
             bool ok = true;
-            for (int c = wz - kTZ; c < kNch; c += kFetchF) {
+            for (int c = wz - kTZ; c < nch; c += kFetchF) {
                 P zp[kCS], qp[kCS];
                 T zv[kCS], qv[kCS];
                 int zi[kCS], zg[kCS], qi[kCS], qsrc[kCS];
                 unsigned want = 0;  // bit q: z entry of step q; bit kCS + q: x / y entry
 #pragma unroll
                 for (int q = 0; q < kCS; ++q) {
-                    const int s = c * kCS + q;
+                    const int s = rg.lo + c * kCS + q;
                     int which = 0;
-                    zi[q] = s < kSteps ? z_entry(s, lane) : -1;
+                    zi[q] = s <= rg.hi ? z_entry(s, lane) : -1;
                     zg[q] = FN::z + zdiag(min(s, 62)) + lane;
-                    qi[q] = s < kSteps ? xy_entry(s, lane, which) : -1;
+                    qi[q] = s <= rg.hi ? xy_entry(s, lane, which) : -1;
                     qsrc[q] = which ? sy : sx;
                     zp[q] = Ops::zero();
                     qp[q] = Ops::zero();
                     zv[q] = T(0);
                     qv[q] = T(0);
-                    if (zi[q] >= 0 && sz >= 0) want |= 1u << q;
-                    if (qi[q] >= 0 && qsrc[q] >= 0) want |= 1u << (kCS + q);
+                    if (zi[q] >= 0 && rz.has(s + kTZ - 1)) want |= 1u << q;
+                    if (qi[q] >= 0 && (which ? ry : rx).has(s + 31)) want |= 1u << (kCS + q);
                 }
                 // poll until every wanted entry is set (all of a round's loads are in flight
                 // together); a wait that gives up leaves zeros and reports the timeout
@@ -561,6 +648,11 @@ __global__ void __launch_bounds__(kThreadsIC) k_ic_fwd(IcArgs a, PivScal pc) {
                     if (Ops::kLo) lr[i] = hL;
                 }
             }
+            // hyperplanes before the first are 0: the z exchange starts from that
+            for (int i = tid; i < 2 * kTZ * 32; i += kCompute) {
+                zb_v[i] = T(0);
+                if (mode == 0) zb_ip[i] = Ops::zero();
+            }
             bar_compute();
 
             // sweep the local hyperplanes s = lx + ly + lz.  The body is branch-free: a lane
@@ -576,18 +668,22 @@ __global__ void __launch_bounds__(kThreadsIC) k_ic_fwd(IcArgs a, PivScal pc) {
             const int zr = (lz > 0 ? lz - 1 : 0) * 32 + ly, zw = lz * 32 + ly;
             P* oip = face_ip(tile);
             T* ov = face_v(tile);
+            // steps whose face entries a successor reads
+            const Range ux = tile_range(a.range, X + 1 < a.ntx ? tile + 1 : -1);
+            const Range uy = tile_range(a.range, Y + 1 < a.nty ? tile + a.ntx : -1);
+            const Range uz = tile_range(a.range, Z + 1 < a.ntz ? tile + a.ntx * a.nty : -1);
             P out_ip = Ops::zero();
             T out_v = 0;
             bool bad = false;
             // zdiag(t) - max(0, t - 31) for this warp's current diagonal t = s - lz (0 while t < 0):
             // the z-face entry of lane ly at step s is FN::z + zbase + lx
-            int zbase = 0;
-            for (int c = 0; c < kNch; ++c) {
-              wait_chunk(&s_mbar[c], par, a.spin_limit, a.istate);
+            int zbase = rg.lo > lz ? zdiag(min(rg.lo - lz, 62)) - max(0, rg.lo - lz - 31) : 0;
+            for (int c = 0; c < nch; ++c) {
+              wait_chunk(&s_mbar[c], (par >> c) & 1u, a.spin_limit, a.istate);
 #pragma unroll
               for (int q = 0; q < kCS; ++q) {
-                const int s = c * kCS + q;
-                if (kSteps % kCS != 0 && s >= kSteps) break;
+                const int s = rg.lo + c * kCS + q;
+                if (s > rg.hi) break;
                 const P up_ip = shfl_up(out_ip);
                 const T up_v = __shfl_up_sync(0xffffffffu, out_v, 1);
                 const int lx = s - l0;
@@ -631,7 +727,8 @@ __global__ void __launch_bounds__(kThreadsIC) k_ic_fwd(IcArgs a, PivScal pc) {
                 out_v = vj;
                 zb_v[par + zw] = vj;
                 // outgoing faces go out as they are produced
-                const bool fx_out = act & (lx == 31), fy_out = act & (ly == 31), fz_out = act & (lz == kTZ - 1);
+                const bool fx_out = act & (lx == 31) & ux.has(s - 31), fy_out = act & (ly == 31) & uy.has(s - 31),
+                           fz_out = act & (lz == kTZ - 1) & uz.has(s - (kTZ - 1));
                 const int zo = FN::z + zbase + lw;
                 if constexpr (MODE == 0) {
                     st_if(fx_out, oip + FN::x + zw, ipj);
@@ -659,21 +756,23 @@ __global__ void __launch_bounds__(kThreadsIC) k_ic_fwd(IcArgs a, PivScal pc) {
                 unset_faces<T>(sx >= 0 ? face_v(sx) : nullptr, sy >= 0 ? face_v(sy) : nullptr,
                                sz >= 0 ? face_v(sz) : nullptr);
             }
-            // write back row-coalesced (warp lz writes its 32 rows, lane = x)
+            // write back row-coalesced (warp lz writes its 32 rows, lane = x); a voxel on a hyperplane
+            // that was not swept lies outside the mask
             const int nvalid = min(32, nx - x0);
             const int z = z0 + wz;
             if (z < nz && lane < nvalid) {
                 for (int ly2 = 0; ly2 < 32 && y0 + ly2 < ny; ++ly2) {
                     const long long j = (long long)z * nxy + (long long)(y0 + ly2) * nx + x0 + lane;
                     const int i = (wz * 32 + ly2) * 32 + lane;
-                    v[j] = sg[i];
-                    if (mode == 0 && ipo) ipo[j] = sd[i];
-                    if (Ops::kLo && mode == 0 && a.ip_lo_out) a.ip_lo_out[j] = (float)sl[i];
+                    const bool in = rg.has(lane + ly2 + wz);
+                    v[j] = in ? sg[i] : T(0);
+                    if (mode == 0 && ipo) ipo[j] = in ? sd[i] : T(0);
+                    if (Ops::kLo && mode == 0 && a.ip_lo_out) a.ip_lo_out[j] = in ? (float)sl[i] : 0.0f;
                 }
             }
         }
         __syncthreads();
-        par ^= 1u;
+        par ^= (1u << nch) - 1u;
     }
 }
 
@@ -713,7 +812,7 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
     T* sip = sv + kTZ * 1024;         // 1/pi
     T* f_p = sip + kTZ * 1024;        // incoming faces (the successors' -x, -y, -z faces)
     T* zb = f_p + FN::n;              // [2][TZ][32]
-    __shared__ int s_tile;
+    __shared__ int s_tile, s_claim;
     constexpr int kCS = kCSB, kNch = (kSteps + kCS - 1) / kCS;
     __shared__ __align__(8) unsigned long long s_mbar[kNch];
     __shared__ bool s_last;
@@ -735,28 +834,34 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
         return (T*)(faceb + (size_t)t * face_bytes_per_tile<T>() + (size_t)FN::n * (sizeof(P) + sizeof(T)));
     };
 
+    const int ntile = a.istate[I_NTILE];
     if (tid == 0) {
         s_last = false;
         for (int c = 0; c < kNch; ++c) mbar_init(&s_mbar[c], 1);
+        if (ntile == 0 && blockIdx.x == 0 && a.tile_part) a.scal[S_GP] = a.scal[S_GPREVP] = 0.0;  // empty mask
     }
-    unsigned par = 0;  // phase parity of this CTA's current tile
+    unsigned par = 0;  // bit c: phase parity of chunk c's barrier
     for (;;) {
         if (tid == 0) {
             const int t = atomicAdd(a.ticket, 1);
-            s_tile = t < a.ntiles ? a.order[a.ntiles - 1 - t] : -1;
+            s_claim = t;
+            s_tile = t < ntile ? a.order[ntile - 1 - t] : -1;
         }
         __syncthreads();
         const int tile = s_tile;
         if (tile < 0) break;
         const int X = tile % a.ntx, Y = (tile / a.ntx) % a.nty, Z = tile / (a.ntx * a.nty);
         const int x0 = X * 32, y0 = Y * 32, z0 = Z * kTZ;
+        const Range rg = tile_range(a.range, tile);
+        const int nch = (rg.hi - rg.lo) / kCS + 1;
 
         if (wz >= kTZ) {
             // fetch warps: the +x, +y, +z neighbours' outgoing low faces, alternate chunks each
             const int sx = X + 1 < a.ntx ? tile + 1 : -1, sy = Y + 1 < a.nty ? tile + a.ntx : -1;
             const int sz = Z + 1 < a.ntz ? tile + a.ntx * a.nty : -1;
+            const Range rx = tile_range(a.range, sx), ry = tile_range(a.range, sy), rz = tile_range(a.range, sz);
             bool ok = true;
-            for (int c = wz - kTZ; c < kNch; c += kFetchB) {
+            for (int c = wz - kTZ; c < nch; c += kFetchB) {
                 T zv[kCS], qv[kCS];
                 int zi[kCS], zg[kCS], qi[kCS], qsrc[kCS];
                 unsigned want = 0;
@@ -764,17 +869,17 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
                 for (int q = 0; q < kCS; ++q) {
                     // reverse step c * kCS + q is local hyperplane s; the +z face entry (lx, ly) is
                     // used at s = lx + ly + kTZ - 1, the +x / +y entries at s = 31 + ly + lz / lx + lz
-                    const int s = kSteps - 1 - (c * kCS + q);
+                    const int s = rg.hi - (c * kCS + q);
                     int which = 0;
-                    const bool in = s >= 0;
+                    const bool in = s >= rg.lo;
                     zi[q] = in ? z_entry(s - (kTZ - 1), lane) : -1;
                     zg[q] = FN::z + zdiag(min(max(s - (kTZ - 1), 0), 62)) + lane;
                     qi[q] = in ? xy_entry(s - 31, lane, which) : -1;
                     qsrc[q] = which ? sy : sx;
                     zv[q] = T(0);
                     qv[q] = T(0);
-                    if (zi[q] >= 0 && sz >= 0) want |= 1u << q;
-                    if (qi[q] >= 0 && qsrc[q] >= 0) want |= 1u << (kCS + q);
+                    if (zi[q] >= 0 && rz.has(s - (kTZ - 1))) want |= 1u << q;
+                    if (qi[q] >= 0 && (which ? ry : rx).has(s - 31)) want |= 1u << (kCS + q);
                 }
                 unsigned todo = ok ? want : 0u;
                 long long tries = 0;
@@ -815,6 +920,7 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
             stage_row<T>(sv, vin, tid, x0, y0, z0, geo, T(0));
             stage_row<T>(sip, ipb, tid, x0, y0, z0, geo, T(0));
             cp_wait_all();
+            for (int i = tid; i < 2 * kTZ * 32; i += kCompute) zb[i] = T(0);  // hyperplanes after the last are 0
             bar_compute();
 
             // sweep in reverse, branch-free as in the forward kernel; the low-face entries a chunk
@@ -826,14 +932,18 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
             const T* fz = f_p + FN::z + ly * 32;
             const int zr = (lz < kTZ - 1 ? lz + 1 : lz) * 32 + ly, zw = lz * 32 + ly;
             T* op = face_p(tile);
+            // steps whose face entries a successor reads
+            const Range ux = tile_range(a.range, X > 0 ? tile - 1 : -1);
+            const Range uy = tile_range(a.range, Y > 0 ? tile - a.ntx : -1);
+            const Range uz = tile_range(a.range, Z > 0 ? tile - a.ntx * a.nty : -1);
             T out = 0;
-            for (int c = 0; c < kNch; ++c) {
-                wait_chunk(&s_mbar[c], par, a.spin_limit, a.istate);
+            for (int c = 0; c < nch; ++c) {
+                wait_chunk(&s_mbar[c], (par >> c) & 1u, a.spin_limit, a.istate);
                 const T fxv = f_p[fxi];  // used at s = 31 + l0, in the chunk whose fetch brought it
 #pragma unroll
                 for (int q = 0; q < kCS; ++q) {
-                    const int s = kSteps - 1 - (c * kCS + q);
-                    if (kSteps % kCS != 0 && s < 0) break;
+                    const int s = rg.hi - (c * kCS + q);
+                    if (s < rg.lo) break;
                     const T dn = __shfl_down_sync(0xffffffffu, out, 1);
                     const int lx = s - l0;
                     const bool act = (unsigned)lx < 32u;
@@ -857,14 +967,14 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
                 // this thread's lx = 0 voxel, produced at s = l0; y face (lx, lz) was produced by
                 // lane 0 of warp lz, one per step, and lane q stores step s1 - q; z face diagonal
                 // s1 - wz (warps 0..kCS-1) holds entries (lx, ly) of the lz = 0 plane
-                const int s1 = kSteps - 1 - c * kCS, s0 = max(s1 - kCS + 1, 0);
+                const int s1 = rg.hi - c * kCS, s0 = max(s1 - kCS + 1, rg.lo);
                 const int sy_ = s1 - lane, lxy = sy_ - lz;
                 const int sz_ = s1 - wz, lxz = sz_ - ly;
                 const T vx = sv[row], vy = sv[lz * 1024 + (lxy & 31)], vz = sv[ly * 32 + (lxz & 31)];
                 const int zo = FN::z + zdiag(min(max(sz_, 0), 62)) - max(0, sz_ - 31) + (lxz & 31);
-                st_if(l0 >= s0 && l0 <= s1, op + FN::x + zw, canon(vx));
-                st_if(lane < kCS && sy_ >= s0 && (unsigned)lxy < 32u, op + FN::y + lz * 32 + (lxy & 31), canon(vy));
-                st_if(wz < kCS && sz_ >= s0 && (unsigned)lxz < 32u, op + zo, canon(vz));
+                st_if(l0 >= s0 && l0 <= s1 && ux.has(l0 + 31), op + FN::x + zw, canon(vx));
+                st_if(lane < kCS && sy_ >= s0 && (unsigned)lxy < 32u && uy.has(sy_ + 31), op + FN::y + lz * 32 + (lxy & 31), canon(vy));
+                st_if(wz < kCS && sz_ >= s0 && (unsigned)lxz < 32u && uz.has(sz_ + kTZ - 1), op + zo, canon(vz));
             }
 
             {
@@ -915,11 +1025,11 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
             if (a.tile_part) {
                 block_sum_compute(acc, sbuf);
                 if (tid == 0) {
-                    a.tile_part[tile] = acc[0];
-                    a.tile_part[a.ntiles + tile] = acc[1];
+                    a.tile_part[s_claim] = acc[0];  // by claim position: the order is fixed, so is the sum
+                    a.tile_part[ntile + s_claim] = acc[1];
                     __threadfence();
                     const int prev = atomicAdd(a.done, 1);
-                    s_last = (prev == a.ntiles - 1);
+                    s_last = (prev == ntile - 1);
                     if (s_last) __threadfence();
                 }
             }
@@ -927,7 +1037,7 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
         __syncthreads();
         if (a.tile_part && s_last) {
             double tot[2];
-            sum_partials<2>(a.tile_part, a.ntiles, tot, sbuf);
+            sum_partials<2>(a.tile_part, ntile, tot, sbuf);
             if (tid == 0) {
                 a.scal[S_GP] = tot[0];
                 a.scal[S_GPREVP] = tot[1];
@@ -936,8 +1046,18 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
             __syncthreads();
             if (tid == 0) s_last = false;
         }
-        par ^= 1u;
+        par ^= (1u << nch) - 1u;
     }
+}
+
+cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, int* range,
+                             cudaStream_t s) {
+    k_ic_range<<<ntiles, kCompute, 0, s>>>(geo, ntx, nty, nb, range);
+    return cudaGetLastError();
+}
+cudaError_t launch_ic_order(const int* order, const int* range, int ntiles, int* out, int* istate, cudaStream_t s) {
+    k_ic_order<<<2, 1024, 0, s>>>(order, range, ntiles, out, istate);
+    return cudaGetLastError();
 }
 
 template <typename T> int ic_tz() { return kTZ; }
