@@ -45,11 +45,12 @@ struct fm_ctx {
     int hist_cap = 0;
     int hist_gen = 0;      // bumped when the history buffers move (captured graphs hold them)
     int* istate = nullptr;
-    int* icint = nullptr;  // IC sweeps: [0] forward ticket, [1] back-substitution ticket, [2] its done count, [3] pad
+    int* icint = nullptr;  // IC sweeps: [0] forward ticket, [1] back-substitution ticket, [2] its done count,
+                           // [3] its unit ticket, [4 ..] its written flags, one per tile
     int* order = nullptr;      // claim orders of all tiles: forward, then the back substitution's
-    int* order_act = nullptr;  // the same without the tiles the mask leaves empty
-    int* tile_rng = nullptr;   // per tile: hyperplanes that hold a mask voxel
-    int ntx = 0, nty = 0, ntz = 0, ntiles = 0;
+    int* order_act = nullptr;  // the same without the tiles the mask leaves empty, and the dot-product units
+    unsigned* tile_rng = nullptr;  // per tile: steps of the sweeps that reach a mask voxel
+    int ntx = 0, nty = 0, ntz = 0, ntiles = 0, npart = 0;
     int ic_wxy = 2, ic_wz = 1;  // forward tile claim order weights
     int nsm = 0, grid_data = 0, grid_ls = 0, grid_ic = 0, grid_icb = 0;  // grid_icb: backward IC sweep
     int base_data = 0, base_ls = 0, base_ic = 0, base_icb = 0;
@@ -249,7 +250,7 @@ cudaError_t run_grad(fm_ctx* c, const void* w_in, const void* zdir, void* w_out,
 template <typename T>
 cudaError_t run_ic0(fm_ctx* c, const void* d, const void* g, void* p, const void* gdot, const void* gpdot,
                     int slot, float* ip_lo = nullptr) {
-    cudaError_t e = cudaMemsetAsync(c->icint, 0, 4 * sizeof(int), c->stream);
+    cudaError_t e = cudaMemsetAsync(c->icint, 0, (4 + (size_t)c->ntiles) * sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
     IcArgs f = ic_args(c);
     f.ticket = c->icint + 0;
@@ -272,13 +273,17 @@ cudaError_t run_ic0(fm_ctx* c, const void* d, const void* g, void* p, const void
     IcArgs b = ic_args(c);
     b.ticket = c->icint + 1;
     b.done = c->icint + 2;
+    b.unit_ticket = c->icint + 3;
+    b.written = c->icint + 4;
     b.order = c->order_act + c->ntiles;
+    b.unit = c->order_act + 2 * (size_t)c->ntiles;
     b.vin = c->v;
     b.ipb = c->ip;
     b.p = p;
     b.gdot = gdot;
     b.gpdot = gpdot;
     b.tile_part = (gdot || gpdot) ? c->tile_part : nullptr;
+    b.npart = c->npart;
     if (slot >= 0 && c->profiling) prof_record(c->ev[slot][FM_K_IC_BWD][0], c->stream);
     e = launch_ic_bwd<T>(b, c->grid_icb, c->stream);
     if (slot >= 0 && c->profiling) {
@@ -813,18 +818,20 @@ int implicit_t(fm_ctx* c, const void* y, const void* smap, const void* w_hat, co
 #define FM_IC_BXY 2
 #endif
 #ifndef FM_IC_BBLK
-#define FM_IC_BBLK 2
+#define FM_IC_BBLK 1
+#endif
+#ifndef FM_IC_FBLK
+#define FM_IC_FBLK 1
 #endif
 #ifndef FM_IC_BZ
 #define FM_IC_BZ 1
 #endif
 
-// Tile claim orders: a weighted tile hyperplane wxy (X + Y) + wz Z (ties: z, y, x).  Every
-// weight is positive, so a tile's -x, -y, -z neighbours always come first.  Both sweeps
-// stream faces, and a tile starts about 38 steps plus one hand-off behind its x / y
-// predecessors and 14 steps plus one hand-off behind its z predecessor, so the forward order
-// takes wxy : wz (default 2 : 1) and the back substitution walks FM_IC_BXY : FM_IC_BZ
-// (2 : 1; measured on the 256 x 256 x 128 volume against 1 : 1 and 3 : 2) backwards.
+// Tile claim orders: a weighted tile hyperplane wxy (4 X + Y) + 2 wz Z (ties: z, y, x), for tiles of
+// 64 x 16 x 8.  Every weight is positive, so a tile's -x, -y, -z neighbours always come first.  Both
+// sweeps stream faces, and a tile starts 63, 15 and 16 steps plus one hand-off behind its x, y and
+// z predecessors; the forward order takes wxy : wz (default 2 : 1) and the back substitution walks
+// FM_IC_BXY : FM_IC_BZ (2 : 1) backwards.
 // Uploads both orders synchronously and relists the tiles of the current mask.
 bool set_ic_order(fm_ctx* c, int wxy, int wz) {
     std::vector<int> ord(2 * (size_t)c->ntiles);
@@ -834,8 +841,8 @@ bool set_ic_order(fm_ctx* c, int wxy, int wz) {
         auto first = ord.begin() + (size_t)pass * c->ntiles;
         for (int t = 0; t < c->ntiles; ++t) first[t] = t;
         std::stable_sort(first, first + c->ntiles, [&](int a, int b) {
-            const int ha = a_xy * (a % ntx + (a / ntx) % nty) + a_z * (a / (ntx * nty));
-            const int hb = a_xy * (b % ntx + (b / ntx) % nty) + a_z * (b / (ntx * nty));
+            const int ha = a_xy * (4 * (a % ntx) + (a / ntx) % nty) + a_z * 2 * (a / (ntx * nty));
+            const int hb = a_xy * (4 * (b % ntx) + (b / ntx) % nty) + a_z * 2 * (b / (ntx * nty));
             return ha != hb ? ha < hb : a < b;
         });
     }
@@ -843,7 +850,7 @@ bool set_ic_order(fm_ctx* c, int wxy, int wz) {
     c->ic_wz = wz;
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;  // launches that read the order are done
     if (cudaMemcpy(c->order, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return false;
-    return !c->have_data || launch_ic_order(c->order, c->tile_rng, c->ntiles, c->order_act, c->istate, c->stream) == cudaSuccess;
+    return !c->have_data || launch_ic_order(c->order, c->tile_rng, c->ntx, c->nty, c->ntiles, c->order_act, c->istate, c->stream) == cudaSuccess;
 }
 
 // Cooperative line-search grid: every block must be co-resident, so the grid follows the
@@ -969,15 +976,15 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     c->ntz = (nz + tz - 1) / tz;
     c->ntiles = c->ntx * c->nty * c->ntz;
     {
-        // the two sweeps claim tiles from their own tickets, so each sizes its own grid: the
-        // forward sweep by its footprint (1 block/SM), the back substitution by its footprint
-        // capped at 2 blocks/SM -- a third block per SM only adds tiles waiting on their
-        // successors' flags (256x256x128 volume: 0.328 / 0.284 / 0.293 ms per sweep at 1 / 2 / 3)
+        // the two sweeps claim tiles from their own tickets, so each sizes its own grid: one block
+        // per SM, as a second slows the other's steps (256x256x128 volume: forward 122 / 149 us per
+        // sweep at 1 / 2; back substitution on 192x192x96 71 / 77); a batch may take more
+        // (fm_batch_autotune)
         const bool f64 = o.precision == FM_FP64;
         const int occ_f = f64 ? ic_max_blocks_per_sm<double>(false) : ic_max_blocks_per_sm<float>(false);
         const int occ_b = f64 ? ic_max_blocks_per_sm<double>(true) : ic_max_blocks_per_sm<float>(true);
         if (occ_f < 1 || occ_b < 1) return bail(FM_ERR_CUDA);
-        c->grid_ic = std::max(1, std::min(c->ntiles, occ_f * c->nsm));
+        c->grid_ic = std::max(1, std::min(c->ntiles, std::min(occ_f, FM_IC_FBLK) * c->nsm));
         c->grid_icb = std::max(1, std::min(c->ntiles, std::min(occ_b, FM_IC_BBLK) * c->nsm));
         c->occ_icb = occ_b;
     }
@@ -1022,12 +1029,13 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     c->face_bytes = (size_t)c->ntiles *
                     (o.precision == FM_FP64 ? ic_face_bytes_per_tile<double>() : ic_face_bytes_per_tile<float>());
     A(&c->face, c->face_bytes);
-    A(&c->tile_part, 2 * (size_t)c->ntiles * sizeof(double));
+    c->npart = (int)((long long)((nx + 31) / 32) * ((ny + 31) / 32) * c->ntz);  // blocks of 32 x 32 x 8
+    A(&c->tile_part, 2 * (size_t)c->npart * sizeof(double));
     A(&c->istate, I_NISTATE * sizeof(int));
-    A(&c->icint, 4 * sizeof(int));
+    A(&c->icint, (4 + (size_t)c->ntiles) * sizeof(int));
     A(&c->order, 2 * (size_t)c->ntiles * sizeof(int));
-    A(&c->order_act, 2 * (size_t)c->ntiles * sizeof(int));
-    A(&c->tile_rng, (size_t)c->ntiles * sizeof(int));
+    A(&c->order_act, 3 * (size_t)c->ntiles * sizeof(int));  // and the dot-product units
+    A(&c->tile_rng, (size_t)c->ntiles * sizeof(unsigned));
 
     if (!ok) { cudaGetLastError(); return bail(FM_ERR_OOM); }
 #ifndef FM_IC_WXY
@@ -1158,9 +1166,11 @@ int fm_set_data(fm_ctx* c, const void* y, const void* smap, const double* te, co
     cudaError_t e = c->o.precision == FM_FP64 ? launch_setup<double>(a, c->stream)
                                               : launch_setup<float>(a, c->stream);
     if (e == cudaSuccess) e = launch_ic_ranges(a.geo, c->ntx, c->nty, c->ntiles, c->nb, c->tile_rng, c->stream);
-    if (e == cudaSuccess) e = launch_ic_order(c->order, c->tile_rng, c->ntiles, c->order_act, c->istate, c->stream);
+    if (e == cudaSuccess) e = launch_ic_order(c->order, c->tile_rng, c->ntx, c->nty, c->ntiles, c->order_act, c->istate, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "setup kernel");
-    // the IC sweeps leave out tiles outside the mask: their inverse pivots are 0
+    // the IC sweeps leave out tiles outside the mask: their inverse pivots and their part of the dot
+    // products are 0
+    FM_CK(cudaMemsetAsync(c->tile_part, 0, 2 * (size_t)c->npart * sizeof(double), c->stream), "clear sums");
     FM_CK(cudaMemsetAsync(c->ip, 0, (size_t)c->nv * c->ts, c->stream), "clear pivots");
     // rows outside the new mask must read as empty in the drop-tolerance factor
     if (c->ict_L)

@@ -44,6 +44,7 @@ enum IState {
     I_ERR = 0, I_ITER, I_DONE0, I_DONE1, I_BAR_COUNT, I_BAR_GEN, I_NMASK, I_CG_IT, I_CG_DONE,
     I_ICT_BAD,  // drop-tolerance IC: a pivot <= 0 on the held pattern (reported after the fill check)
     I_NTILE,    // IC tiles that hold a mask voxel
+    I_NUNIT,    // dot-product units of the IC back substitution
     I_NISTATE
 };
 
@@ -261,7 +262,7 @@ struct IcArgs {
     Geo geo;
     int ntx, nty, ntz, ntiles;
     const int* order;      // [istate[I_NTILE]] tiles that hold a mask voxel, in a dependency-respecting order
-    const int* range;      // [ntiles] local hyperplanes that hold a mask voxel (tile_range)
+    const unsigned* range; // [ntiles] steps that reach a mask voxel (tile_range)
     int* ticket;           // claim counter
     int* done;             // finished-tile counter
     double beta;
@@ -280,7 +281,11 @@ struct IcArgs {
     void* p;               // T [nv]
     const void* gdot;      // T [nv] or null: g for g'p
     const void* gpdot;     // T [nv] or null: g_prev for g_prev'p
-    double* tile_part;     // [2][ntiles]
+    double* tile_part;     // [2][npart] sums of 32 x 32 x 8 voxel blocks, or null: no dot products
+    int npart;
+    const int* unit;       // [istate[I_NUNIT]] tiles that stand for a dot-product unit, in claim order
+    int* written;          // [ntiles] 1 once a tile's p is in memory (0 before the launch)
+    int* unit_ticket;      // claim counter of the units
     double* scal;
     int* istate;
     long long spin_limit;
@@ -375,9 +380,10 @@ template <typename T> cudaError_t launch_pdiag(const DataArgs& a, int mode, int 
 template <typename T> int ls_max_blocks_per_sm(const DataArgs& a);
 template <typename T> cudaError_t launch_rb_black(const DataArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_rb_red(const DataArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, int* range,
+cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, unsigned* range,
                              cudaStream_t s);
-cudaError_t launch_ic_order(const int* order, const int* range, int ntiles, int* out, int* istate, cudaStream_t s);
+cudaError_t launch_ic_order(const int* order, const unsigned* range, int ntx, int nty, int ntiles, int* out, int* istate,
+                            cudaStream_t s);
 template <typename T> cudaError_t launch_ic_fwd(const IcArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_ic_bwd(const IcArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_inv_pivot64(const float* hi, const float* lo, double* out, long long nv, int grid, cudaStream_t s);
@@ -404,6 +410,6 @@ template <typename T> size_t ic_face_bytes_per_tile();
 template <typename T> int ic_max_blocks_per_sm(bool bwd);  // resident IC sweep blocks per SM
 
 constexpr int kThreads = 256;     // data-term / stencil kernels
-constexpr int kTileX = 32, kTileY = 32;
+constexpr int kTileX = 64, kTileY = 16;  // IC sweep tiles (k_ic.cu)
 
 }  // namespace fm

@@ -12,29 +12,44 @@
 // Voxels outside the mask are identity rows with 1/pi = v = p = 0, so every sum may run over
 // all grid neighbours: an outside neighbour contributes exactly 0.
 //
-// Parallel schedule: voxel (x, y, z) depends on (x-1, y, z), (x, y-1, z), (x, y, z-1), so
-// every hyperplane x + y + z = const is independent.  The grid is cut into 32 x 32 x 8
-// tiles; a CTA claims tiles through an atomic ticket in a dependency-respecting order (a
-// tile's predecessors always hold smaller tickets, so no co-residency is assumed), starts
-// the asynchronous copy of the tile's inputs into shared memory, forms H_jj and sweeps the
-// tile's 70 local hyperplanes: lane = y, warp = z, and each thread walks its x row one step
-// per hyperplane, taking the -y value from the neighbouring lane by shuffle, the -z value
-// from the warp below through shared memory and the -x value from its own register.  The
-// step body is branch-free (divergent branches cost more per step than the idle lanes'
-// arithmetic).  In both sweeps faces stream between tiles while they sweep (see "streamed
-// faces" below): a tile runs a fixed number of hyperplanes behind its predecessors instead
-// of waiting for them to finish.  The row-coalesced write-back of the whole tile follows the
-// sweep.
+// Parallel schedule: voxel (x, y, z) depends on (x-1, y, z), (x, y-1, z), (x, y, z-1).  The grid
+// is cut into 64 x 16 x 8 tiles; a CTA claims tiles through an atomic ticket in a
+// dependency-respecting order (a tile's predecessors always hold smaller tickets, so no
+// co-residency is assumed) and starts the asynchronous copy of the tile's inputs into shared
+// memory.  A warp holds 16 rows (lane & 15 = y) of two planes (lane >> 4), and each thread walks
+// its x row one voxel per step, every row one step behind its -y neighbour and the upper plane
+// one step behind the lower: the -y and -z values come from the neighbouring lanes by shuffle,
+// the -x value from the thread's own register.  The four warps (z pairs) run a chunk of steps
+// plus one behind each other, so that what a warp needs from the warp below was computed a whole
+// chunk earlier: one barrier per chunk, none per step.  Voxel (lx, ly, lz) is computed at step
+// lx + ly + tz(lz).  The back substitution is the same sweep in mirrored coordinates.  In both
+// sweeps faces stream between tiles while they sweep (see "streamed faces" below): a tile runs a
+// fixed number of steps behind its predecessors instead of waiting for them to finish.  The
+// row-coalesced write-back of the whole tile follows the sweep.
+//
+// What bounds the sweeps is latency: the steps of the longest chain of voxels through the tiles
+// times the time of a step, plus a hand-off (about 1.3 us) per tile on it; no pipe is more than a
+// few percent busy.  A step of one warp is a chain of about 25 dependent operations (two shuffles'
+// 24 cycles, the FP32 adds' 4.6 each, the reciprocal), so what a step holds beside that chain decides:
+// measured on one tile, a barrier per step cost 21 to 57 cycles, a branch (a face store under an if) 20 to
+// 35, a load that must follow the step's stores 30.  So a step is registers, shuffles and stores
+// only: everything from outside is loaded per chunk, one record per row and step goes to a ring in
+// shared memory, and a warp of its own publishes the faces from there.  Per step: forward 440 ->
+// 195 cycles, back substitution 200 -> 120, against 32 x 32 x 8 tiles with a warp per plane and a
+// barrier per step.  More than one CTA per SM slows the steps (780 -> 1010 cycles per forward chunk)
+// more than the extra slots give: 256 x 256 x 128, forward 149 us at two, 122 at one.  The long x
+// side keeps the lanes busy (64 of 95 steps) and makes hand-offs along x rare.
 //
 // Support mask.  A voxel outside the mask has 1/pi = v = p = 0 whatever its neighbours hold, so
 // the sweeps leave out what the mask leaves empty.  fm_set_data records, per tile, the first
-// and last local hyperplane that holds a mask voxel (k_ic_range) and lists the tiles that hold
-// any (k_ic_order).  Only listed tiles are claimed, a tile sweeps its own hyperplanes only, and
-// a face entry is handed over only where the producer's and the consumer's hyperplanes both
+// and last step of each sweep that reaches a mask voxel (k_ic_range) and lists the tiles that hold
+// any (k_ic_order).  Only listed tiles are claimed, a tile sweeps its own steps only, and
+// a face entry is handed over only where the producer's and the consumer's steps both
 // reach it (both sides evaluate the same test); every other incoming entry is 0.  An ellipsoid
 // mask fills a quarter of its grid, and the chain through it is about half as long as the
-// grid's: 256 x 256 x 128 voxels, forward 271 -> 128 us, back substitution 194 -> 118 us.
-// Without a mask every tile keeps its 70 hyperplanes and nothing changes.
+// grid's: 256 x 256 x 128 voxels, forward 271 -> 128 us, back substitution 194 -> 118 us (with the
+// 32 x 32 x 8 tiles of the time; 122 and 109 us now).
+// Without a mask every tile keeps all of its steps.
 //
 // Pivot arithmetic.  FP64 mode uses IEEE double.  FP32 mode carries each inverse pivot as
 // an unevaluated pair a + b of floats (about 46 significant bits, like double-float), but
@@ -45,15 +60,13 @@
 //   1/pi = a (1 + e_r - dpi a) + O(eps^2),  e_r = 1 - pi_f a  (exact by FMA),
 // so b = a (e_r - dpi a) with a relative truncation of order (dpi/pi)^2 ~ 1e-14.  The GB300
 // FP64 pipe issues at about 1/64 of the FP32 rate and would sit on the sweep's critical path.
+#include <type_traits>
+
 #include "fm_internal.h"
 
 namespace fm {
 
 // ------------------------------------------------------------------ split pivot (FP32 mode)
-
-struct PF {
-    float a, b;  // inverse pivot = a + b
-};
 
 __device__ __forceinline__ void two_sum(float x, float y, float& s, float& e) {
     s = __fadd_rn(x, y);
@@ -72,73 +85,57 @@ struct PivScal {     // beta-derived constants of the pivot recurrence
     float b2h, b2l;  // beta^2 = b2h + b2l
 };
 
-// Per precision: H_jj = d_j + beta n_j is formed once per voxel while the tile is staged
-// (stored as hi in the d slot, -1 outside the mask, and, in FP32 mode, its low part in a
-// second array); the sweep then only needs 1/pi_j = 1/(H_jj - beta^2 sum_k 1/pi_k).
-template <typename T> struct PivOps;
-template <> struct PivOps<double> {
-    using P = double;
-    static constexpr bool kLo = false;
-    static __device__ __forceinline__ P zero() { return 0.0; }
-    static __device__ __forceinline__ double hi(P x) { return x; }
-    static __device__ __forceinline__ double lo(P) { return 0.0; }
-    static __device__ __forceinline__ P make(double a, double) { return a; }
-    static __device__ __forceinline__ void form_h(double d, int n, double beta, const PivScal&, double& hH,
-                                                  double&) {
-        hH = d + beta * (double)n;
-    }
-    static __device__ __forceinline__ P inv_pivot(double hH, double, double beta, const PivScal&, P x, P y, P z,
-                                                  bool& ok) {
-        const double piv = hH - beta * beta * ((x + y) + z);
-        ok = piv > 0.0;
-        return ok ? 1.0 / piv : 0.0;
-    }
-};
-template <> struct PivOps<float> {
-    using P = PF;
-    static constexpr bool kLo = true;
-    static __device__ __forceinline__ P zero() { return {0.0f, 0.0f}; }
-    static __device__ __forceinline__ float hi(P x) { return x.a; }
-    static __device__ __forceinline__ float lo(P x) { return x.b; }
-    static __device__ __forceinline__ P make(float a, float b) { return {a, b}; }
-    // H = d + beta n as hH + hL (n <= 6, so bh * n has one rounding, recovered by FMA)
-    static __device__ __forceinline__ void form_h(float d, int n, double, const PivScal& c, float& hH, float& hL) {
-        const float fn = (float)n;
-        const float bn = __fmul_rn(c.bh, fn);
-        const float bn_e = __fmaf_rn(c.bh, fn, -bn);
-        float hE;
-        two_sum(d, bn, hH, hE);
-        hL = __fadd_rn(hE, __fmaf_rn(c.bl, fn, bn_e));
-    }
-    static __device__ __forceinline__ P inv_pivot(float hH, float hL, double, const PivScal& c, P x, P y, P z,
-                                                  bool& ok) {
-        // hi chain: S = (a_x + a_y) + a_z, pi_f = hH - b2h S, a ~ 1/pi_f
-        float s1, e1, S, e2;
-        two_sum(x.a, y.a, s1, e1);
-        two_sum(s1, z.a, S, e2);
-        const float th = __fmul_rn(c.b2h, S);
-        const float tl = __fmaf_rn(c.b2h, S, -th);
-        float pf, pe;
-        two_sum(hH, -th, pf, pe);
-        ok = pf > 0.0f;
-        const float a = rcp_approx(pf);
-        const float er = __fmaf_rn(-pf, a, 1.0f);  // exact residual of the reciprocal
-        // lo: dpi = pe + hL - tl - b2l S - b2h (e1 + e2 + sum b)
-        const float base = __fsub_rn(__fadd_rn(pe, hL), __fmaf_rn(c.b2l, S, tl));
-        const float sb = __fadd_rn(__fadd_rn(__fadd_rn(x.b, y.b), z.b), __fadd_rn(e1, e2));
-        const float dpi = __fmaf_rn(-c.b2h, sb, base);
-        const float b = __fmul_rn(a, __fmaf_rn(-dpi, a, er));
-        return ok ? P{a, b} : P{0.0f, 0.0f};
-    }
-};
+// What the forward sweep carries of a voxel and hands on: the inverse pivot (FP32: hi + lo) and
+// v.  FP32 leaves its fourth float 0.  The apply-only sweep carries v alone (Ent = T).
+template <typename T> struct EntOf;
+template <> struct EntOf<float> { using t = float4; };   // 1/pi hi, 1/pi lo, v, 0
+template <> struct EntOf<double> { using t = double2; }; // 1/pi, v
 
+// H_jj = d_j + beta n_j of a mask voxel with n in-mask neighbours; FP32 as hH + hL (n <= 6, so
+// bh * n has one rounding, recovered by FMA).
+__device__ __forceinline__ double form_h(double d, int n, double beta, const PivScal&, double&) {
+    return d + beta * (double)n;
+}
+__device__ __forceinline__ float form_h(float d, int n, double, const PivScal& c, float& hL) {
+    const float fn = (float)n;
+    const float bn = __fmul_rn(c.bh, fn);
+    const float bn_e = __fmaf_rn(c.bh, fn, -bn);
+    float hH, hE;
+    two_sum(d, bn, hH, hE);
+    hL = __fadd_rn(hE, __fmaf_rn(c.bl, fn, bn_e));
+    return hH;
+}
 
-// Faces are written by other CTAs of the same launch: read them through L2.
-__device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
-__device__ __forceinline__ float ld_cg(const float* p) { return __ldcg(p); }
-__device__ __forceinline__ PF ld_cg(const PF* p) {
-    const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
-    return {v.x, v.y};
+// 1/pi_j = 1/(H_jj - beta^2 sum_k 1/pi_k) into o, and 0 where the pivot is not positive: outside
+// the mask (H = -1), or not positive definite (returns false with H >= 0).
+__device__ __forceinline__ bool pivot(double hH, double, double beta, const PivScal&, double2 x, double2 y, double2 z,
+                                      double2& o) {
+    const double piv = hH - beta * beta * ((x.x + y.x) + z.x);
+    const bool ok = piv > 0.0;
+    o.x = ok ? 1.0 / piv : 0.0;
+    return ok;
+}
+__device__ __forceinline__ bool pivot(float hH, float hL, double, const PivScal& c, float4 x, float4 y, float4 z,
+                                      float4& o) {
+    // hi chain: S = (a_x + a_y) + a_z, pi_f = hH - b2h S, a ~ 1/pi_f
+    float s1, e1, S, e2;
+    two_sum(x.x, y.x, s1, e1);
+    two_sum(s1, z.x, S, e2);
+    const float th = __fmul_rn(c.b2h, S);
+    const float tl = __fmaf_rn(c.b2h, S, -th);
+    float pf, pe;
+    two_sum(hH, -th, pf, pe);
+    const bool ok = pf > 0.0f;
+    const float a = rcp_approx(pf);
+    const float er = __fmaf_rn(-pf, a, 1.0f);  // exact residual of the reciprocal
+    // lo: dpi = pe + hL - tl - b2l S - b2h (e1 + e2 + sum b)
+    const float base = __fsub_rn(__fadd_rn(pe, hL), __fmaf_rn(c.b2l, S, tl));
+    const float sb = __fadd_rn(__fadd_rn(__fadd_rn(x.y, y.y), z.y), __fadd_rn(e1, e2));
+    const float dpi = __fmaf_rn(-c.b2h, sb, base);
+    const float b = __fmul_rn(a, __fmaf_rn(-dpi, a, er));
+    o.x = ok ? a : 0.0f;
+    o.y = ok ? b : 0.0f;
+    return ok;
 }
 
 // ------------------------------------------------------------------ asynchronous staging
@@ -159,181 +156,171 @@ __device__ __forceinline__ void cp_wait_all() {
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-// Start copying row r = (ly, lz) = (r & 31, r >> 5) of a T tile into s[r * 32 ..]; elements
-// outside the grid are filled with `fill`.
-template <typename T>
-__device__ __forceinline__ void stage_row(T* s, const T* g, int r, int x0, int y0, int z0, const Geo& geo,
-                                          T fill) {
-    T* srow = s + r * 32;
-    const int y = y0 + (r & 31), z = z0 + (r >> 5);
-    if (y >= geo.ny || z >= geo.nz) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) srow[i] = fill;
-        return;
-    }
-    const T* grow = g + ((long long)z * geo.ny + y) * geo.nx + x0;
-    const int nvalid = min(32, geo.nx - x0);
-    if (nvalid == 32 && ((reinterpret_cast<uintptr_t>(grow) & 15) == 0)) {
-        constexpr int per = 16 / sizeof(T);
-#pragma unroll
-        for (int i = 0; i < 32; i += per) cp16(srow + i, grow + i);
-    } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            if (i < nvalid) {
-                if (sizeof(T) == 4) cp4(srow + i, grow + i);
-                else cp8(srow + i, grow + i);
-            } else {
-                srow[i] = fill;
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ void stage_row_u8(uint8_t* s, const uint8_t* g, int r, int x0, int y0, int z0,
-                                             const Geo& geo) {
-    uint8_t* srow = s + r * 32;
-    const int y = y0 + (r & 31), z = z0 + (r >> 5);
-    if (y >= geo.ny || z >= geo.nz) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) srow[i] = 0;
-        return;
-    }
-    const uint8_t* grow = g + ((long long)z * geo.ny + y) * geo.nx + x0;
-    const int nvalid = min(32, geo.nx - x0);
-    if (nvalid == 32 && ((reinterpret_cast<uintptr_t>(grow) & 15) == 0)) {
-        cp16(srow, grow);
-        cp16(srow + 16, grow + 16);
-    } else {
-        uint8_t v[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = i < nvalid ? grow[i] : (uint8_t)0;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) srow[i] = v[i];
-    }
-}
-
 // ------------------------------------------------------------------ tile geometry
 
 #ifndef FM_IC_CSF
 #define FM_IC_CSF 4
 #endif
 #ifndef FM_IC_CSB
-#define FM_IC_CSB 8
+#define FM_IC_CSB 4
 #endif
-constexpr int kTZ = 8;              // tile = 32 x 32 x 8 voxels, 8 compute warps
-constexpr int kSteps = 62 + kTZ;    // local hyperplanes lx + ly + lz of a tile
-// Steps per chunk (the unit of the face hand-off): forward 4, back substitution 8.  With 8
-// the back substitution's per-chunk face flush lines up with what its successors' chunks
-// need (x / y faces 31 steps later, z faces 7); at most kTZ, one z diagonal per warp.
+#ifndef FM_IC_FWF
+#define FM_IC_FWF 2
+#endif
+#ifndef FM_IC_FWB
+#define FM_IC_FWB 3
+#endif
+constexpr int kTX = kTileX, kTY = kTileY, kTZ = 8;  // 64 x 16 x 8 voxels
+constexpr int kRows = kTY * kTZ;                     // rows along x: one per compute thread
+constexpr int kWarps = kRows / 32;                   // compute warps, two z planes each
+constexpr int kVox = kTX * kRows;
+static_assert(kTX == 64 && kTY == 16 && kWarps == 4, "lane = (y, plane of the warp's pair)");
+// Steps per chunk (the unit of the face hand-off, of the barrier between the warps and of
+// their lag), and the warps that fetch incoming faces, taking the chunks in turn, so that the
+// polls for consecutive chunks are in flight together (a poll round trip is about 0.7 us, a chunk
+// 0.2 to 0.4).  Forward / back substitution on 256 x 256 x 128 (us): chunks of 4 with 2 fetch warps
+// 122 / 97, with 3 125 / 98, with 4 127 / 103; chunks of 3 with 3 130 / 95, of 2 with 4 146 / 101,
+// of 6 with 2 126 / 104.
 constexpr int kCSF = FM_IC_CSF, kCSB = FM_IC_CSB;
-static_assert(kCSB <= kTZ, "the back substitution's face flush takes one z diagonal per warp");
-constexpr int kCompute = 32 * kTZ;  // compute threads
-// Warps that fetch incoming faces, taking alternate chunks, so that the polls for consecutive
-// chunks are in flight together (one poll round trip is longer than a chunk of the back
-// substitution's steps)
-constexpr int kFetchF = 2, kFetchB = 2;
-constexpr int kThreadsIC = kCompute + 32 * kFetchF;
-constexpr int kThreadsB = kCompute + 32 * kFetchB;
+constexpr int kFetchF = FM_IC_FWF, kFetchB = FM_IC_FWB;
+// compute warps, one warp that publishes the outgoing faces, fetch warps
+constexpr int kThreadsF = kRows + 32 + 32 * kFetchF, kThreadsB = kRows + 32 + 32 * kFetchB;
+constexpr int kSweep = kRows + 32;  // threads that meet at the end of a chunk: compute and publishing warps
 
-// Face layout per tile (counts of values): x face [TZ][32] (lz, ly), y face [TZ][32]
-// (lz, lx), z face [32][32].  In shared memory the z face is (ly, lx); in the forward
-// sweep's global face buffer it is stored by diagonals t = lx + ly (see zdiag), so the
-// entries produced at one step, and fetched for one step, are contiguous.
-struct FN {
-    static constexpr int x = 0, y = kTZ * 32, z = 2 * kTZ * 32, n = 2 * kTZ * 32 + 1024;
+// First step of plane lz with chunks of C steps: the two planes of a warp follow each other by
+// one step, and each warp starts C + 1 steps after the warp below.
+template <int C> __host__ __device__ constexpr int tz(int lz) { return (C + 1) * (lz >> 1) + (lz & 1); }
+template <int C> struct Steps {
+    static constexpr int n = kTX + kTY - 1 + tz<C>(kTZ - 1), chunks = (n + C - 1) / C;
+    static_assert(n < 255 && chunks <= 64, "steps in a byte, chunks in a mask");
 };
 
+// Shared memory position of voxel (x, row), rows of 64; odd planes are turned by 16, so that the
+// 32 lanes of a warp -- neighbouring rows at neighbouring x -- meet on two banks at most once.
+__device__ __forceinline__ int vox(int x, int row) { return row * kTX + ((x + 16 * (row / kTY & 1)) & (kTX - 1)); }
+
+// Face layout per tile (counts of values), in the sweep's own (back substitution: mirrored)
+// coordinates: x face (lz, ly), y face (lz, lx), z face (t, ly) by its diagonals t = lx + ly, so
+// that the entries of one step are contiguous.  The same in the global face buffer and in shared
+// memory.
+struct FN {
+    static constexpr int x = 0, y = kTZ * kTY, z = y + kTZ * kTX, n = z + (kTX + kTY - 1) * kTY;
+};
+// Shared memory: two tiles of T (forward: g -> v, d -> 1/pi; back substitution: v -> p, 1/pi), the
+// incoming faces, and the records of every row at the steps of the last two chunks (the z
+// exchange between the warps, and what the publishing warp hands on).
 template <typename T>
 struct FwdSmem {
-    using P = typename PivOps<T>::P;
-    static constexpr int nface = FN::n + 2 * kTZ * 32;  // incoming faces + z exchange
-    static constexpr size_t bytes = (PivOps<T>::kLo ? 3 : 2) * kTZ * 1024 * sizeof(T) +
-                                    nface * (sizeof(P) + sizeof(T)) + kTZ * 1024;
+    static constexpr size_t bytes = 2 * kVox * sizeof(T) + (FN::n + 2 * kCSF * kRows) * 16;
 };
 template <typename T>
 struct BwdSmem {
-    static constexpr size_t bytes = 2 * kTZ * 1024 * sizeof(T) + (FN::n + 2 * kTZ * 32) * sizeof(T);
+    static constexpr size_t bytes = 2 * kVox * sizeof(T) + (FN::n + 2 * kCSB * kRows) * sizeof(T);
 };
 
-__device__ __forceinline__ double shfl_up(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }
-__device__ __forceinline__ PF shfl_up(PF v) {
-    return {__shfl_up_sync(0xffffffffu, v.a, 1), __shfl_up_sync(0xffffffffu, v.b, 1)};
-}
-
-// Per-tile face buffer (device): forward pivots [P][n], forward v [T][n], backward p [T][n].
+// Per-tile face buffer (device): the forward sweep's records [n] (v alone in the apply-only
+// sweep), then the back substitution's p [n].
 template <typename T>
 __host__ __device__ constexpr size_t face_bytes_per_tile() {
-    return (size_t)FN::n * (sizeof(typename PivOps<T>::P) + 2 * sizeof(T));
+    return (size_t)FN::n * (16 + sizeof(T));
 }
+static_assert(sizeof(EntOf<float>::t) == 16 && sizeof(EntOf<double>::t) == 16, "face records of 16 bytes");
 
-// smem index of voxel (lx, ly, lz) and of each outgoing face entry i
-__device__ __forceinline__ int vox(int lx, int ly, int lz) { return (lz * 32 + ly) * 32 + lx; }
-__device__ __forceinline__ int out_face_vox(int i, bool fwd) {
-    // forward: the +x (lx = 31), +y (ly = 31) and +z (lz = TZ-1) faces; backward: lx = 0, ly = 0, lz = 0
-    if (i < FN::y) return vox(fwd ? 31 : 0, i & 31, i >> 5);
-    if (i < FN::z) { const int k = i - FN::y; return vox(k & 31, fwd ? 31 : 0, k >> 5); }
-    const int k = i - FN::z;
-    return vox(k & 31, k >> 5, fwd ? kTZ - 1 : 0);
+// Stage one array's tile: 16-byte copies along x where whole 16-byte pieces of an aligned row are
+// inside the grid (nx a multiple of 4 floats / 2 doubles), else one element per lane.  Rows and
+// columns outside the grid read 0.  kRows threads; completion by cp_wait_all.
+template <typename T>
+__device__ __forceinline__ void stage_tile(T* s, const T* g, int x0, int y0, int z0, const Geo& geo) {
+    const int nvalid = min(kTX, geo.nx - x0);
+    constexpr int per = 16 / sizeof(T), cols = kTX / per;
+    if (geo.nx % per == 0 && (reinterpret_cast<uintptr_t>(g) & 15) == 0) {
+#pragma unroll 8
+        for (int i = threadIdx.x; i < kRows * cols; i += kRows) {
+            const int r = i / cols, x = (i % cols) * per, y = y0 + r % kTY, z = z0 + r / kTY;
+            T* to = s + vox(x, r);
+            if (x < nvalid && y < geo.ny && z < geo.nz) {
+                cp16(to, g + ((long long)z * geo.ny + y) * geo.nx + x0 + x);
+            } else {
+#pragma unroll
+                for (int k = 0; k < per; ++k) to[k] = T(0);
+            }
+        }
+    } else {
+#pragma unroll 8
+        for (int i = threadIdx.x; i < kVox; i += kRows) {
+            const int r = i / kTX, x = i % kTX, y = y0 + r % kTY, z = z0 + r / kTY;
+            T* to = s + vox(x, r);
+            if (x < nvalid && y < geo.ny && z < geo.nz) {
+                const T* from = g + ((long long)z * geo.ny + y) * geo.nx + x0 + x;
+                if (sizeof(T) == 4) cp4(to, from);
+                else cp8(to, from);
+            } else {
+                *to = T(0);
+            }
+        }
+    }
 }
-
-// Hyperplanes of a tile that hold a mask voxel, first | last << 8 (an empty tile: 255, none
-// after it), as the sweeps read them.
+// Steps of a tile's sweeps that reach a mask voxel, a byte each: first and last of the forward
+// sweep, first and last of the back substitution; an empty tile has first 255, last 0.
 struct Range {
     int lo, hi;
     __device__ __forceinline__ bool has(int s) const { return s >= lo && s <= hi; }
 };
-__device__ __forceinline__ Range tile_range(const int* range, int tile) {
+template <bool FWD>
+__device__ __forceinline__ Range tile_range(const unsigned* range, int tile) {
     if (tile < 0) return {255, 0};
-    const int r = range[tile];
-    return {r & 255, r >> 8};
+    const unsigned r = range[tile] >> (FWD ? 0 : 16);
+    return {(int)(r & 255u), (int)(r >> 8 & 255u)};
 }
 
-// One block per tile, one thread per (y, z) row.
-__global__ void __launch_bounds__(kCompute) k_ic_range(Geo geo, int ntx, int nty, const uint8_t* nb, int* range) {
+// One block per tile, one thread per row.
+__global__ void __launch_bounds__(kRows) k_ic_range(Geo geo, int ntx, int nty, const uint8_t* nb, unsigned* range) {
+    __shared__ int s_lim[4];
     const int tile = blockIdx.x, X = tile % ntx, Y = (tile / ntx) % nty, Z = tile / (ntx * nty);
-    const int ly = threadIdx.x & 31, lz = threadIdx.x >> 5;
-    const int y = Y * 32 + ly, z = Z * kTZ + lz, x0 = X * 32;
-    int lo = 255, hi = 0;
+    const int ly = threadIdx.x % kTY, lz = threadIdx.x / kTY;
+    const int y = Y * kTY + ly, z = Z * kTZ + lz, x0 = X * kTX;
+    if (threadIdx.x < 4) s_lim[threadIdx.x] = (threadIdx.x & 1) ? 0 : 255;
+    __syncthreads();
     if (y < geo.ny && z < geo.nz) {
         const uint8_t* row = nb + ((long long)z * geo.ny + y) * geo.nx + x0;
-        const int n = min(32, geo.nx - x0);
+        const int n = min(kTX, geo.nx - x0);
+        int lo = 255, hi = -1;
         for (int i = 0; i < n; ++i)
             if (row[i] & NB_IN) {
-                lo = min(lo, i + ly + lz);
-                hi = i + ly + lz;
+                lo = min(lo, i);
+                hi = i;
             }
-    }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    __shared__ int s_lo[kTZ], s_hi[kTZ];
-    if (ly == 0) {
-        s_lo[lz] = lo;
-        s_hi[lz] = hi;
+        if (hi >= 0) {
+            const int f = ly + tz<kCSF>(lz), b = (kTY - 1 - ly) + tz<kCSB>(kTZ - 1 - lz);
+            atomicMin(&s_lim[0], lo + f);
+            atomicMax(&s_lim[1], hi + f);
+            atomicMin(&s_lim[2], kTX - 1 - hi + b);
+            atomicMax(&s_lim[3], kTX - 1 - lo + b);
+        }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kTZ; ++w) {
-            lo = min(lo, s_lo[w]);
-            hi = max(hi, s_hi[w]);
-        }
-        range[tile] = lo | hi << 8;
-    }
+    if (threadIdx.x == 0)
+        range[tile] = (unsigned)s_lim[0] | (unsigned)s_lim[1] << 8 | (unsigned)s_lim[2] << 16 | (unsigned)s_lim[3] << 24;
 }
 
-// The non-empty tiles of both claim orders (order[0..ntiles) forward, order[ntiles..) for the
-// back substitution), kept in order: one block per claim order.
-__global__ void __launch_bounds__(1024) k_ic_order(const int* order, const int* range, int ntiles, int* out,
-                                                   int* istate) {
+// Lists in claim order, one block each: block 0 the non-empty tiles of the forward order
+// (order[0..ntiles)), block 1 those of the back substitution's (order[ntiles..)), and block 2, in
+// the same order, the tiles that stand for a dot-product unit: a unit is a pair of tiles Y = 2k,
+// 2k + 1 and belongs to the lower one (the later of the two to be swept back) if that is not empty.
+__global__ void __launch_bounds__(1024) k_ic_order(const int* order, const unsigned* range, int ntx, int nty, int ntiles,
+                                                   int* out, int* istate) {
     __shared__ int s_warp[32], s_base;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const size_t off = (size_t)blockIdx.x * ntiles;
+    const int* in = order + (blockIdx.x == 0 ? 0 : ntiles);
+    out += (size_t)blockIdx.x * ntiles;
+    auto empty = [&](int t) { return (range[t] & 255u) == 255u; };
     if (threadIdx.x == 0) s_base = 0;
     __syncthreads();
     for (int b = 0; b < ntiles; b += 1024) {
         const int i = b + threadIdx.x;
-        const int t = i < ntiles ? order[off + i] : -1;
-        const bool keep = t >= 0 && (range[t] & 255) != 255;
+        const int t = i < ntiles ? in[i] : -1;
+        bool keep = t >= 0 && !empty(t);
+        if (blockIdx.x == 2 && keep && ((t / ntx) % nty & 1)) keep = empty(t - ntx);
         const unsigned bal = __ballot_sync(0xffffffffu, keep);
         if (lane == 0) s_warp[wid] = __popc(bal);
         __syncthreads();
@@ -342,24 +329,21 @@ __global__ void __launch_bounds__(1024) k_ic_order(const int* order, const int* 
             if (w < wid) at += s_warp[w];
             tot += s_warp[w];
         }
-        if (keep) out[off + at + __popc(bal & ((1u << lane) - 1u))] = t;
+        if (keep) out[at + __popc(bal & ((1u << lane) - 1u))] = t;
         __syncthreads();
         if (threadIdx.x == 0) s_base += tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0 && blockIdx.x == 0) istate[I_NTILE] = s_base;
+    if (threadIdx.x == 0 && blockIdx.x != 1) istate[blockIdx.x == 0 ? I_NTILE : I_NUNIT] = s_base;
 }
 
 // ------------------------------------------------------------------ streamed faces
 //
 // A forward tile's sweep does not wait for its predecessor tiles to finish: every voxel of a
 // tile's three outgoing faces is written to the face buffer as soon as it is computed.  A
-// successor's step s needs, from its -x and -y neighbours, face values those tiles produce
-// at their step s + 31, and from its -z neighbour values produced at step s + kTZ - 1.  So a
-// successor runs about 32 steps behind its x / y predecessors and kTZ behind its z
-// predecessor instead of a whole tile (70 steps) behind; the chain through the grid shrinks
-// from (tile levels) x 70 steps towards the nx + ny + nz hyperplanes of the global wavefront,
-// plus one hand-off latency per tile hop.
+// successor's step s needs, from its -x, -y and -z neighbours, face values those tiles produce
+// at their step s + 63, s + 15 and s + tz(7).  So a successor runs those many steps (and one
+// hand-off) behind its predecessors instead of a whole tile behind.
 //
 // The face entries are their own ready signal.  Between launches every forward face entry
 // holds an all-ones bit pattern -- a NaN that no FP32 / FP64 operation produces (arithmetic
@@ -377,19 +361,28 @@ __global__ void __launch_bounds__(1024) k_ic_order(const int* order, const int* 
 // signals the compute warps through a shared-memory counter.  The compute warps synchronise
 // among themselves with a named barrier and never poll global memory.
 
-__device__ __forceinline__ void bar_compute() { asm volatile("bar.sync 1, %0;" ::"n"(kCompute) : "memory"); }
+template <int NT>
+__device__ __forceinline__ void bar_warps() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
+template <int NT>
+__device__ __forceinline__ void bar_warps2() { asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory"); }
+__device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 // the unset pattern of a face entry, and values kept clear of it
 __device__ __forceinline__ bool unset(float x) { return __float_as_uint(x) == 0xffffffffu; }
 __device__ __forceinline__ bool unset(double x) { return __double_as_longlong(x) == -1LL; }
-__device__ __forceinline__ bool unset(PF x) { return unset(x.a) || unset(x.b); }
+__device__ __forceinline__ bool unset(float4 e) { return unset(e.x) || unset(e.y) || unset(e.z) || unset(e.w); }
+__device__ __forceinline__ bool unset(double2 e) { return unset(e.x) || unset(e.y); }
 __device__ __forceinline__ float canon(float x) { return unset(x) ? __uint_as_float(0x7fffffffu) : x; }
 __device__ __forceinline__ double canon(double x) {
     return unset(x) ? __longlong_as_double(0x7fffffffffffffffLL) : x;
 }
-__device__ __forceinline__ PF canon(PF x) { return {canon(x.a), canon(x.b)}; }
+// an inverse pivot is finite by construction (0 where the pivot is not positive), and v is the
+// result of a multiplication: the canonical NaN in FP32, while FP64 may carry an operand's NaN on
+__device__ __forceinline__ float4 canon(float4 e) { return e; }
+__device__ __forceinline__ double2 canon(double2 e) { e.y = canon(e.y); return e; }
 
-// relaxed (gpu scope) loads and stores of face entries
+// relaxed (gpu scope) loads and stores of face entries; a record's components are ordered by
+// nothing but their own values, and unset() looks at each
 __device__ __forceinline__ float ld_rlx(const float* p) {
     float v;
     asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
@@ -400,9 +393,15 @@ __device__ __forceinline__ double ld_rlx(const double* p) {
     asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ PF ld_rlx(const PF* p) {
-    PF v;
-    asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.a), "=f"(v.b) : "l"(p));
+__device__ __forceinline__ float4 ld_rlx(const float4* p) {
+    float4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_rlx(const double2* p) {
+    double2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
     return v;
 }
 __device__ __forceinline__ void st_unset(float* p) {
@@ -411,65 +410,30 @@ __device__ __forceinline__ void st_unset(float* p) {
 __device__ __forceinline__ void st_unset(double* p) {
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(-1LL) : "memory");
 }
-__device__ __forceinline__ void st_unset(PF* p) {
-    asm volatile("st.relaxed.gpu.global.v2.b32 [%0], {%1, %1};" ::"l"(p), "r"(-1) : "memory");
+__device__ __forceinline__ void st_unset(float4* p) {
+    asm volatile("st.relaxed.gpu.global.v4.b32 [%0], {%1, %1, %1, %1};" ::"l"(p), "r"(-1) : "memory");
 }
+__device__ __forceinline__ void st_unset(double2* p) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %1};" ::"l"(p), "l"(-1LL) : "memory");
+}
+__device__ __forceinline__ float zero_ent(const float*) { return 0.f; }
+__device__ __forceinline__ double zero_ent(const double*) { return 0.0; }
+__device__ __forceinline__ float4 zero_ent(const float4*) { return {0.f, 0.f, 0.f, 0.f}; }
+__device__ __forceinline__ double2 zero_ent(const double2*) { return {0.0, 0.0}; }
 
-// Offset of diagonal t = lx + ly (0 <= t <= 62) in the diagonal-major z face: diagonal t holds
-// min(t + 1, 63 - t) entries, ordered by lx.
-__device__ __forceinline__ int zdiag(int t) { return t <= 32 ? t * (t + 1) / 2 : 528 + (t - 32) * (95 - t) / 2; }
-
-// Face entries used at local step s of the forward sweep: x face (ly, lz) with ly + lz = s,
-// y face (lx, lz) with lx + lz = s, z face (lx, ly) with lx + ly = s.  Each lane takes at most
-// one z-face entry and one x- or y-face entry per step; -1 = none.  z_entry returns the shared
-// memory index; lane k of a z diagonal reads global entry FN::z + zdiag(s) + k.
-__device__ __forceinline__ int z_entry(int s, int lane) {
-    const int lx = max(0, s - 31) + lane;
-    return (s >= 0 && lx <= min(31, s)) ? FN::z + (s - lx) * 32 + lx : -1;
+// relaxed stores of outgoing face entries (no compiler memory clobber: nothing in the kernel reads
+// the entry back)
+__device__ __forceinline__ void st_rlx(float* a, float v) {
+    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(a), "f"(v));
 }
-__device__ __forceinline__ int xy_entry(int s, int lane, int& which) {
-    if (lane < kTZ) {  // x face: lanes 0..TZ-1 take lz = lane
-        const int ly = s - lane;
-        which = 0;
-        return (ly >= 0 && ly < 32) ? FN::x + lane * 32 + ly : -1;
-    }
-    if (lane >= 16 && lane < 16 + kTZ) {  // y face: lanes 16.. take lz = lane - 16
-        const int lz = lane - 16, lx = s - lz;
-        which = 1;
-        return (lx >= 0 && lx < 32) ? FN::y + lz * 32 + lx : -1;
-    }
-    return -1;
+__device__ __forceinline__ void st_rlx(double* a, double v) {
+    asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(a), "d"(v));
 }
-
-// Predicated relaxed stores of outgoing face entries: written by the one lane that produces
-// the entry at a step, without a divergent branch in the step body.  No compiler memory
-// clobber: the stored value is an operand, nothing in the kernel reads the entry back, and
-// volatile asm keeps its order relative to the barriers.  The caller keeps the
-// value clear of the unset pattern: an inverse pivot is finite by construction (0 where the
-// pivot is not positive or outside the mask), and v passes through canon.
-__device__ __forceinline__ void st_if(bool p, double* a, double v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q st.relaxed.gpu.global.f64 [%1], %2;\n\t}"
-                 ::"r"((int)p), "l"(a), "d"(v));
+__device__ __forceinline__ void st_rlx(float4* a, float4 v) {
+    asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
 }
-__device__ __forceinline__ void st_if(bool p, float* a, float v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q st.relaxed.gpu.global.f32 [%1], %2;\n\t}"
-                 ::"r"((int)p), "l"(a), "f"(v));
-}
-__device__ __forceinline__ void st_if(bool p, PF* a, PF v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t@q st.relaxed.gpu.global.v2.f32 [%1], {%2, %3};\n\t}"
-                 ::"r"((int)p), "l"(a), "f"(v.a), "f"(v.b));
-}
-
-// After a tile's sweep every entry of its incoming faces has been read (the compute warps
-// waited for every chunk), so the compute warps return them to the unset pattern for the
-// next launch: the -x (or +x) neighbour's x face, the y neighbour's y face and the z
-// neighbour's z face are contiguous ranges of those tiles' face buffers.
-template <typename T>
-__device__ __forceinline__ void unset_faces(T* fx, T* fy, T* fz) {
-    for (int i = threadIdx.x; i < FN::n; i += kCompute) {
-        T* f = i < FN::y ? fx : i < FN::z ? fy : fz;
-        if (f) st_unset(f + i);
-    }
+__device__ __forceinline__ void st_rlx(double2* a, double2 v) {
+    asm volatile("st.relaxed.gpu.global.v2.f64 [%0], {%1, %2};" ::"l"(a), "d"(v.x), "d"(v.y));
 }
 
 // Chunk hand-off from the fetch warp to the compute warps: one mbarrier per chunk with an
@@ -505,43 +469,147 @@ __device__ __forceinline__ void wait_chunk(unsigned long long* m, unsigned parit
     }
 }
 
-// MODE 0: pivots from d (factor + forward); MODE 1: stored 1/pi (forward only)
+// Which face entry lane `lane` of a fetch or publishing warp handles at step s: lanes 0..15 the
+// z face (ly = lane), lanes 16..23 the x face of plane lane - 16, lanes 24..31 the y face of
+// plane lane - 24.  With k = s - first (0 <= k < count) the entry is base + k * pitch.
+template <int C>
+struct FaceLane {
+    int cls, lz, first, count, base, pitch;
+    __device__ __forceinline__ explicit FaceLane(int lane) {
+        cls = lane < 16 ? 2 : lane < 24 ? 0 : 1;
+        lz = lane & 7;
+        first = cls == 2 ? lane : tz<C>(lz);
+        count = cls == 0 ? kTY : kTX;
+        base = cls == 2 ? FN::z + lane * (kTY + 1) : cls == 0 ? FN::x + lz * kTY : FN::y + lz * kTX;
+        pitch = cls == 2 ? kTY : 1;
+    }
+    // steps between the producer's and the consumer's use of an entry
+    __device__ __forceinline__ int lag() const { return cls == 2 ? tz<C>(kTZ - 1) : cls == 0 ? kTX - 1 : kTY - 1; }
+    template <typename V> __device__ __forceinline__ V pick(V x, V y, V z) const { return cls == 2 ? z : cls == 0 ? x : y; }
+};
+
+// Fetch warp `w` of `nw`: brings the incoming face entries of chunks w, w + nw, .. into shared
+// memory from the neighbours' face records (tiles px, py, pz; -1: none).
+template <int C, bool FWD, typename Ent, typename Face>
+__device__ __forceinline__ void fetch_faces(Ent* f_in, const IcArgs& a, Face face, int px, int py, int pz, Range rg, int nch,
+                                            int w, int nw, unsigned long long* mbar) {
+    const FaceLane<C> fl(threadIdx.x & 31);
+    const int tile = fl.pick(px, py, pz);
+    const Ent* from = tile >= 0 ? face(tile) : nullptr;
+    const Range rs = tile_range<FWD>(a.range, tile);
+    const int lag = fl.lag();
+    bool ok = true;
+    for (int c = w; c < nch; c += nw) {
+        Ent e[C];
+        int at[C];
+        unsigned todo = 0;
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+            const int s = rg.lo + c * C + q, k = s - fl.first;
+            at[q] = (unsigned)k < (unsigned)fl.count ? fl.base + k * fl.pitch : -1;
+            e[q] = zero_ent((const Ent*)nullptr);  // stays 0 where the neighbour hands nothing over
+            if (at[q] >= 0 && s <= rg.hi && rs.has(s + lag)) todo |= 1u << q;
+        }
+        // poll until every wanted entry is set (all of a round's loads are in flight together); a
+        // wait that gives up leaves zeros and reports the timeout
+        if (!ok) todo = 0u;
+        long long tries = 0;
+        while (__any_sync(0xffffffffu, todo != 0u)) {
+#pragma unroll
+            for (int q = 0; q < C; ++q)
+                if (todo & (1u << q)) e[q] = ld_rlx(from + at[q]);
+#pragma unroll
+            for (int q = 0; q < C; ++q)
+                if ((todo & (1u << q)) && !unset(e[q])) todo &= ~(1u << q);
+            if (++tries > a.spin_limit && __any_sync(0xffffffffu, todo != 0u)) {
+                ok = false;
+#pragma unroll
+                for (int q = 0; q < C; ++q)
+                    if (todo & (1u << q)) e[q] = zero_ent((const Ent*)nullptr);
+                todo = 0u;
+            } else if (todo != 0u) {
+                __nanosleep(20);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < C; ++q)
+            if (at[q] >= 0) f_in[at[q]] = e[q];
+        __syncwarp();
+        if (lane_id() == 0) mbar_arrive(&mbar[c]);
+    }
+    if (!ok) set_err(a.istate, FM_ERR_TIMEOUT);  // the host resets the faces with the error
+}
+
+// Publishing warp: after each chunk, the face entries that the successors (tiles sx, sy, sz; -1:
+// none) read go from the ring of step records to this tile's face records.  A compute warp that
+// stores them itself spends 10 to 20 cycles a step on each face's predicate, address and store.
+template <int C, bool FWD, typename Ent>
+__device__ __forceinline__ void publish_faces(const Ent* ring, Ent* out, const IcArgs& a, int sx, int sy, int sz, Range rg,
+                                              int nch) {
+    const FaceLane<C> fl(threadIdx.x & 31);
+    const Range r = tile_range<FWD>(a.range, fl.pick(sx, sy, sz));
+    const int lag = fl.lag();
+    // entry k is made at step first + lag + k by the row of the face (x face: row of entry k)
+    const int lane = threadIdx.x & 31;
+    const int row0 = fl.pick(fl.lz * kTY, fl.lz * kTY + kTY - 1, (kTZ - 1) * kTY + lane), drow = fl.cls == 0 ? 1 : 0;
+    for (int c = 0; c < nch; ++c) {
+        bar_warps<kSweep>();
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+            const int s = rg.lo + c * C + q, k = s - lag - fl.first;
+            const bool go = (unsigned)k < (unsigned)fl.count && s <= rg.hi && r.has(s - lag);
+            if (go) st_rlx(out + fl.base + k * fl.pitch, canon(ring[((c & 1) * C + q) * kRows + row0 + k * drow]));
+        }
+    }
+}
+
+// After a tile's sweep every entry of its incoming faces has been read (the compute warps
+// waited for every chunk), so they return to the unset pattern for the next launch: the x
+// neighbour's x face, the y neighbour's y face and the z neighbour's z face are contiguous
+// ranges of those tiles' face buffers.
+template <typename E>
+__device__ __forceinline__ void unset_faces(E* fx, E* fy, E* fz) {
+    for (int i = threadIdx.x; i < FN::n; i += blockDim.x) {
+        E* f = i < FN::y ? fx : i < FN::z ? fy : fz;
+        if (f) st_unset(f + i);
+    }
+}
+
+__device__ __forceinline__ float shfl_up(float v, int n) { return __shfl_up_sync(0xffffffffu, v, n); }
+__device__ __forceinline__ double shfl_up(double v, int n) { return __shfl_up_sync(0xffffffffu, v, n); }
+
+__device__ __forceinline__ float v_of(float4 e) { return e.z; }
+__device__ __forceinline__ double v_of(double2 e) { return e.y; }
+__device__ __forceinline__ float v_of(float e) { return e; }
+__device__ __forceinline__ double v_of(double e) { return e; }
+
+// MODE 0: pivots from d (factor + forward); MODE 1: stored 1/pi (forward only); MODE 2: as 0, and
+// FP32's low parts of the inverse pivots go out too (the inspection call)
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kThreadsIC) k_ic_fwd(IcArgs a, PivScal pc) {
-    constexpr int mode = MODE;
-    using Ops = PivOps<T>;
-    using P = typename Ops::P;
+__global__ void __launch_bounds__(kThreadsF, sizeof(T) == 4 ? 2 : 1) k_ic_fwd(IcArgs a, PivScal pc) {
+    using Ent = std::conditional_t<MODE != 1, typename EntOf<T>::t, T>;
+    constexpr int C = kCSF;
     extern __shared__ __align__(16) unsigned char smem[];
-    T* sg = (T*)smem;                              // [TZ][32][32]: g, then v
-    T* sd = sg + kTZ * 1024;                       // d -> H_hi (-1 outside) -> 1/pi hi; or stored 1/pi
-    T* sl = sd + kTZ * 1024;                       // FP32: H_lo -> 1/pi lo
-    P* f_ip = (P*)(sd + (Ops::kLo ? 2 : 1) * kTZ * 1024);  // incoming faces: x, y, z
-    P* zb_ip = f_ip + FN::n;                       // [2][TZ][32]
-    T* f_v = (T*)(zb_ip + 2 * kTZ * 32);
-    T* zb_v = f_v + FN::n;
-    uint8_t* snb = (uint8_t*)(zb_v + 2 * kTZ * 32);  // [TZ][32][32]
+    T* sg = (T*)smem;                 // g, then v
+    T* sd = sg + kVox;                // d, then 1/pi; or stored 1/pi
+    Ent* f_in = (Ent*)(sd + kVox);    // incoming faces
+    Ent* ring = f_in + FN::n;         // step records [2][C][kRows]
     __shared__ int s_tile;
-    constexpr int kCS = kCSF, kNch = (kSteps + kCS - 1) / kCS;
-    __shared__ __align__(8) unsigned long long s_mbar[kNch];
+    __shared__ __align__(8) unsigned long long s_mbar[Steps<C>::chunks];
 
     const Geo geo = a.geo;
     const int nx = geo.nx, ny = geo.ny, nz = geo.nz;
     const long long nxy = (long long)nx * ny;
     const int tid = threadIdx.x, lane = tid & 31, wz = tid >> 5;
-    const T* g = (const T*)a.g;
-    const T* d = (const T*)a.d;
-    const T* ipin = (const T*)a.ip_in;
     T* v = (T*)a.v;
     T* ipo = (T*)a.ip_out;
-    unsigned char* faceb = (unsigned char*)a.face;
     const T betaT = (T)a.beta;
-    auto face_ip = [&](int t) { return (P*)(faceb + (size_t)t * face_bytes_per_tile<T>()); };
-    auto face_v = [&](int t) { return (T*)(face_ip(t) + FN::n); };
+    auto face = [&](int t) { return (Ent*)((unsigned char*)a.face + (size_t)t * face_bytes_per_tile<T>()); };
 
     if (tid == 0)
-        for (int c = 0; c < kNch; ++c) mbar_init(&s_mbar[c], 1);
+        for (int c = 0; c < Steps<C>::chunks; ++c) mbar_init(&s_mbar[c], 1);
     const int ntile = a.istate[I_NTILE];
-    unsigned par = 0;  // bit c: phase parity of chunk c's barrier (one phase per tile that has the chunk)
+    unsigned long long par = 0;  // bit c: phase parity of chunk c's barrier (one phase per tile that has the chunk)
     for (;;) {
         if (tid == 0) {
             const int t = atomicAdd(a.ticket, 1);
@@ -551,270 +619,237 @@ __global__ void __launch_bounds__(kThreadsIC) k_ic_fwd(IcArgs a, PivScal pc) {
         const int tile = s_tile;
         if (tile < 0) break;
         const int X = tile % a.ntx, Y = (tile / a.ntx) % a.nty, Z = tile / (a.ntx * a.nty);
-        const int x0 = X * 32, y0 = Y * 32, z0 = Z * kTZ;
-        const Range rg = tile_range(a.range, tile);
-        const int nch = (rg.hi - rg.lo) / kCS + 1;
+        const int x0 = X * kTX, y0 = Y * kTY, z0 = Z * kTZ;
+        const Range rg = tile_range<true>(a.range, tile);
+        const int nch = (rg.hi - rg.lo) / C + 1, nvalid = min(kTX, nx - x0);
+        const int px = X > 0 ? tile - 1 : -1, py = Y > 0 ? tile - a.ntx : -1, pz = Z > 0 ? tile - a.ntx * a.nty : -1;
 
-        if (wz >= kTZ) {
-            // fetch warps: the -x, -y, -z neighbours' outgoing +x, +y, +z faces, alternate chunks each
-            const int sx = X > 0 ? tile - 1 : -1, sy = Y > 0 ? tile - a.ntx : -1;
-            const int sz = Z > 0 ? tile - a.ntx * a.nty : -1;
-            const Range rx = tile_range(a.range, sx), ry = tile_range(a.range, sy), rz = tile_range(a.range, sz);
-            bool ok = true;
-            for (int c = wz - kTZ; c < nch; c += kFetchF) {
-                P zp[kCS], qp[kCS];
-                T zv[kCS], qv[kCS];
-                int zi[kCS], zg[kCS], qi[kCS], qsrc[kCS];
-                unsigned want = 0;  // bit q: z entry of step q; bit kCS + q: x / y entry
-#pragma unroll
-                for (int q = 0; q < kCS; ++q) {
-                    const int s = rg.lo + c * kCS + q;
-                    int which = 0;
-                    zi[q] = s <= rg.hi ? z_entry(s, lane) : -1;
-                    zg[q] = FN::z + zdiag(min(s, 62)) + lane;
-                    qi[q] = s <= rg.hi ? xy_entry(s, lane, which) : -1;
-                    qsrc[q] = which ? sy : sx;
-                    zp[q] = Ops::zero();
-                    qp[q] = Ops::zero();
-                    zv[q] = T(0);
-                    qv[q] = T(0);
-                    if (zi[q] >= 0 && rz.has(s + kTZ - 1)) want |= 1u << q;
-                    if (qi[q] >= 0 && (which ? ry : rx).has(s + 31)) want |= 1u << (kCS + q);
-                }
-                // poll until every wanted entry is set (all of a round's loads are in flight
-                // together); a wait that gives up leaves zeros and reports the timeout
-                unsigned todo = ok ? want : 0u;
-                long long tries = 0;
-                while (__any_sync(0xffffffffu, todo != 0u)) {
-#pragma unroll
-                    for (int q = 0; q < kCS; ++q) {
-                        if (todo & (1u << q)) {
-                            if (mode == 0) zp[q] = ld_rlx(face_ip(sz) + zg[q]);
-                            zv[q] = ld_rlx(face_v(sz) + zg[q]);
-                        }
-                        if (todo & (1u << (kCS + q))) {
-                            if (mode == 0) qp[q] = ld_rlx(face_ip(qsrc[q]) + qi[q]);
-                            qv[q] = ld_rlx(face_v(qsrc[q]) + qi[q]);
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < kCS; ++q) {
-                        if ((todo & (1u << q)) && !unset(zv[q]) && (mode != 0 || !unset(zp[q])))
-                            todo &= ~(1u << q);
-                        if ((todo & (1u << (kCS + q))) && !unset(qv[q]) && (mode != 0 || !unset(qp[q])))
-                            todo &= ~(1u << (kCS + q));
-                    }
-                    if (++tries > a.spin_limit && __any_sync(0xffffffffu, todo != 0u)) {
-                        ok = false;
-#pragma unroll
-                        for (int q = 0; q < kCS; ++q) {
-                            if (todo & (1u << q)) { zp[q] = Ops::zero(); zv[q] = T(0); }
-                            if (todo & (1u << (kCS + q))) { qp[q] = Ops::zero(); qv[q] = T(0); }
-                        }
-                        want &= ~todo;
-                        todo = 0u;
-                    } else if (todo != 0u) {
-                        __nanosleep(20);
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < kCS; ++q) {
-                    if (zi[q] >= 0) { f_ip[zi[q]] = zp[q]; f_v[zi[q]] = zv[q]; }
-                    if (qi[q] >= 0) { f_ip[qi[q]] = qp[q]; f_v[qi[q]] = qv[q]; }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&s_mbar[c]);
-            }
-            if (!ok) set_err(a.istate, FM_ERR_TIMEOUT);  // the host resets the faces with the error
+        if (wz > kWarps) {
+            fetch_faces<C, true>(f_in, a, face, px, py, pz, rg, nch, wz - kWarps - 1, kFetchF, s_mbar);
+        } else if (wz == kWarps) {
+            publish_faces<C, true>(ring, face(tile), a, X + 1 < a.ntx ? tile + 1 : -1, Y + 1 < a.nty ? tile + a.ntx : -1,
+                                   Z + 1 < a.ntz ? tile + a.ntx * a.nty : -1, rg, nch);
         } else {
-            // stage this tile's inputs and form H while the predecessors are still running
-            stage_row<T>(sg, g, tid, x0, y0, z0, geo, T(0));
-            stage_row<T>(sd, mode == 0 ? d : ipin, tid, x0, y0, z0, geo, T(0));
-            if (mode == 0) stage_row_u8(snb, a.nb, tid, x0, y0, z0, geo);
-            cp_wait_all();
-            if (mode == 0) {
-                T* dr = sd + tid * 32;
-                T* lr = sl + tid * 32;
-                const uint8_t* br = snb + tid * 32;
-                // each thread walks its own row; starting at column `lane` keeps the 32 lanes
-                // of a warp on 32 different banks (rows are 32 elements apart)
-#pragma unroll 4
-                for (int k = 0; k < 32; ++k) {
-                    const int i = (k + lane) & 31;
-                    const uint8_t b = br[i];
-                    T hH = T(-1), hL = T(0);
-                    if (b & NB_IN) Ops::form_h(dr[i], __popc((unsigned)(b >> 1) & 0x3fu), a.beta, pc, hH, hL);
-                    dr[i] = hH;
-                    if (Ops::kLo) lr[i] = hL;
-                }
-            }
-            // hyperplanes before the first are 0: the z exchange starts from that
-            for (int i = tid; i < 2 * kTZ * 32; i += kCompute) {
-                zb_v[i] = T(0);
-                if (mode == 0) zb_ip[i] = Ops::zero();
-            }
-            bar_compute();
-
-            // sweep the local hyperplanes s = lx + ly + lz.  The body is branch-free: a lane
-            // outside its row (lx not in [0, 32)) computes on the wrapped index lx & 31 -- every
-            // lane keeps its own shared-memory bank -- and only active lanes store.
-            const int ly = lane, lz = wz, l0 = ly + lz;
-            const int row = (lz * 32 + ly) * 32;
-            const P* fy_ip = f_ip + FN::y + lz * 32;
-            const T* fy_v = f_v + FN::y + lz * 32;
-            const P* fz_ip = f_ip + FN::z + ly * 32;
-            const T* fz_v = f_v + FN::z + ly * 32;
-            const int fxi = FN::x + lz * 32 + ly;
-            const int zr = (lz > 0 ? lz - 1 : 0) * 32 + ly, zw = lz * 32 + ly;
-            P* oip = face_ip(tile);
-            T* ov = face_v(tile);
-            // steps whose face entries a successor reads
-            const Range ux = tile_range(a.range, X + 1 < a.ntx ? tile + 1 : -1);
-            const Range uy = tile_range(a.range, Y + 1 < a.nty ? tile + a.ntx : -1);
-            const Range uz = tile_range(a.range, Z + 1 < a.ntz ? tile + a.ntx * a.nty : -1);
-            P out_ip = Ops::zero();
-            T out_v = 0;
-            bool bad = false;
-            // zdiag(t) - max(0, t - 31) for this warp's current diagonal t = s - lz (0 while t < 0):
-            // the z-face entry of lane ly at step s is FN::z + zbase + lx
-            int zbase = rg.lo > lz ? zdiag(min(rg.lo - lz, 62)) - max(0, rg.lo - lz - 31) : 0;
-            for (int c = 0; c < nch; ++c) {
-              wait_chunk(&s_mbar[c], (par >> c) & 1u, a.spin_limit, a.istate);
+            const int ly = lane & 15, up = lane >> 4, lz = 2 * wz + up, row = lz * kTY + ly;
+            // stage this tile's inputs while the predecessors are still running
+            stage_tile<T>(sg, (const T*)a.g, x0, y0, z0, geo);
+            stage_tile<T>(sd, (const T*)(MODE != 1 ? a.d : a.ip_in), x0, y0, z0, geo);
+            // steps before the first are 0: the z exchange starts from that
+            for (int i = tid; i < 2 * C * kRows; i += kRows) ring[i] = zero_ent((const Ent*)nullptr);
+            // the row's neighbour bits, read one chunk ahead
+            const bool row_in = y0 + ly < ny && z0 + lz < nz;
+            const uint8_t* nbp = a.nb + (long long)(z0 + lz) * nxy + (long long)(y0 + ly) * nx + x0;
+            unsigned nbq[C];
+            auto load_bits = [&](int lx) {
 #pragma unroll
-              for (int q = 0; q < kCS; ++q) {
-                const int s = rg.lo + c * kCS + q;
-                if (s > rg.hi) break;
-                const P up_ip = shfl_up(out_ip);
-                const T up_v = __shfl_up_sync(0xffffffffu, out_v, 1);
-                const int lx = s - l0;
-                const bool act = (unsigned)lx < 32u;
-                const int lw = lx & 31;
-                const int i = row + lw;
-                const int par = (s & 1) * kTZ * 32;
-                const T fyq = fy_v[lw], fzq = fz_v[lw], zbq = zb_v[(kTZ * 32 - par) + zr];
-                const T fxq = f_v[fxi];
-                const T xv = lx == 0 ? fxq : out_v;
-                const T yv = ly == 0 ? fyq : up_v;
-                const T zv = lz == 0 ? fzq : zbq;
-                const T hH = sd[i];
-                const T gi = sg[i];
-                const T rhs = gi + betaT * ((xv + yv) + zv);
-                P ipj = Ops::zero();
-                T vj;
-                if constexpr (MODE == 0) {
-                    const P fyp = fy_ip[lw], fzp = fz_ip[lw], zbp = zb_ip[(kTZ * 32 - par) + zr];
-                    const P fxp = f_ip[fxi];
-                    const P xip = lx == 0 ? fxp : out_ip;
-                    const P yip = ly == 0 ? fyp : up_ip;
-                    const P zip = lz == 0 ? fzp : zbp;
-                    const T hL = Ops::kLo ? sl[i] : T(0);
-                    const bool inm = hH >= T(0);  // H_jj, or -1 outside the mask
-                    bool ok = true;
-                    ipj = Ops::inv_pivot(hH, hL, a.beta, pc, xip, yip, zip, ok);
-                    if (!inm) ipj = Ops::zero();
-                    bad |= act & !(ok || !inm);
-                    vj = rhs * (T)Ops::hi(ipj);
-                    // every lane stores: an inactive lane writes back what it read
-                    sd[i] = act ? (T)Ops::hi(ipj) : hH;
-                    if (Ops::kLo) sl[i] = act ? (T)Ops::lo(ipj) : hL;
-                    zb_ip[par + zw] = ipj;
-                } else {
-                    vj = rhs * hH;  // stored 1/pi
+                for (int q = 0; q < C; ++q) nbq[q] = row_in && (unsigned)(lx + q) < (unsigned)nvalid ? nbp[lx + q] : 0u;
+            };
+            if (MODE != 1) load_bits(rg.lo - ly - tz<C>(lz));
+            cp_wait_all();
+            bar_warps2<kRows>();
+
+            // A step touches registers, shuffles and stores only -- a branch, or a load that has to
+            // follow the step's stores, costs more than its arithmetic -- so that the compiler can run
+            // one step's low parts under the next one's chain.  A lane outside its row (lx not in
+            // [0, 64)) computes on the wrapped index lx & 63 and only active lanes store; an inactive
+            // lane's outputs are read by no active lane at the next step.  A last chunk runs to its
+            // end: steps after the last reach no mask voxel, and their entries are not handed over.
+            Ent o = zero_ent((const Ent*)nullptr);  // this thread's values of the step before
+            bool bad = false;
+            for (int c = 0; c < nch; ++c) {
+                // a row's entries belong to this thread alone, so the chunk's inputs are read, and its
+                // H_jj formed, ahead of the chain
+                const int s0 = rg.lo + c * C, lx0 = s0 - ly - tz<C>(lz);
+                T gg[C], hH[C], hL[C];
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int i = vox(lx0 + q, row);
+                    gg[q] = sg[i];
+                    hH[q] = sd[i];
+                    if constexpr (MODE != 1) {
+                        const T h = form_h(hH[q], __popc((nbq[q] >> 1) & 0x3fu), a.beta, pc, hL[q]);
+                        hH[q] = nbq[q] & NB_IN ? h : T(-1);
+                    }
                 }
-                sg[i] = act ? vj : gi;
-                // an inactive lane's outputs are read by no active lane at the next step
-                out_ip = ipj;
-                out_v = vj;
-                zb_v[par + zw] = vj;
-                // outgoing faces go out as they are produced
-                const bool fx_out = act & (lx == 31) & ux.has(s - 31), fy_out = act & (ly == 31) & uy.has(s - 31),
-                           fz_out = act & (lz == kTZ - 1) & uz.has(s - (kTZ - 1));
-                const int zo = FN::z + zbase + lw;
-                if constexpr (MODE == 0) {
-                    st_if(fx_out, oip + FN::x + zw, ipj);
-                    st_if(fy_out, oip + FN::y + lz * 32 + lw, ipj);
-                    st_if(fz_out, oip + zo, ipj);
+                if (MODE != 1) load_bits(lx0 + C);
+                wait_chunk(&s_mbar[c], (unsigned)(par >> c) & 1u, a.spin_limit, a.istate);
+                // neighbours from outside the warp: the x-face record (used at lx = 0, in the chunk whose
+                // fetch brought it), the y face (lanes ly = 0), and for the lower plane the z face or
+                // what the warp below left one chunk ago
+                const Ent fx = f_in[FN::x + row];
+                const Ent* zp = wz == 0 ? f_in + FN::z + s0 * kTY + ly
+                                        : ring + ((c + 1) & 1) * C * kRows + (2 * wz - 1) * kTY + ly;
+                const int zpitch = wz == 0 ? kTY : kRows;
+                Ent fy[C], fz[C];
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    fy[q] = f_in[FN::y + lz * kTX + ((lx0 + q + ly) & (kTX - 1))];
+                    fz[q] = zp[q * zpitch];
                 }
-                const T vc = canon(vj);
-                st_if(fx_out, ov + FN::x + zw, vc);
-                st_if(fy_out, ov + FN::y + lz * 32 + lw, vc);
-                st_if(fz_out, ov + zo, vc);
-                {  // next step's diagonal t + 1 = s + 1 - lz: zbase(t + 1) = zbase(t) + max(0, min(t + 1, 62 - t))
-                    const int t = s - lz;
-                    zbase += max(0, min(t + 1, 62 - t));
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int lx = lx0 + q, i = vox(lx, row);
+                    const bool act = (unsigned)lx < (unsigned)kTX, first = lx == 0;
+                    auto ny_ = [&](T f, T own) { const T u = shfl_up(own, 1); return ly == 0 ? f : u; };
+                    auto nz_ = [&](T f, T own) { const T u = shfl_up(own, 16); return up == 0 ? f : u; };
+                    if constexpr (MODE != 1) {
+                        const Ent in = o;
+                        Ent x, y, z;
+                        x.x = first ? fx.x : in.x;
+                        y.x = ny_(fy[q].x, in.x);
+                        z.x = nz_(fz[q].x, in.x);
+                        if constexpr (sizeof(T) == 4) {
+                            x.y = first ? fx.y : in.y;
+                            y.y = ny_(fy[q].y, in.y);
+                            z.y = nz_(fz[q].y, in.y);
+                        }
+                        const T vx = first ? v_of(fx) : v_of(in), vy = ny_(v_of(fy[q]), v_of(in)), vz = nz_(v_of(fz[q]), v_of(in));
+                        const T rhs = gg[q] + betaT * ((vx + vy) + vz);
+                        const bool ok = pivot(hH[q], hL[q], a.beta, pc, x, y, z, o);
+                        bad |= act & !ok & (hH[q] >= T(0));
+                        const T vj = rhs * o.x;
+                        if constexpr (sizeof(T) == 4) o.z = vj;
+                        else o.y = vj;
+                        if (act) sd[i] = o.x;
+                        if constexpr (sizeof(T) == 4 && MODE == 2) {
+                            if (act && hH[q] >= 0.f)
+                                a.ip_lo_out[(long long)(z0 + lz) * nxy + (long long)(y0 + ly) * nx + x0 + lx] = o.y;
+                        }
+                    } else {
+                        const T vx = first ? fx : o, vy = ny_(fy[q], o), vz = nz_(fz[q], o);
+                        o = (gg[q] + betaT * ((vx + vy) + vz)) * hH[q];  // stored 1/pi
+                    }
+                    if (act) sg[i] = v_of(o);
+                    ring[((c & 1) * C + q) * kRows + row] = o;
                 }
-                bar_compute();
-              }
+                bar_warps<kSweep>();
             }
             if (bad) set_err(a.istate, FM_ERR_NOT_PD);
-            {
-                const int sx = X > 0 ? tile - 1 : -1, sy = Y > 0 ? tile - a.ntx : -1;
-                const int sz = Z > 0 ? tile - a.ntx * a.nty : -1;
-                if (mode == 0)
-                    unset_faces<P>(sx >= 0 ? face_ip(sx) : nullptr, sy >= 0 ? face_ip(sy) : nullptr,
-                                   sz >= 0 ? face_ip(sz) : nullptr);
-                unset_faces<T>(sx >= 0 ? face_v(sx) : nullptr, sy >= 0 ? face_v(sy) : nullptr,
-                               sz >= 0 ? face_v(sz) : nullptr);
-            }
-            // write back row-coalesced (warp lz writes its 32 rows, lane = x); a voxel on a hyperplane
-            // that was not swept lies outside the mask
-            const int nvalid = min(32, nx - x0);
-            const int z = z0 + wz;
-            if (z < nz && lane < nvalid) {
-                for (int ly2 = 0; ly2 < 32 && y0 + ly2 < ny; ++ly2) {
-                    const long long j = (long long)z * nxy + (long long)(y0 + ly2) * nx + x0 + lane;
-                    const int i = (wz * 32 + ly2) * 32 + lane;
-                    const bool in = rg.has(lane + ly2 + wz);
-                    v[j] = in ? sg[i] : T(0);
-                    if (mode == 0 && ipo) ipo[j] = in ? sd[i] : T(0);
-                    if (Ops::kLo && mode == 0 && a.ip_lo_out) a.ip_lo_out[j] = in ? (float)sl[i] : 0.0f;
-                }
+        }
+        __syncthreads();
+        // every warp: faces back to unset, then write back row-coalesced (lane = x); a voxel on a step
+        // that was not swept lies outside the mask
+        unset_faces<Ent>(px >= 0 ? face(px) : nullptr, py >= 0 ? face(py) : nullptr, pz >= 0 ? face(pz) : nullptr);
+#pragma unroll 4
+        for (int r = wz; r < kRows; r += kThreadsF / 32) {
+            const int y = y0 + r % kTY, z = z0 + r / kTY;
+            if (y >= ny || z >= nz) continue;
+            const long long j = (long long)z * nxy + (long long)y * nx + x0;
+#pragma unroll
+            for (int x = lane; x < kTX; x += 32) {
+                if (x >= nvalid) break;
+                const bool in = rg.has(x + r % kTY + tz<C>(r / kTY));
+                v[j + x] = in ? sg[vox(x, r)] : T(0);
+                if (MODE != 1 && ipo) ipo[j + x] = in ? sd[vox(x, r)] : T(0);
             }
         }
         __syncthreads();
-        par ^= (1u << nch) - 1u;
+        par ^= (2ull << (nch - 1)) - 1ull;
     }
 }
 
-// Deterministic sum of Q doubles over the compute warps (named barrier, the same tree as
-// block_sum over 8 warps); result valid in thread 0.
-template <int Q>
-__device__ __forceinline__ void block_sum_compute(double (&v)[Q], double* sbuf /* >= 32*Q */) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) v[q] = warp_sum(v[q]);
-    bar_compute();
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < Q; ++q) sbuf[q * 32 + wid] = v[q];
-    bar_compute();
-    if (wid == 0) {
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const double x = lane < kTZ ? sbuf[q * 32 + lane] : 0.0;
-            v[q] = warp_sum(x);
+// Sums of the two lists part[q * n + i] over i, in the order of a block of 320 threads (thread i
+// adds i, i + 320, .., then a tree over lanes and over the ten warps), whatever the block's size:
+// the sums decide the step sizes, and a fixed order keeps every solve reproducible bit for bit.
+// Result valid in thread 0.
+__device__ __forceinline__ void sum_columns(const double* part, int n, double (&out)[2], double* sbuf /* >= 64 */) {
+    constexpr int kOrder = 320;
+    const int lane = threadIdx.x & 31;
+    for (int w = threadIdx.x >> 5; w < kOrder / 32; w += blockDim.x >> 5) {
+        double v[2] = {0.0, 0.0};
+        for (int i = w * 32 + lane; i < n; i += kOrder) {
+            v[0] += __ldcg(part + i);
+            v[1] += __ldcg(part + n + i);
+        }
+        v[0] = warp_sum(v[0]);
+        v[1] = warp_sum(v[1]);
+        if (lane == 0) {
+            sbuf[w] = v[0];
+            sbuf[32 + w] = v[1];
         }
     }
-    bar_compute();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        out[0] = warp_sum(lane < kOrder / 32 ? sbuf[lane] : 0.0);
+        out[1] = warp_sum(lane < kOrder / 32 ? sbuf[32 + lane] : 0.0);
+    }
 }
 
-// Back substitution, streamed like the forward sweep: the reverse sweep of a tile needs, at
-// its local hyperplane s, the +x / +y neighbours' low-face values those tiles produce 31
-// steps earlier in their own reverse sweeps, and the +z neighbour's 7 (kTZ - 1) steps
-// earlier.  Every low-face voxel (lx = 0, ly = 0, lz = 0) goes to the face buffer as it is
-// computed (the z face by diagonals, as in the forward sweep), and a fetch warp polls the
-// entries each chunk of kCS reverse steps needs, with the same unset-pattern hand-off.
+// Waits (bounded) for a tile's p to be in memory.
+__device__ __forceinline__ bool wait_written(const int* flag, long long limit) {
+    long long n = 0;
+    while (ld_acquire(flag) == 0) {
+        if (++n > limit) return false;
+        __nanosleep(20);
+    }
+    return true;
+}
+
+// s + x y with Kahan compensation c, every operation rounded as written (a compiler that may
+// contract across the first, zero terms would give a sum that depends on the unrolling).
+__device__ __forceinline__ void kahan_add(float& s, float& c, float x, float y) {
+    const float a = __fmaf_rn(x, y, -c), t = __fadd_rn(s, a);
+    c = __fsub_rn(__fsub_rn(t, s), a);
+    s = t;
+}
+__device__ __forceinline__ void kahan_add(double& s, double& c, double x, double y) {
+    const double a = __fma_rn(x, y, -c), t = __dadd_rn(s, a);
+    c = __dsub_rn(__dsub_rn(t, s), a);
+    s = t;
+}
+
+// The dot products g'p and g_prev'p of half a unit (32 x 32 x 8 voxels at x0, y0, z0), a warp to a
+// plane: each lane sums a column of 32 voxels along y in order, in T with Kahan compensation, and
+// converts it to double once (per-product FP64 additions would queue on GB300's narrow FP64 pipe,
+// about 1/64 of the FP32 rate); the columns are added in double.  All of a column's loads are in
+// flight together.  p comes from other blocks of this launch.
 template <typename T>
-__global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
-    using P = typename PivOps<T>::P;
+__device__ __forceinline__ void unit_dots(const T* p, const T* g, const T* gp, int x0, int y0, int z0, const Geo& geo,
+                                          double (&acc)[2]) {
+    constexpr int B = sizeof(T) == 4 ? 32 : 16;  // voxels in flight
+    static_assert(kThreadsB == 32 * kTZ, "one column per thread");
+    const int x = x0 + (threadIdx.x & 31), z = z0 + (threadIdx.x >> 5);
+    if (x < geo.nx && z < geo.nz) {
+        T s0 = 0, c0 = 0, s1 = 0, c1 = 0;
+#pragma unroll
+        for (int r0 = 0; r0 < 32; r0 += B) {
+            T pv[B], gv[B], qv[B];
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                const int y = y0 + r0 + k;
+                const long long j = ((long long)z * geo.ny + y) * geo.nx + x;
+                const bool in = y < geo.ny;
+                pv[k] = in ? __ldcg(p + j) : T(0);
+                gv[k] = in && g ? g[j] : T(0);
+                qv[k] = in && gp ? gp[j] : T(0);
+            }
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                kahan_add(s0, c0, gv[k], pv[k]);
+                kahan_add(s1, c1, qv[k], pv[k]);
+            }
+        }
+        acc[0] = (double)s0 - (double)c0;
+        acc[1] = (double)s1 - (double)c1;
+    }
+}
+
+// Back substitution: the same sweep in mirrored coordinates (lx' = 63 - lx, ly' = 15 - ly,
+// lz' = 7 - lz), in which the +x, +y, +z neighbours are the predecessors.  A CTA that finds no
+// more tiles turns to the dot products, a unit at a time, as soon as the unit's tiles are written
+// back: most CTAs are idle by then, and a tile does not hold its CTA for them (9 us of tail after a
+// 7 us sweep when it did).  A column of 32 voxels spans two tiles, so the sums wait for both: they
+// end about 8 us after the last sweep.
+template <typename T>
+__global__ void __launch_bounds__(kThreadsB, sizeof(T) == 4 ? 2 : 1) k_ic_bwd(IcArgs a) {
+    constexpr int C = kCSB;
     extern __shared__ __align__(16) unsigned char smem[];
-    T* sv = (T*)smem;                 // [TZ][32][32]: v, then p
-    T* sip = sv + kTZ * 1024;         // 1/pi
-    T* f_p = sip + kTZ * 1024;        // incoming faces (the successors' -x, -y, -z faces)
-    T* zb = f_p + FN::n;              // [2][TZ][32]
-    __shared__ int s_tile, s_claim;
-    constexpr int kCS = kCSB, kNch = (kSteps + kCS - 1) / kCS;
-    __shared__ __align__(8) unsigned long long s_mbar[kNch];
+    T* sv = (T*)smem;            // v, then p
+    T* sip = sv + kVox;          // 1/pi
+    T* f_in = sip + kVox;        // incoming faces
+    T* ring = f_in + FN::n;      // step records [2][C][kRows]
+    __shared__ int s_tile;
+    __shared__ __align__(8) unsigned long long s_mbar[Steps<C>::chunks];
     __shared__ bool s_last;
     __shared__ double sbuf[2 * 32];
 
@@ -822,241 +857,168 @@ __global__ void __launch_bounds__(kThreadsB, 2) k_ic_bwd(IcArgs a) {
     const int nx = geo.nx, ny = geo.ny, nz = geo.nz;
     const long long nxy = (long long)nx * ny;
     const int tid = threadIdx.x, lane = tid & 31, wz = tid >> 5;
-    const T* vin = (const T*)a.vin;
-    const T* ipb = (const T*)a.ipb;
     T* p = (T*)a.p;
     const T* gd = (const T*)a.gdot;
     const T* gpd = (const T*)a.gpdot;
     const T beta = (T)a.beta;
-    unsigned char* faceb = (unsigned char*)a.face;
-    // backward faces live after the forward pivot and v faces of each tile
-    auto face_p = [&](int t) {
-        return (T*)(faceb + (size_t)t * face_bytes_per_tile<T>() + (size_t)FN::n * (sizeof(P) + sizeof(T)));
+    // backward faces live after each tile's forward records
+    auto face = [&](int t) {
+        return (T*)((unsigned char*)a.face + (size_t)t * face_bytes_per_tile<T>() + (size_t)FN::n * 16);
     };
 
     const int ntile = a.istate[I_NTILE];
     if (tid == 0) {
-        s_last = false;
-        for (int c = 0; c < kNch; ++c) mbar_init(&s_mbar[c], 1);
+        for (int c = 0; c < Steps<C>::chunks; ++c) mbar_init(&s_mbar[c], 1);
         if (ntile == 0 && blockIdx.x == 0 && a.tile_part) a.scal[S_GP] = a.scal[S_GPREVP] = 0.0;  // empty mask
     }
-    unsigned par = 0;  // bit c: phase parity of chunk c's barrier
+    unsigned long long par = 0;  // bit c: phase parity of chunk c's barrier
     for (;;) {
         if (tid == 0) {
             const int t = atomicAdd(a.ticket, 1);
-            s_claim = t;
             s_tile = t < ntile ? a.order[ntile - 1 - t] : -1;
         }
         __syncthreads();
         const int tile = s_tile;
         if (tile < 0) break;
         const int X = tile % a.ntx, Y = (tile / a.ntx) % a.nty, Z = tile / (a.ntx * a.nty);
-        const int x0 = X * 32, y0 = Y * 32, z0 = Z * kTZ;
-        const Range rg = tile_range(a.range, tile);
-        const int nch = (rg.hi - rg.lo) / kCS + 1;
+        const int x0 = X * kTX, y0 = Y * kTY, z0 = Z * kTZ;
+        const Range rg = tile_range<false>(a.range, tile);
+        const int nch = (rg.hi - rg.lo) / C + 1, nvalid = min(kTX, nx - x0);
+        const int px = X + 1 < a.ntx ? tile + 1 : -1, py = Y + 1 < a.nty ? tile + a.ntx : -1,
+                  pz = Z + 1 < a.ntz ? tile + a.ntx * a.nty : -1;
 
-        if (wz >= kTZ) {
-            // fetch warps: the +x, +y, +z neighbours' outgoing low faces, alternate chunks each
-            const int sx = X + 1 < a.ntx ? tile + 1 : -1, sy = Y + 1 < a.nty ? tile + a.ntx : -1;
-            const int sz = Z + 1 < a.ntz ? tile + a.ntx * a.nty : -1;
-            const Range rx = tile_range(a.range, sx), ry = tile_range(a.range, sy), rz = tile_range(a.range, sz);
-            bool ok = true;
-            for (int c = wz - kTZ; c < nch; c += kFetchB) {
-                T zv[kCS], qv[kCS];
-                int zi[kCS], zg[kCS], qi[kCS], qsrc[kCS];
-                unsigned want = 0;
-#pragma unroll
-                for (int q = 0; q < kCS; ++q) {
-                    // reverse step c * kCS + q is local hyperplane s; the +z face entry (lx, ly) is
-                    // used at s = lx + ly + kTZ - 1, the +x / +y entries at s = 31 + ly + lz / lx + lz
-                    const int s = rg.hi - (c * kCS + q);
-                    int which = 0;
-                    const bool in = s >= rg.lo;
-                    zi[q] = in ? z_entry(s - (kTZ - 1), lane) : -1;
-                    zg[q] = FN::z + zdiag(min(max(s - (kTZ - 1), 0), 62)) + lane;
-                    qi[q] = in ? xy_entry(s - 31, lane, which) : -1;
-                    qsrc[q] = which ? sy : sx;
-                    zv[q] = T(0);
-                    qv[q] = T(0);
-                    if (zi[q] >= 0 && rz.has(s - (kTZ - 1))) want |= 1u << q;
-                    if (qi[q] >= 0 && (which ? ry : rx).has(s - 31)) want |= 1u << (kCS + q);
-                }
-                unsigned todo = ok ? want : 0u;
-                long long tries = 0;
-                while (__any_sync(0xffffffffu, todo != 0u)) {
-#pragma unroll
-                    for (int q = 0; q < kCS; ++q) {
-                        if (todo & (1u << q)) zv[q] = ld_rlx(face_p(sz) + zg[q]);
-                        if (todo & (1u << (kCS + q))) qv[q] = ld_rlx(face_p(qsrc[q]) + qi[q]);
-                    }
-#pragma unroll
-                    for (int q = 0; q < kCS; ++q) {
-                        if ((todo & (1u << q)) && !unset(zv[q])) todo &= ~(1u << q);
-                        if ((todo & (1u << (kCS + q))) && !unset(qv[q])) todo &= ~(1u << (kCS + q));
-                    }
-                    if (++tries > a.spin_limit && __any_sync(0xffffffffu, todo != 0u)) {
-                        ok = false;
-#pragma unroll
-                        for (int q = 0; q < kCS; ++q) {
-                            if (todo & (1u << q)) zv[q] = T(0);
-                            if (todo & (1u << (kCS + q))) qv[q] = T(0);
-                        }
-                        want &= ~todo;
-                        todo = 0u;
-                    } else if (todo != 0u) {
-                        __nanosleep(20);
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < kCS; ++q) {
-                    if (zi[q] >= 0) f_p[zi[q]] = zv[q];
-                    if (qi[q] >= 0) f_p[qi[q]] = qv[q];
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&s_mbar[c]);
-            }
-            if (!ok) set_err(a.istate, FM_ERR_TIMEOUT);  // the host resets the faces with the error
+        if (wz > kWarps) {
+            fetch_faces<C, false>(f_in, a, face, px, py, pz, rg, nch, wz - kWarps - 1, kFetchB, s_mbar);
+        } else if (wz == kWarps) {
+            publish_faces<C, false>(ring, face(tile), a, X > 0 ? tile - 1 : -1, Y > 0 ? tile - a.ntx : -1,
+                                    Z > 0 ? tile - a.ntx * a.nty : -1, rg, nch);
         } else {
-            stage_row<T>(sv, vin, tid, x0, y0, z0, geo, T(0));
-            stage_row<T>(sip, ipb, tid, x0, y0, z0, geo, T(0));
+            stage_tile<T>(sv, (const T*)a.vin, x0, y0, z0, geo);
+            stage_tile<T>(sip, (const T*)a.ipb, x0, y0, z0, geo);
+            for (int i = tid; i < 2 * C * kRows; i += kRows) ring[i] = T(0);
             cp_wait_all();
-            for (int i = tid; i < 2 * kTZ * 32; i += kCompute) zb[i] = T(0);  // hyperplanes after the last are 0
-            bar_compute();
+            bar_warps2<kRows>();
 
-            // sweep in reverse, branch-free as in the forward kernel; the low-face entries a chunk
-            // produces go out after the chunk, read back from shared memory by every warp
-            const int ly = lane, lz = wz, l0 = ly + lz;
-            const int row = (lz * 32 + ly) * 32;
-            const int fxi = FN::x + lz * 32 + ly;
-            const T* fy = f_p + FN::y + lz * 32;
-            const T* fz = f_p + FN::z + ly * 32;
-            const int zr = (lz < kTZ - 1 ? lz + 1 : lz) * 32 + ly, zw = lz * 32 + ly;
-            T* op = face_p(tile);
-            // steps whose face entries a successor reads
-            const Range ux = tile_range(a.range, X > 0 ? tile - 1 : -1);
-            const Range uy = tile_range(a.range, Y > 0 ? tile - a.ntx : -1);
-            const Range uz = tile_range(a.range, Z > 0 ? tile - a.ntx * a.nty : -1);
-            T out = 0;
+            // mirrored row (ly, lz) of the sweep and the actual row it stands for
+            const int ly = lane & 15, up = lane >> 4, lz = 2 * wz + up, mrow = lz * kTY + ly, row = kRows - 1 - mrow;
+            T o = 0;
+            T vv[C], bi[C];
+            auto load_chunk = [&](int lx) {
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int i = vox(kTX - 1 - lx - q, row);
+                    vv[q] = sv[i];
+                    bi[q] = beta * sip[i];
+                }
+            };
+            load_chunk(rg.lo - ly - tz<C>(lz));
             for (int c = 0; c < nch; ++c) {
-                wait_chunk(&s_mbar[c], (par >> c) & 1u, a.spin_limit, a.istate);
-                const T fxv = f_p[fxi];  // used at s = 31 + l0, in the chunk whose fetch brought it
+                const int s0 = rg.lo + c * C, lx0 = s0 - ly - tz<C>(lz);
+                wait_chunk(&s_mbar[c], (unsigned)(par >> c) & 1u, a.spin_limit, a.istate);
+                const T fx = f_in[FN::x + mrow];
+                const T* zp = wz == 0 ? f_in + FN::z + s0 * kTY + ly
+                                      : ring + ((c + 1) & 1) * C * kRows + (2 * wz - 1) * kTY + ly;
+                const int zpitch = wz == 0 ? kTY : kRows;
+                T fy[C], fz[C];
 #pragma unroll
-                for (int q = 0; q < kCS; ++q) {
-                    const int s = rg.hi - (c * kCS + q);
-                    if (s < rg.lo) break;
-                    const T dn = __shfl_down_sync(0xffffffffu, out, 1);
-                    const int lx = s - l0;
-                    const bool act = (unsigned)lx < 32u;
-                    const int lw = lx & 31;
-                    const int i = row + lw;
-                    const int par = (s & 1) * kTZ * 32;
-                    const T fyv = fy[lw], fzv = fz[lw], zbv = zb[(kTZ * 32 - par) + zr];
-                    const T px = lx == 31 ? fxv : out;
-                    const T py = ly == 31 ? fyv : dn;
-                    const T pz = lz == kTZ - 1 ? fzv : zbv;
-                    const T vi = sv[i];
-                    const T pj = vi + beta * sip[i] * ((px + py) + pz);
-                    // every lane stores (an inactive lane writes back what it read); an inactive
-                    // lane's outputs are read by no active lane at the next step
-                    sv[i] = act ? pj : vi;
-                    out = pj;
-                    zb[par + zw] = pj;
-                    bar_compute();
+                for (int q = 0; q < C; ++q) {
+                    fy[q] = f_in[FN::y + lz * kTX + ((lx0 + q + ly) & (kTX - 1))];
+                    fz[q] = zp[q * zpitch];
                 }
-                // low faces produced at local hyperplanes s0..s1 of this chunk: x face (ly, lz) is
-                // this thread's lx = 0 voxel, produced at s = l0; y face (lx, lz) was produced by
-                // lane 0 of warp lz, one per step, and lane q stores step s1 - q; z face diagonal
-                // s1 - wz (warps 0..kCS-1) holds entries (lx, ly) of the lz = 0 plane
-                const int s1 = rg.hi - c * kCS, s0 = max(s1 - kCS + 1, rg.lo);
-                const int sy_ = s1 - lane, lxy = sy_ - lz;
-                const int sz_ = s1 - wz, lxz = sz_ - ly;
-                const T vx = sv[row], vy = sv[lz * 1024 + (lxy & 31)], vz = sv[ly * 32 + (lxz & 31)];
-                const int zo = FN::z + zdiag(min(max(sz_, 0), 62)) - max(0, sz_ - 31) + (lxz & 31);
-                st_if(l0 >= s0 && l0 <= s1 && ux.has(l0 + 31), op + FN::x + zw, canon(vx));
-                st_if(lane < kCS && sy_ >= s0 && (unsigned)lxy < 32u && uy.has(sy_ + 31), op + FN::y + lz * 32 + (lxy & 31), canon(vy));
-                st_if(wz < kCS && sz_ >= s0 && (unsigned)lxz < 32u && uz.has(sz_ + kTZ - 1), op + zo, canon(vz));
-            }
-
-            {
-                const int sx = X + 1 < a.ntx ? tile + 1 : -1, sy = Y + 1 < a.nty ? tile + a.ntx : -1;
-                const int sz = Z + 1 < a.ntz ? tile + a.ntx * a.nty : -1;
-                unset_faces<T>(sx >= 0 ? face_p(sx) : nullptr, sy >= 0 ? face_p(sy) : nullptr,
-                               sz >= 0 ? face_p(sz) : nullptr);
-            }
-            // write back, then the dot products (off the wavefront's critical path).  The loads of
-            // g and g_prev go out kWb rows at a time, so that a tile pays a few memory round
-            // trips here, not one per row (the CTA claims its next tile only after this).  A
-            // thread's 32 products are summed in T with Kahan compensation and converted to
-            // double once: per-product FP64 additions would queue on GB300's narrow FP64 pipe
-            // (about 1/64 of the FP32 rate) behind every other CTA on the SM.
-            const int nvalid = min(32, nx - x0);
-            const int z = z0 + wz;
-            const bool zin = z < nz && lane < nvalid;
-            const int nrow = min(32, ny - y0);
-            double acc[2] = {0.0, 0.0};
-            if (zin) {
-                constexpr int kWb = 16;
-                T s0 = 0, c0 = 0, s1 = 0, c1 = 0;  // Kahan sums of g p and g_prev p
-                for (int r0 = 0; r0 < 32; r0 += kWb) {
-                    T pv[kWb], gv[kWb], gpv[kWb];
+                T v1[C], b1[C];
 #pragma unroll
-                    for (int k = 0; k < kWb; ++k) {
-                        const int ly2 = r0 + k;
-                        const bool in = ly2 < nrow;
-                        const long long j = (long long)z * nxy + (long long)(y0 + (in ? ly2 : 0)) * nx + x0 + lane;
-                        pv[k] = in ? sv[(wz * 32 + ly2) * 32 + lane] : T(0);
-                        gv[k] = (gd && in) ? gd[j] : T(0);
-                        gpv[k] = (gpd && in) ? gpd[j] : T(0);
-                        if (in) p[j] = pv[k];
-                    }
+                for (int q = 0; q < C; ++q) {
+                    v1[q] = vv[q];
+                    b1[q] = bi[q];
+                }
+                load_chunk(lx0 + C);
 #pragma unroll
-                    for (int k = 0; k < kWb; ++k) {
-                        const T y0k = gv[k] * pv[k] - c0, t0 = s0 + y0k;
-                        c0 = (t0 - s0) - y0k;
-                        s0 = t0;
-                        const T y1k = gpv[k] * pv[k] - c1, t1 = s1 + y1k;
-                        c1 = (t1 - s1) - y1k;
-                        s1 = t1;
-                    }
+                for (int q = 0; q < C; ++q) {
+                    const int lx = lx0 + q;
+                    const T yu = shfl_up(o, 1), zu = shfl_up(o, 16);
+                    const T x = lx == 0 ? fx : o, y = ly == 0 ? fy[q] : yu, z = up == 0 ? fz[q] : zu;
+                    o = v1[q] + b1[q] * ((x + y) + z);
+                    if ((unsigned)lx < (unsigned)kTX) sv[vox(kTX - 1 - lx, row)] = o;
+                    ring[((c & 1) * C + q) * kRows + mrow] = o;
                 }
-                acc[0] = (double)s0 - (double)c0;
-                acc[1] = (double)s1 - (double)c1;
-            }
-            if (a.tile_part) {
-                block_sum_compute(acc, sbuf);
-                if (tid == 0) {
-                    a.tile_part[s_claim] = acc[0];  // by claim position: the order is fixed, so is the sum
-                    a.tile_part[ntile + s_claim] = acc[1];
-                    __threadfence();
-                    const int prev = atomicAdd(a.done, 1);
-                    s_last = (prev == ntile - 1);
-                    if (s_last) __threadfence();
-                }
+                bar_warps<kSweep>();
             }
         }
         __syncthreads();
-        if (a.tile_part && s_last) {
+        // every warp: faces back to unset and write-back of p
+        unset_faces<T>(px >= 0 ? face(px) : nullptr, py >= 0 ? face(py) : nullptr, pz >= 0 ? face(pz) : nullptr);
+#pragma unroll 4
+        for (int r = wz; r < kRows; r += kThreadsB / 32) {
+            const int y = y0 + r % kTY, z = z0 + r / kTY;
+            if (y >= ny || z >= nz) continue;
+            const long long j = (long long)z * nxy + (long long)y * nx + x0;
+#pragma unroll
+            for (int x = lane; x < kTX; x += 32)
+                if (x < nvalid) p[j + x] = sv[vox(x, r)];
+        }
+        __syncthreads();
+        if (a.tile_part && tid == 0) {  // the tile's p is in memory: its unit may be summed
+            __threadfence();
+            st_release(a.written + tile, 1);
+        }
+        par ^= (2ull << (nch - 1)) - 1ull;
+    }
+    if (!a.tile_part) return;
+    const int nhalf = 2 * a.istate[I_NUNIT];  // every unit in two halves along x
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) {
+            const int u = atomicAdd(a.unit_ticket, 1);
+            s_tile = u < nhalf ? u : -1;
+            if (u < nhalf) {
+                const int t = a.unit[nhalf / 2 - 1 - u / 2], Y = (t / a.ntx) % a.nty;
+                bool ok = wait_written(a.written + t, a.spin_limit);
+                if (!(Y & 1) && Y + 1 < a.nty && (a.range[t + a.ntx] & 255u) != 255u)
+                    ok = wait_written(a.written + t + a.ntx, a.spin_limit) && ok;
+                if (!ok) set_err(a.istate, FM_ERR_TIMEOUT);
+            }
+        }
+        __syncthreads();
+        const int u = s_tile;
+        if (u < 0) break;
+        const int t = a.unit[nhalf / 2 - 1 - u / 2], X = t % a.ntx, Y = (t / a.ntx) % a.nty, Z = t / (a.ntx * a.nty);
+        double acc[2] = {0.0, 0.0};
+        unit_dots<T>(p, gd, gpd, X * kTX + 32 * (u & 1), (Y & ~1) * kTY, Z * kTZ, geo, acc);
+        block_sum<2>(acc, sbuf);
+        if (tid == 0) {
+            // by place, in blocks of 32 x 32 x 8 voxels (blocks outside the mask stay 0)
+            const int n32 = (nx + 31) / 32, m32 = (ny + 31) / 32, x32 = 2 * X + (u & 1);
+            const int at = x32 + n32 * ((Y >> 1) + m32 * Z);
+            if (x32 < n32) {
+                a.tile_part[at] = acc[0];
+                a.tile_part[a.npart + at] = acc[1];
+            }
+            __threadfence();
+            const int prev = atomicAdd(a.done, 1);
+            s_last = (prev == nhalf - 1);
+            if (s_last) __threadfence();
+        }
+        __syncthreads();
+        if (s_last) {
             double tot[2];
-            sum_partials<2>(a.tile_part, ntile, tot, sbuf);
+            sum_columns(a.tile_part, a.npart, tot, sbuf);
             if (tid == 0) {
                 a.scal[S_GP] = tot[0];
                 a.scal[S_GPREVP] = tot[1];
                 if (!isfinite(tot[0]) || !isfinite(tot[1])) set_err(a.istate, FM_ERR_NONFINITE);
             }
-            __syncthreads();
-            if (tid == 0) s_last = false;
         }
-        par ^= (1u << nch) - 1u;
     }
 }
 
-cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, int* range,
+cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, unsigned* range,
                              cudaStream_t s) {
-    k_ic_range<<<ntiles, kCompute, 0, s>>>(geo, ntx, nty, nb, range);
+    k_ic_range<<<ntiles, kRows, 0, s>>>(geo, ntx, nty, nb, range);
     return cudaGetLastError();
 }
-cudaError_t launch_ic_order(const int* order, const int* range, int ntiles, int* out, int* istate, cudaStream_t s) {
-    k_ic_order<<<2, 1024, 0, s>>>(order, range, ntiles, out, istate);
+cudaError_t launch_ic_order(const int* order, const unsigned* range, int ntx, int nty, int ntiles, int* out, int* istate,
+                            cudaStream_t s) {
+    k_ic_order<<<3, 1024, 0, s>>>(order, range, ntx, nty, ntiles, out, istate);
     return cudaGetLastError();
 }
 
@@ -1072,6 +1034,8 @@ static cudaError_t prep() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_ic_fwd<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FwdSmem<T>::bytes);
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_ic_fwd<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FwdSmem<T>::bytes);
+    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_ic_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)BwdSmem<T>::bytes);
     if (e == cudaSuccess) done = true;
@@ -1084,7 +1048,7 @@ int ic_max_blocks_per_sm(bool bwd) {
     int n = 0;
     const cudaError_t e =
         bwd ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ic_bwd<T>, kThreadsB, BwdSmem<T>::bytes)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ic_fwd<T, 0>, kThreadsIC, FwdSmem<T>::bytes);
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ic_fwd<T, 0>, kThreadsF, FwdSmem<T>::bytes);
     return e == cudaSuccess ? n : 0;
 }
 
@@ -1102,10 +1066,12 @@ template <typename T>
 cudaError_t launch_ic_fwd(const IcArgs& a, int grid, cudaStream_t s) {
     cudaError_t e = prep<T>();
     if (e != cudaSuccess) return e;
-    if (a.d)
-        k_ic_fwd<T, 0><<<grid, kThreadsIC, FwdSmem<T>::bytes, s>>>(a, piv_scal(a.beta));
+    if (a.d && a.ip_lo_out)
+        k_ic_fwd<T, 2><<<grid, kThreadsF, FwdSmem<T>::bytes, s>>>(a, piv_scal(a.beta));
+    else if (a.d)
+        k_ic_fwd<T, 0><<<grid, kThreadsF, FwdSmem<T>::bytes, s>>>(a, piv_scal(a.beta));
     else
-        k_ic_fwd<T, 1><<<grid, kThreadsIC, FwdSmem<T>::bytes, s>>>(a, piv_scal(a.beta));
+        k_ic_fwd<T, 1><<<grid, kThreadsF, FwdSmem<T>::bytes, s>>>(a, piv_scal(a.beta));
     return cudaGetLastError();
 }
 

@@ -14,7 +14,7 @@ from synth import make_volume
 pytestmark = pytest.mark.gpu
 
 TOL = {"fp64": (1e-11, 1e-10), "fp32": (3e-5, 2e-4)}
-SHAPES = [(97, 70, 35), (64, 33, 16), (31, 100, 9)]  # nx, ny, nz: ragged and exact 32 x 32 x 8 tiles
+SHAPES = [(97, 70, 35), (64, 33, 16), (31, 100, 9)]  # nx, ny, nz: ragged and exact 64 x 16 x 8 tiles
 
 
 def _masks(nx, ny, nz):
@@ -29,7 +29,7 @@ def _masks(nx, ny, nz):
         "corners": corners,
         "all": np.ones_like(one),
         "two slabs": (x < 5) | (x >= nx - 5),
-        "layers": (z == 0) | (z == nz - 1) | (y % 32 == 31),
+        "layers": (z == 0) | (z == nz - 1) | (y % 16 == 15) | (x == 64),
         "staircase": np.abs(x * ny - y * nx) < 2 * nx,
         "sparse": rng.uniform(size=one.shape) < 0.01,
         "holes": rng.uniform(size=one.shape) < 0.9,
