@@ -52,6 +52,7 @@ struct fm_ctx {
     unsigned* tile_rng = nullptr;  // per tile: steps of the sweeps that reach a mask voxel
     int ntx = 0, nty = 0, ntz = 0, ntiles = 0, npart = 0;
     int ic_wxy = 2, ic_wz = 1;  // forward tile claim order weights
+    int lanes = 1;  // lanes that share a voxel in the data-term kernels
     int nsm = 0, grid_data = 0, grid_ls = 0, grid_ic = 0, grid_icb = 0;  // grid_icb: backward IC sweep
     int base_data = 0, base_ls = 0, base_ic = 0, base_icb = 0;
     int occ_icb = 0;  // resident back-substitution blocks per SM the kernel allows
@@ -886,11 +887,13 @@ int pwls_t(fm_ctx* c, const void* wt, int niter, void* w0) {
 bool set_ls_grid(fm_ctx* c) {
     DataArgs probe{};
     probe.nc = c->nc;
+    probe.L = c->L;
     probe.literal = c->literal;
     probe.wf = c->wf;
     const int occ = c->o.precision == FM_FP64 ? ls_max_blocks_per_sm<double>(probe) : ls_max_blocks_per_sm<float>(probe);
     if (occ < 1) return false;
-    const long long nblk = (c->nv + kThreads - 1) / kThreads;
+    c->lanes = c->o.precision == FM_FP64 ? 1 : data_lanes(probe);
+    const long long nblk = (c->nv * c->lanes + kThreads - 1) / kThreads;
     c->grid_ls = (int)std::max(1LL, std::min<long long>(nblk, (long long)occ * c->nsm));
     c->base_ls = c->grid_ls;
     return true;
@@ -967,9 +970,9 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
         c->own_stream = true;
     }
     if (cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return bail(FM_ERR_CUDA);
-    const long long nblk = (c->nv + kThreads - 1) / kThreads;
-    c->grid_data = (int)std::max(1LL, std::min<long long>(nblk, 4LL * c->nsm));
     if (!set_ls_grid(c)) return bail(FM_ERR_CUDA);
+    const long long nblk = (c->nv * c->lanes + kThreads - 1) / kThreads;
+    c->grid_data = (int)std::max(1LL, std::min<long long>(nblk, 4LL * c->nsm));
     c->ntx = (nx + kTileX - 1) / kTileX;
     c->nty = (ny + kTileY - 1) / kTileY;
     const int tz = o.precision == FM_FP64 ? ic_tz<double>() : ic_tz<float>();
@@ -1121,6 +1124,7 @@ int fm_set_data(fm_ctx* c, const void* y, const void* smap, const double* te, co
             pr.m[pr.P] = m;
             pr.n[pr.P] = n;
             pr.dt[pr.P] = te[m] - te[n];
+            pr.dtf[pr.P] = (float)pr.dt[pr.P];
             pr.dtt[pr.P] = (float)(pr.dt[pr.P] * 683565275.57643158);  // 2^32 / (2 pi)
             pr.gmag[pr.P] = std::abs(lgam[(size_t)m * c->L + n]);
             pr.gph[pr.P] = c->wf ? std::arg(lgam[(size_t)m * c->L + n]) : 0.0;

@@ -57,6 +57,7 @@ struct Pairs {
     double dt[kMaxPairs];   // t_m - t_n
     double gmag[kMaxPairs]; // L |Gamma_mn| (1 in the field-map case)
     double gph[kMaxPairs];  // angle Gamma_mn (0 in the field-map case)
+    float dtf[kMaxPairs];   // t_m - t_n as float (a conversion on the device runs on the narrow FP64 pipe)
     float dtt[kMaxPairs];   // (t_m - t_n) 2^32 / (2 pi): a field value's fixed-point phase per unit
 };
 
@@ -378,6 +379,7 @@ template <typename T> cudaError_t launch_grad(const DataArgs& a, int grid, cudaS
 template <typename T> cudaError_t launch_ls(const DataArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_pdiag(const DataArgs& a, int mode, int grid, cudaStream_t s);
 template <typename T> int ls_max_blocks_per_sm(const DataArgs& a);
+int data_lanes(const DataArgs& a);  // FP32: lanes that share a voxel in the data-term kernels
 template <typename T> cudaError_t launch_rb_black(const DataArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_rb_red(const DataArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, unsigned* range,

@@ -15,7 +15,7 @@
 // FP32 mode evaluates the voxel arithmetic in float and sums in double; FP64 mode is double
 // throughout.  Global sums are block partials reduced in a fixed order (bitwise
 // reproducible).
-#include <cooperative_groups.h>
+#include <type_traits>
 
 #include "fm_internal.h"
 
@@ -52,9 +52,11 @@ __device__ __forceinline__ double sinc_wrapped(double u) { return u == 0.0 ? 1.0
 // fraction of a turn in the bits of the float slot: 2^32 is one turn, so a difference of two
 // angles wraps into [-1/2, 1/2) turn by the integer subtraction's own wrap-around (Eq. 11's
 // "mod pi" of the half angle).  The water-fat model and FP64 mode store radians.
+
 __device__ __forceinline__ float fixed_to_radians(float bits) {
     return (float)__float_as_int(bits) * 1.4629180792671596e-09f;  // 2 pi / 2^32
 }
+// A stored coil angle in radians, for the general evaluator, which takes either storage.
 template <typename T>
 __device__ __forceinline__ T coil_angle(const DataArgs& a, T y) {
     if constexpr (sizeof(T) == 4) return a.wf ? y : fixed_to_radians(y);
@@ -68,6 +70,14 @@ __device__ __forceinline__ unsigned phase_fixed(float w, float dtt) {
     return (unsigned)(unsigned long long)__float2ll_rn(hi) + (unsigned)__float2int_rn(lo);
 }
 
+// w (t_m - t_n) as a fixed-point angle, reduced by turns in float before the conversion (the 64-bit
+// conversion of phase_fixed runs on the narrow FP64 pipe).
+__device__ __forceinline__ unsigned phase_fixed_32(float w, float dtt) {
+    const float hi = w * dtt, lo = fmaf(w, dtt, -hi);
+    const float k = fmaf(hi, 2.3283064365386963e-10f, 12582912.0f) - 12582912.0f;  // whole turns
+    return (unsigned)__float2int_rn(fmaf(k, -4294967296.0f, hi)) + (unsigned)__float2int_rn(lo);
+}
+
 // sin(2 pi x)/(2 pi x) for x in [-1/2, 1/2] turns as a degree-5 polynomial in x^2: the
 // discrete minimax fit derived by csrc/sinc_poly.py (truncation error 6.1e-8, 2.1e-7 in
 // float Horner form).
@@ -77,21 +87,6 @@ constexpr float kSincT2 = 12.987038612365723f;
 constexpr float kSincT3 = -12.193624496459961f;
 constexpr float kSincT4 = 6.580165386199951f;
 constexpr float kSincT5 = -1.9852460622787476f;
-
-// The wrapped angle in turns from the difference t of two fixed-point angles that carry the
-// offset 2^31 + 2^8: one funnel shift makes the float 1 + (x + 1/2) in [1, 2) with 23
-// fraction bits (the 2^8 rounds the 9 bits the shift drops), and subtracting 1.5 is exact.
-__device__ __forceinline__ float turns_of(unsigned t) {
-    return __uint_as_float(__funnelshift_r(t, 0x7Fu, 9)) - 1.5f;
-}
-__device__ __forceinline__ float sinc_turns(float x) {
-    const float v = x * x;
-    float p = fmaf(kSincT5, v, kSincT4);
-    p = fmaf(p, v, kSincT3);
-    p = fmaf(p, v, kSincT2);
-    p = fmaf(p, v, kSincT1);
-    return fmaf(p, v, kSincT0);
-}
 
 // The inner coil sum of Eq. 10 for one echo pair (m, n) in FP32, two coils d per
 // instruction (the f32x2 forms of add, multiply and fused multiply-add, rounding each
@@ -142,6 +137,13 @@ __device__ __forceinline__ float coil_pair_sum_x2(const float2 (&Wm)[NC], const 
 __device__ __forceinline__ void sin_cos(float x, float* s, float* c) { sincosf(x, s, c); }
 __device__ __forceinline__ void sin_cos(double x, double* s, double* c) { sincos(x, s, c); }
 
+// t_m - t_n of pair p in the voxel type
+template <typename T>
+__device__ __forceinline__ T pair_dt(const Pairs& pr, int p) {
+    if constexpr (sizeof(T) == 4) return pr.dtf[p];
+    else return pr.dt[p];
+}
+
 // ------------------------------------------------------------------ per-voxel data term
 
 // Adds the data-term pieces of voxel j at field value w.  NC > 0: literal curvature over
@@ -156,7 +158,7 @@ __device__ __forceinline__ void eval_voxel(const DataArgs& a, long long j /* com
     const T2* coils = (const T2*)a.coils;
     T c_acc = 0, g_acc = 0, d_acc = 0;
     for (int p = 0; p < a.pr.P; ++p) {
-        const T dt = (T)a.pr.dt[p];
+        const T dt = pair_dt<T>(a.pr, p);
         const T2 R = pairs[(size_t)p * nv + j];
         const T th = R.y + w * dt;
         T s, c;
@@ -173,7 +175,7 @@ __device__ __forceinline__ void eval_voxel(const DataArgs& a, long long j /* com
                 for (int dd = 0; dd < NC; ++dd) {
                     const T2 q = coils[((size_t)n * NC + dd) * nv + j];
                     ad[dd] = q.x;
-                    psi[dd] = coil_angle(a, q.y) + w * dt;
+                    psi[dd] = q.y + w * dt;
                 }
                 T inner = 0;
 #pragma unroll
@@ -181,33 +183,14 @@ __device__ __forceinline__ void eval_voxel(const DataArgs& a, long long j /* com
                     const T2 q = coils[((size_t)m * NC + cc) * nv + j];
                     T acc = 0;
 #pragma unroll
-                    for (int dd = 0; dd < NC; ++dd) acc += ad[dd] * sinc_wrapped(wrap_angle(psi[dd] - coil_angle(a, q.y)));
+                    for (int dd = 0; dd < NC; ++dd) acc += ad[dd] * sinc_wrapped(wrap_angle(psi[dd] - q.y));
                     inner += q.x * acc;
                 }
                 d_acc += dt * dt * inner;
             } else {
-                // runtime coil count; also the water-fat model, whose angle r_cdmn carries the
+                // runtime coil count (FP64), and the water-fat model, whose angle r_cdmn carries the
                 // phase of Gamma_mn and |r_cdmn| the factor L |Gamma_mn| (0 and 1 otherwise)
                 const int m = a.pr.m[p], n = a.pr.n[p], nc = a.nc;
-                if constexpr (sizeof(T) == 4) {
-                    if (!a.wf) {
-                        // field-map model in FP32: fixed-point angles (as in coil_pair_sum_x2)
-                        const unsigned ph = phase_fixed(w, a.pr.dtt[p]) + 0x80000100u;
-                        float inner = 0;
-                        for (int cc = 0; cc < nc; ++cc) {
-                            const float2 q = coils[((size_t)m * nc + cc) * nv + j];
-                            const unsigned bm = (unsigned)__float_as_int(q.y) - ph;
-                            float acc = 0;
-                            for (int dd = 0; dd < nc; ++dd) {
-                                const float2 r = coils[((size_t)n * nc + dd) * nv + j];
-                                acc += r.x * sinc_turns(turns_of((unsigned)__float_as_int(r.y) - bm));
-                            }
-                            inner += q.x * acc;
-                        }
-                        d_acc += dt * dt * inner;
-                        continue;  // the curvature is the last piece of the pair's work
-                    }
-                }
                 const T gph = (T)a.pr.gph[p];
                 T inner = 0;
                 for (int cc = 0; cc < nc; ++cc) {
@@ -255,7 +238,7 @@ __device__ __forceinline__ void eval_voxel_fixed(const DataArgs& a, long long j 
     for (int m = 0; m < L; ++m) {
 #pragma unroll
         for (int n = m + 1; n < L; ++n, ++p) {
-            const T dt = (T)a.pr.dt[p];
+            const T dt = pair_dt<T>(a.pr, p);
             const T th = R[p].y + w * dt;
             T s, c;
             sin_cos(th * T(0.5), &s, &c);
@@ -269,14 +252,14 @@ __device__ __forceinline__ void eval_voxel_fixed(const DataArgs& a, long long j 
                 } else {
                     T psi[NCL];
 #pragma unroll
-                    for (int dd = 0; dd < NCL; ++dd) psi[dd] = coil_angle(a, W[n][dd].y) + w * dt;
+                    for (int dd = 0; dd < NCL; ++dd) psi[dd] = W[n][dd].y + w * dt;
                     T inner = 0;
 #pragma unroll
                     for (int cc = 0; cc < NCL; ++cc) {
                         T acc = 0;
 #pragma unroll
                         for (int dd = 0; dd < NCL; ++dd)
-                            acc += W[n][dd].x * sinc_wrapped(wrap_angle(psi[dd] - coil_angle(a, W[m][cc].y)));
+                            acc += W[n][dd].x * sinc_wrapped(wrap_angle(psi[dd] - W[m][cc].y));
                         inner += W[m][cc].x * acc;
                     }
                     d_acc += dt * dt * inner;
@@ -289,11 +272,155 @@ __device__ __forceinline__ void eval_voxel_fixed(const DataArgs& a, long long j 
     curv = T(2) * d_acc;
 }
 
-// Dispatch to the unrolled three-echo path when it applies.
+// FP32 literal curvature of up to NR coils (two coils per instruction, so NR is even) and any
+// echo count: a pair's coil weights in registers, coils past a.nc counting as |W| = 0.  Bound by
+// FP32 issue at 6 slots per term of NR^2; the runtime-count form it replaces took 11 to 15 per
+// term.  133 x 117 x 45 voxels, four coils and echoes: line search 163 -> 129 us, gradient 32 -> 28.
+template <int NR, bool COST, bool CURV>
+__device__ __forceinline__ void eval_padded(const DataArgs& a, long long j, float w, float& cost, float& grad,
+                                            float& curv) {
+    const size_t nv = (size_t)a.geo.nv;
+    const float2* pairs = (const float2*)a.pairs + j;
+    const float2* coils = (const float2*)a.coils + j;
+    const int nc = a.nc, L = a.L;
+    auto load = [&](float2 (&W)[NR], int m) {
+#pragma unroll
+        for (int c = 0; c < NR; ++c) W[c] = c < nc ? coils[(size_t)(m * nc + c) * nv] : make_float2(0.f, 0.f);
+    };
+    float c_acc = 0, g_acc = 0, d_acc = 0;
+    int p = 0;
+    for (int m = 0; m + 1 < L; ++m) {
+        float2 Wm[NR];
+        if (CURV) load(Wm, m);
+        for (int n = m + 1; n < L; ++n, ++p) {
+            float2 Wn[NR];
+            if (CURV) load(Wn, n);
+            const float dt = a.pr.dtf[p];
+            const float2 R = pairs[(size_t)p * nv];
+            float s, c;
+            sin_cos((R.y + w * dt) * 0.5f, &s, &c);
+            if (COST) c_acc += R.x * (s * s);
+            g_acc += dt * R.x * (s * c);
+            if (CURV) d_acc += dt * dt * coil_pair_sum_x2<NR>(Wm, Wn, phase_fixed_32(w, a.pr.dtt[p]));
+        }
+    }
+    cost = 4.f * c_acc;
+    grad = 4.f * g_acc;
+    curv = 2.f * d_acc;
+}
+
+// Evaluator codes of the kernels below (with_evaluator): kPadded + NR is eval_padded.
+constexpr int kPadded = 100;
+
+// The three-echo path in registers, the padded one, or the general one.
 template <typename T, int NC, bool COST, bool CURV>
 __device__ __forceinline__ void eval_any(const DataArgs& a, long long j, T w, T& cost, T& grad, T& curv) {
-    if (NC != 0 && a.L == 3) eval_voxel_fixed<T, (NC == 0 ? 1 : NC), 3, COST, CURV>(a, j, w, cost, grad, curv);
-    else eval_voxel<T, NC, COST, CURV>(a, j, w, cost, grad, curv);
+    if constexpr (NC > kPadded) {
+        eval_padded<NC - kPadded, COST, CURV>(a, j, w, cost, grad, curv);
+    } else if constexpr (sizeof(T) == 4 && NC > 1) {
+        eval_voxel_fixed<T, NC, 3, COST, CURV>(a, j, w, cost, grad, curv);
+    } else {
+        if (NC != 0 && a.L == 3) eval_voxel_fixed<T, (NC == 0 ? 1 : NC), 3, COST, CURV>(a, j, w, cost, grad, curv);
+        else eval_voxel<T, NC, COST, CURV>(a, j, w, cost, grad, curv);
+    }
+}
+
+// ------------------------------------------------------------------ voxels shared by lanes
+
+// FP32 literal curvature of more than eight coils, any echo count: SP = 8 lanes share a voxel.
+// Lane slice sl takes the rows c = sl, sl + 8, .. of every pair's sum over (c, d), and the pairs
+// sl, sl + 8, .. of the cost and gradient; the slices' results add up to the voxel's.
+//
+// Bound by FP32 issue: a pair has N_c^2 terms of about 6 slots.  One thread per voxel left the
+// chip idle where coils are many and voxels few (74 x 74 x 10 voxels with 32 coils: 14,000 mask
+// voxels for 152 SMs, each thread 3072 terms in sequence, one coil load per term and no reuse): the
+// line search took 630 us, with 8 lanes per voxel 228 (gradient 108, 47).  Below nine coils the
+// padded form is the faster one (four coils: line search 129 us, with four lanes per voxel 205).  A lane holds eight
+// d in registers for all of its rows, two terms per instruction as in coil_pair_sum_x2; the lanes
+// of a slice are neighbouring voxels, so that a load fetches whole 32-byte sectors of each coil's
+// plane.
+
+// sum over the rows c = sl, sl + SP, .. of |W_cm| sum_{d < DB} |W_dn| sinc(..), entries past the last
+// of nd coils counting as |W_dn| = 0.
+template <int SP, int DB>
+__device__ __forceinline__ float slice_block(const float2* Wm, const float2* Wn, size_t nv, int nc, int sl, int nd,
+                                             unsigned ph) {
+    unsigned an[DB];
+    float2 ad[DB / 2];
+#pragma unroll
+    for (int i = 0; i < DB; ++i, Wn += nv) {
+        const float2 r = i < nd ? *Wn : make_float2(0.f, 0.f);
+        an[i] = (unsigned)__float_as_int(r.y) + ph + 0x80000100u;
+        if (i & 1) ad[i / 2].y = r.x;
+        else ad[i / 2].x = r.x;
+    }
+    const float2 c5 = make_float2(kSincT5, kSincT5), c4 = make_float2(kSincT4, kSincT4);
+    const float2 c3 = make_float2(kSincT3, kSincT3), c2 = make_float2(kSincT2, kSincT2);
+    const float2 c1 = make_float2(kSincT1, kSincT1), c0 = make_float2(kSincT0, kSincT0);
+    const float2 mid = make_float2(-1.5f, -1.5f);
+    float inner = 0;
+    Wm += (size_t)sl * nv;
+#pragma unroll 2
+    for (int c = sl; c < nc; c += SP, Wm += SP * nv) {
+        const float2 q = *Wm;
+        const unsigned bm = (unsigned)__float_as_int(q.y);
+        float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int h = 0; h < DB / 2; ++h) {
+            const float2 f = make_float2(__uint_as_float(__funnelshift_r(an[2 * h] - bm, 0x7Fu, 9)),
+                                         __uint_as_float(__funnelshift_r(an[2 * h + 1] - bm, 0x7Fu, 9)));
+            const float2 x = __fadd2_rn(f, mid);
+            const float2 v = __fmul2_rn(x, x);
+            float2 p = __ffma2_rn(c5, v, c4);
+            p = __ffma2_rn(p, v, c3);
+            p = __ffma2_rn(p, v, c2);
+            p = __ffma2_rn(p, v, c1);
+            p = __ffma2_rn(p, v, c0);
+            acc = __ffma2_rn(ad[h], p, acc);
+        }
+        inner = fmaf(q.x, acc.x + acc.y, inner);
+    }
+    return inner;
+}
+
+// This slice's share of voxel k's cost, gradient and curvature at field value w.
+template <int SP, bool COST>
+__device__ __forceinline__ void eval_slice(const DataArgs& a, long long k, int sl, float w, float& cost, float& grad,
+                                           float& curv) {
+    const size_t nv = (size_t)a.geo.nv;
+    const float2* pairs = (const float2*)a.pairs + k;
+    const float2* coils = (const float2*)a.coils + k;
+    const int nc = a.nc, P = a.pr.P;
+    float c_acc = 0, g_acc = 0, d_acc = 0;
+    for (int p = sl; p < P; p += SP) {
+        const float dt = a.pr.dtf[p];
+        const float2 R = pairs[(size_t)p * nv];
+        float s, c;
+        sin_cos((R.y + w * dt) * 0.5f, &s, &c);
+        if (COST) c_acc += R.x * (s * s);
+        g_acc += dt * R.x * (s * c);
+    }
+    for (int p = 0; p < P; ++p) {
+        const float dt = a.pr.dtf[p];
+        const unsigned ph = phase_fixed_32(w, a.pr.dtt[p]);
+        const float2 *Wm = coils + (size_t)a.pr.m[p] * nc * nv, *Wn = coils + (size_t)a.pr.n[p] * nc * nv;
+        float inner = 0;
+        int d0 = 0;
+        for (; d0 + 4 < nc; d0 += 8, Wn += 8 * nv) inner += slice_block<SP, 8>(Wm, Wn, nv, nc, sl, nc - d0, ph);
+        if (d0 < nc) inner += slice_block<SP, 4>(Wm, Wn, nv, nc, sl, nc - d0, ph);
+        d_acc += dt * dt * inner;
+    }
+    cost = 4.f * c_acc;
+    grad = 4.f * g_acc;
+    curv = 2.f * d_acc;
+}
+
+// The sum of v over the SP lanes of a voxel (lane = slice * (32 / SP) + voxel), in all of them.
+template <int SP>
+__device__ __forceinline__ float slice_sum(float v) {
+#pragma unroll
+    for (int o = 32 / SP; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // ------------------------------------------------------------------ gradient pass
@@ -319,21 +446,36 @@ __global__ void __launch_bounds__(kThreads, 2) k_grad(DataArgs a) {
     // the thread's cost and penalty sums in T with Kahan compensation, converted to double
     // once (per-voxel FP64 additions would queue on GB300's narrow FP64 pipe)
     T cs = 0, cc = 0, rs = 0, rc = 0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nm;
-         k += (long long)gridDim.x * blockDim.x) {
+    constexpr int SP = NC < 0 ? -NC : 1, VW = 32 / SP;  // lanes per voxel, voxels per warp
+    const int lane = threadIdx.x & 31, sl = lane / VW;
+    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long first = SP == 1 ? tid : tid / 32 * VW, stride = (long long)gridDim.x * blockDim.x / SP;
+    for (long long kb = first; kb < nm; kb += stride) {  // SP > 1: the same trips for a whole warp
+        const long long k = SP == 1 ? kb : min(kb + lane % VW, nm - 1);
+        const bool mine = SP == 1 || (sl == 0 && kb + lane % VW < nm);
         const long long j = a.vlist[k];
-        const uint8_t b = a.nb[j];
         const T wj = upd(j);
-        w_out[j] = wj;
         T lap = 0, reg = 0;
-        if (b & NB_XM) lap += wj - upd(j - 1);
-        if (b & NB_YM) lap += wj - upd(j - nx);
-        if (b & NB_ZM) lap += wj - upd(j - nxy);
-        if (b & NB_XP) { const T e = wj - upd(j + 1); lap += e; reg += e * e; }
-        if (b & NB_YP) { const T e = wj - upd(j + nx); lap += e; reg += e * e; }
-        if (b & NB_ZP) { const T e = wj - upd(j + nxy); lap += e; reg += e * e; }
+        if (mine) {
+            const uint8_t b = a.nb[j];
+            w_out[j] = wj;
+            if (b & NB_XM) lap += wj - upd(j - 1);
+            if (b & NB_YM) lap += wj - upd(j - nx);
+            if (b & NB_ZM) lap += wj - upd(j - nxy);
+            if (b & NB_XP) { const T e = wj - upd(j + 1); lap += e; reg += e * e; }
+            if (b & NB_YP) { const T e = wj - upd(j + nx); lap += e; reg += e * e; }
+            if (b & NB_ZP) { const T e = wj - upd(j + nxy); lap += e; reg += e * e; }
+        }
         T cst, gr, cu;
-        eval_any<T, NC, true, true>(a, k, wj, cst, gr, cu);
+        if constexpr (SP > 1) {
+            eval_slice<SP, true>(a, k, sl, wj, cst, gr, cu);
+            cst = slice_sum<SP>(cst);
+            gr = slice_sum<SP>(gr);
+            cu = slice_sum<SP>(cu);
+            if (!mine) continue;
+        } else {
+            eval_any<T, NC, true, true>(a, k, wj, cst, gr, cu);
+        }
         if (g) g[j] = gr + beta * lap;
         if (d) d[j] = cu;
         {
@@ -376,15 +518,24 @@ __global__ void __launch_bounds__(kThreads, 2) k_grad(DataArgs a) {
 // the first nb blocks take part -- one mask voxel per thread at most (fewer threads with
 // several voxels each measured slower: each voxel is a chain of dependent gathers) -- and the
 // rest leave before the first grid barrier, which then counts the nb participants only.
+// Resident blocks per SM the line search is compiled for.  The grid follows from it, and with the
+// grid each thread's voxels and the order of every sum, so it is stated rather than left to the
+// compiler's register count: 128 registers for eight coils in registers and the lane-shared form
+// (whose polynomial constants otherwise do not stay in registers), 64 to 80 for the others.
+template <typename T, int NC> constexpr int ls_blocks() {
+    return sizeof(T) == 8 ? (NC == 0 ? 3 : 2) : NC == 8 || NC < 0 || NC > kPadded + 4 ? 2 : NC > kPadded ? 3 : 4;
+}
+
 template <typename T, int NC>
-__global__ void __launch_bounds__(kThreads) k_ls(DataArgs a) {
+__global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a) {
     __shared__ double sbuf[4 * 32];
     __shared__ double s_tot[4];
     const T* w = (const T*)a.w_out;
     const T* z = (const T*)a.z_new;
     const int it = a.istate[I_ITER];
     const long long nm = a.istate[I_NMASK];
-    const int nb = (int)max(1LL, min((long long)gridDim.x, (nm + kThreads - 1) / kThreads));
+    constexpr int SP = NC < 0 ? -NC : 1, VW = 32 / SP;  // lanes per voxel, voxels per warp
+    const int nb = (int)max(1LL, min((long long)gridDim.x, (nm * SP + kThreads - 1) / kThreads));
     if ((int)blockIdx.x >= nb) return;
     const int nx = a.geo.nx;
     const long long nxy = (long long)nx * a.geo.ny;
@@ -473,7 +624,7 @@ __global__ void __launch_bounds__(kThreads) k_ls(DataArgs a) {
         const T aT = (T)alpha;
         // each thread sums its few voxels in the voxel type, then the block and the grid in FP64
         T t1 = 0, t2 = 0;
-        if (NC == 1) {
+        if constexpr (NC == 1) {
             // HBM-bound form (one coil, or the combined curvature): four voxels per pass with
             // every load issued before the arithmetic, while all four exist; the rest one by
             // one.  The voxels are visited in the same order as below, and a voxel with z = 0
@@ -505,6 +656,18 @@ __global__ void __launch_bounds__(kThreads) k_ls(DataArgs a) {
                 if (zj == T(0)) continue;
                 T cst, gr, cu;
                 eval_any<T, NC, false, true>(a, k, w[j] + aT * zj, cst, gr, cu);
+                t1 += zj * gr;
+                t2 += zj * zj * cu;
+            }
+        } else if constexpr (SP > 1) {
+            // each slice adds its own share: the sums run over all lanes anyway
+            const int lane = threadIdx.x & 31;
+            const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
+            for (long long k = warp * VW + lane % VW; k < nm; k += (long long)nb * blockDim.x / SP) {
+                const long long j = a.vlist[k];
+                const T zj = __ldcg(z + j);  // written by another thread before the grid barrier
+                T cst, gr, cu;
+                eval_slice<SP, false>(a, k, lane / VW, w[j] + aT * zj, cst, gr, cu);
                 t1 += zj * gr;
                 t2 += zj * zj * cu;
             }
@@ -584,60 +747,61 @@ __global__ void __launch_bounds__(kThreads) k_pdiag(DataArgs a, int mode) {
 
 // ------------------------------------------------------------------ launchers
 
-template <typename T, int NC>
-static cudaError_t grad_nc(const DataArgs& a, int grid, cudaStream_t s) {
-    k_grad<T, NC><<<grid, kThreads, 0, s>>>(a);
-    return cudaGetLastError();
+// Calls f(integral constant NC) with the evaluator of a context: 1 coil-combined curvature (or one
+// coil); 2, 4, 8 that many coils and three echoes in registers; kPadded + NR (FP32) other literal
+// curvatures of up to NR coils; -8 (FP32) more than eight coils, eight lanes per voxel; 0 a runtime
+// coil count with one thread per voxel (FP64, and the water-fat model).
+template <typename T, typename F>
+static auto with_evaluator(const DataArgs& a, F f) {
+    if (!a.literal) return f(std::integral_constant<int, 1>());
+    if (a.wf) return f(std::integral_constant<int, 0>());
+    if (sizeof(T) == 8 || a.L == 3) {
+        switch (a.nc) {
+            case 2: return f(std::integral_constant<int, 2>());
+            case 4: return f(std::integral_constant<int, 4>());
+            case 8: return f(std::integral_constant<int, 8>());
+            default: break;
+        }
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (a.nc <= 2) return f(std::integral_constant<int, kPadded + 2>());
+        if (a.nc <= 4) return f(std::integral_constant<int, kPadded + 4>());
+        if (a.nc <= 6) return f(std::integral_constant<int, kPadded + 6>());
+        if (a.nc <= 8) return f(std::integral_constant<int, kPadded + 8>());
+        return f(std::integral_constant<int, -8>());
+    }
+    return f(std::integral_constant<int, 0>());
+}
+
+int data_lanes(const DataArgs& a) {
+    return with_evaluator<float>(a, [](auto nc) { return decltype(nc)::value < 0 ? -decltype(nc)::value : 1; });
 }
 
 template <typename T>
 cudaError_t launch_grad(const DataArgs& a, int grid, cudaStream_t s) {
-    if (!a.literal) return grad_nc<T, 1>(a, grid, s);
-    if (a.wf) return grad_nc<T, 0>(a, grid, s);
-    switch (a.nc) {
-        case 2: return grad_nc<T, 2>(a, grid, s);
-        case 4: return grad_nc<T, 4>(a, grid, s);
-        case 8: return grad_nc<T, 8>(a, grid, s);
-        default: return grad_nc<T, 0>(a, grid, s);
-    }
-}
-
-template <typename T, int NC>
-static cudaError_t ls_nc(const DataArgs& a, int grid, cudaStream_t s) {
-    DataArgs copy = a;
-    void* args[] = {&copy};
-    return cudaLaunchCooperativeKernel((const void*)k_ls<T, NC>, dim3(grid), dim3(kThreads), args, 0, s);
+    return with_evaluator<T>(a, [&](auto nc) {
+        k_grad<T, decltype(nc)::value><<<grid, kThreads, 0, s>>>(a);
+        return cudaGetLastError();
+    });
 }
 
 template <typename T>
 cudaError_t launch_ls(const DataArgs& a, int grid, cudaStream_t s) {
-    if (!a.literal) return ls_nc<T, 1>(a, grid, s);
-    if (a.wf) return ls_nc<T, 0>(a, grid, s);
-    switch (a.nc) {
-        case 2: return ls_nc<T, 2>(a, grid, s);
-        case 4: return ls_nc<T, 4>(a, grid, s);
-        case 8: return ls_nc<T, 8>(a, grid, s);
-        default: return ls_nc<T, 0>(a, grid, s);
-    }
-}
-
-template <typename T, int NC>
-static int ls_occ() {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ls<T, NC>, kThreads, 0) != cudaSuccess) return 0;
-    return n;
+    return with_evaluator<T>(a, [&](auto nc) {
+        DataArgs copy = a;
+        void* args[] = {&copy};
+        return cudaLaunchCooperativeKernel((const void*)k_ls<T, decltype(nc)::value>, dim3(grid), dim3(kThreads), args, 0, s);
+    });
 }
 
 template <typename T>
 int ls_max_blocks_per_sm(const DataArgs& a) {
-    if (!a.literal) return ls_occ<T, 1>();
-    if (a.wf) return ls_occ<T, 0>();
-    switch (a.nc) {
-        case 2: return ls_occ<T, 2>();
-        case 4: return ls_occ<T, 4>();
-        case 8: return ls_occ<T, 8>();
-        default: return ls_occ<T, 0>();
-    }
+    return with_evaluator<T>(a, [&](auto nc) {
+        int n = 0;
+        const cudaError_t e =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ls<T, decltype(nc)::value>, kThreads, 0);
+        return e == cudaSuccess ? n : 0;
+    });
 }
 
 template <typename T>
