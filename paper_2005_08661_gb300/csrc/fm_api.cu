@@ -38,6 +38,7 @@ struct fm_ctx {
     int *vlist = nullptr, *chunk_off = nullptr;
     void *w[2] = {nullptr, nullptr}, *z[2] = {nullptr, nullptr}, *g[2] = {nullptr, nullptr};
     void *d = nullptr, *p = nullptr, *v = nullptr, *ip = nullptr;
+    void* zw = nullptr;  // T2 compact [nv]: (z, w) of the line search
     double *scal = nullptr, *partials = nullptr, *tile_part = nullptr;
     void* face = nullptr;
     size_t face_bytes = 0;  // per-tile IC face buffers (the forward part starts unset: all bits set)
@@ -132,7 +133,7 @@ void free_all(fm_ctx* c) {
             for (cudaEvent_t& e : b)
                 if (e) cudaEventDestroy(e);
     void* bufs[] = {c->pairs, c->coils, c->w0, c->nb, c->vlist, c->chunk_off, c->w[0], c->w[1], c->z[0], c->z[1], c->g[0],
-                    c->g[1], c->d, c->p, c->v, c->ip, c->scal, c->partials, c->face, c->tile_part, c->rho,
+                    c->g[1], c->d, c->p, c->v, c->ip, c->zw, c->scal, c->partials, c->face, c->tile_part, c->rho,
                     c->hist_cost, c->hist_alpha, c->hist_mu, c->istate, c->icint, c->order, c->order_act, c->tile_rng, c->ict_L,
                     c->st_y[0], c->st_y[1], c->st_s[0], c->st_s[1], c->st_m[0], c->st_m[1], c->w_io, c->ip_lo,
                     c->ict_tab, c->ict_qflags, c->ict_w0};
@@ -546,6 +547,7 @@ cudaError_t iteration(fm_ctx* c, int cur) {
     a.p = c->p;
     a.z_old = c->z[cur];
     a.z_new = c->z[nxt];
+    a.zw = c->zw;
     a.w_out = c->w[nxt];
     a.g = c->g[cur];
     a.d = c->d;
@@ -1026,7 +1028,7 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     A(&c->chunk_off, (size_t)nchunks * sizeof(int));
     A(&c->w0, vb);
     for (int k = 0; k < 2; ++k) { A(&c->w[k], vb); A(&c->z[k], vb); A(&c->g[k], vb); }
-    A(&c->d, vb); A(&c->p, vb); A(&c->v, vb); A(&c->ip, vb); A(&c->rho, vb);
+    A(&c->d, vb); A(&c->p, vb); A(&c->v, vb); A(&c->ip, vb); A(&c->rho, vb); A(&c->zw, 2 * vb);
     A(&c->scal, S_NSCAL * sizeof(double));
     A(&c->partials, std::max<size_t>(8 * (size_t)std::max(c->grid_data, c->grid_ls), nchunks) * sizeof(double));
     c->face_bytes = (size_t)c->ntiles *

@@ -245,6 +245,7 @@ struct DataArgs {
     const void* p;         // T [nv]
     const void* z_old;     // T [nv]
     void* z_new;           // T [nv]
+    void* zw;              // T2 [nv] compact order: (z, w) of the line search
     const void* g_prev;    // T [nv]
     const void* ip_in;     // T [nv] stored inverse pivots (red-black apply) or null
     void* ip_out;          // T [nv] inverse pivots out (red-black factor) or null
