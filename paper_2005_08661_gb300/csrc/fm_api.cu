@@ -57,8 +57,11 @@ struct fm_ctx {
     int nsm = 0, grid_data = 0, grid_ls = 0, grid_ic = 0, grid_icb = 0;  // grid_icb: backward IC sweep
     int base_data = 0, base_ls = 0, base_ic = 0, base_icb = 0;
     int occ_icb = 0;  // resident back-substitution blocks per SM the kernel allows
-    int grid_ict = 0, base_ict = 0, block_ict = 0;  // drop-tolerance IC sweeps (persistent, level barriers)
-    int grid_ictg = 0, base_ictg = 0;                // the same for the table-driven sweeps
+    int grid_ict = 0, base_ict = 0;  // drop-tolerance IC: row wavefront (0: volume takes the level sweeps)
+    int grid_ictg = 0, base_ictg = 0, block_ict = 0;  // its table-driven sweeps (persistent, level barriers)
+    double *ict_xch = nullptr, *ict_part = nullptr;   // row wavefront: exchange buffer, dot products
+    size_t ict_xch_bytes = 0;
+    int4* ict_rows = nullptr;
     // drop-tolerance IC: the held pattern (dx, dy, dz per offset, plane order), its device
     // tables, the factor planes [nh + 2][nv] and the candidate fill offsets of the check
     std::vector<int> ict_off, ict_qoff;
@@ -136,7 +139,7 @@ void free_all(fm_ctx* c) {
                     c->g[1], c->d, c->p, c->v, c->ip, c->zw, c->scal, c->partials, c->face, c->tile_part, c->rho,
                     c->hist_cost, c->hist_alpha, c->hist_mu, c->istate, c->icint, c->order, c->order_act, c->tile_rng, c->ict_L,
                     c->st_y[0], c->st_y[1], c->st_s[0], c->st_s[1], c->st_m[0], c->st_m[1], c->w_io, c->ip_lo,
-                    c->ict_tab, c->ict_qflags, c->ict_w0};
+                    c->ict_tab, c->ict_qflags, c->ict_w0, c->ict_xch, c->ict_part, c->ict_rows};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (int k = 0; k < 2; ++k) {
@@ -163,6 +166,7 @@ cudaError_t reset_dev(fm_ctx* c) {
     cudaError_t e = cudaMemsetAsync(c->istate + I_ERR, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = reset_barrier(c);
     if (e == cudaSuccess && c->face) e = cudaMemsetAsync(c->face, 0xff, c->face_bytes, c->stream);
+    if (e == cudaSuccess && c->ict_xch) e = cudaMemsetAsync(c->ict_xch, 0xff, c->ict_xch_bytes, c->stream);
     return e;
 }
 
@@ -461,9 +465,19 @@ cudaError_t run_ict(fm_ctx* c, const void* d, const void* g, void* p, const void
         e = launch_ict_tau<T>(t, c->o.droptol, c->grid_data, c->stream);
         if (e != cudaSuccess) return e;
     }
-    const bool base = c->ict_tb.nh == kIctBaseOffsets;  // the unrolled kernels hold exactly the base pattern
+    // the row wavefront holds exactly the base pattern
+    const bool base = c->ict_tb.nh == kIctBaseOffsets && c->grid_ict > 0;
+    if (base) {
+        e = cudaMemsetAsync(c->icint, 0, 4 * sizeof(int), c->stream);
+        if (e != cudaSuccess) return e;
+        a.rows = c->ict_rows;
+        a.xch = c->ict_xch;
+        a.part = c->ict_part;
+        a.ticket = c->icint + 0;
+        a.done = c->icint + 2;
+    }
     if (prof) prof_record(c->ev[slot][FM_K_IC_FWD][0], c->stream);
-    e = base ? launch_ict_fwd<T>(a, c->grid_ict, c->block_ict, c->stream)
+    e = base ? launch_ictw_fwd<T>(a, c->grid_ict, c->stream)
              : launch_ictg_fwd<T>(a, c->grid_ictg, c->block_ict, c->stream);
     if (prof) {
         prof_record(c->ev[slot][FM_K_IC_FWD][1], c->stream);
@@ -475,7 +489,8 @@ cudaError_t run_ict(fm_ctx* c, const void* d, const void* g, void* p, const void
         if (e != cudaSuccess) return e;
     }
     if (prof) prof_record(c->ev[slot][FM_K_IC_BWD][0], c->stream);
-    e = base ? launch_ict_bwd<T>(a, c->grid_ict, c->block_ict, c->stream)
+    a.ticket = c->icint + 1;
+    e = base ? launch_ictw_bwd<T>(a, c->grid_ict, c->stream)
              : launch_ictg_bwd<T>(a, c->grid_ictg, c->block_ict, c->stream);
     if (prof) {
         prof_record(c->ev[slot][FM_K_IC_BWD][1], c->stream);
@@ -1003,18 +1018,22 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
         const long long cols = (long long)ny * nz;
         const long long per_sm = (cols + c->nsm - 1) / c->nsm;
         c->block_ict = (int)std::min<long long>(kIctThreads, std::max<long long>(32, (per_sm + 31) / 32 * 32));
-        const int occ = o.precision == FM_FP64 ? ict_max_blocks_per_sm<double>(c->block_ict)
-                                               : ict_max_blocks_per_sm<float>(c->block_ict);
-        if (occ < 1) return bail(FM_ERR_CUDA);
-        c->grid_ict = (int)std::max(1LL, std::min<long long>((cols + c->block_ict - 1) / c->block_ict,
-                                                             (long long)occ * c->nsm));
-        c->base_ict = c->grid_ict;
         const int occg = o.precision == FM_FP64 ? ictg_max_blocks_per_sm<double>(c->block_ict)
                                                 : ictg_max_blocks_per_sm<float>(c->block_ict);
         if (occg < 1) return bail(FM_ERR_CUDA);
         c->grid_ictg = (int)std::max(1LL, std::min<long long>((cols + c->block_ict - 1) / c->block_ict,
                                                               (long long)occg * c->nsm));
         c->base_ictg = c->grid_ictg;
+        // row wavefront: blocks claim row groups, eight one-warp blocks per SM at most.  Its exchange
+        // buffer holds 32 lanes per row group, so thin volumes (few rows per plane) of large size
+        // would need many times their factor; they take the table-driven sweeps.
+        const Geo geo{nx, ny, nz, c->nv};
+        const size_t xb = ictw_exchange_bytes(geo), limit = std::max<size_t>((size_t)1 << 30, 4 * kIctPlanes * sizeof(double) * (size_t)c->nv);
+        if (xb <= limit) {
+            c->ict_xch_bytes = xb;
+            c->grid_ict = std::min(ictw_units(geo), 8 * c->nsm);
+            c->base_ict = c->grid_ict;
+        }
     }
     const size_t vb = (size_t)c->nv * c->ts;
     const int P = necho * (necho - 1) / 2;
@@ -1041,6 +1060,12 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     A(&c->order, 2 * (size_t)c->ntiles * sizeof(int));
     A(&c->order_act, 3 * (size_t)c->ntiles * sizeof(int));  // and the dot-product units
     A(&c->tile_rng, (size_t)c->ntiles * sizeof(unsigned));
+    if (c->ict_xch_bytes) {
+        const int units = ictw_units(Geo{nx, ny, nz, c->nv});
+        A(&c->ict_xch, c->ict_xch_bytes);
+        A(&c->ict_part, 2 * (size_t)units * sizeof(double));
+        A(&c->ict_rows, (size_t)units * sizeof(int4));
+    }
 
     if (!ok) { cudaGetLastError(); return bail(FM_ERR_OOM); }
 #ifndef FM_IC_WXY
@@ -1057,7 +1082,8 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
         cudaMemset(c->scal, 0, S_NSCAL * sizeof(double)) != cudaSuccess ||
         cudaMemset(c->istate, 0, I_NISTATE * sizeof(int)) != cudaSuccess ||
         cudaMemset(c->nb, 0, (size_t)c->nv) != cudaSuccess ||
-        cudaMemset(c->face, 0xff, c->face_bytes) != cudaSuccess)  // forward faces start unset
+        cudaMemset(c->face, 0xff, c->face_bytes) != cudaSuccess ||  // faces start unset
+        (c->ict_xch && cudaMemset(c->ict_xch, 0xff, c->ict_xch_bytes) != cudaSuccess))
         return bail(FM_ERR_CUDA);
     *out = c;
     return FM_OK;
@@ -1173,6 +1199,7 @@ int fm_set_data(fm_ctx* c, const void* y, const void* smap, const double* te, co
                                               : launch_setup<float>(a, c->stream);
     if (e == cudaSuccess) e = launch_ic_ranges(a.geo, c->ntx, c->nty, c->ntiles, c->nb, c->tile_rng, c->stream);
     if (e == cudaSuccess) e = launch_ic_order(c->order, c->tile_rng, c->ntx, c->nty, c->ntiles, c->order_act, c->istate, c->stream);
+    if (e == cudaSuccess && c->ict_rows) e = launch_ictw_rows(a.geo, c->nb, c->ict_rows, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "setup kernel");
     // the IC sweeps leave out tiles outside the mask: their inverse pivots and their part of the dot
     // products are 0
@@ -1332,8 +1359,8 @@ int fm_ic_apply(fm_ctx* c, const void* g, void* p) {
         if (e == cudaSuccess)
             e = f64 ? launch_rb_red<double>(a, c->grid_data, c->stream) : launch_rb_red<float>(a, c->grid_data, c->stream);
     } else {
-        // the sweeps leave out tiles outside the mask
-        if (c->o.precond != FM_PC_ICT) FM_CK(cudaMemsetAsync(p, 0, (size_t)c->nv * c->ts, c->stream), "clear");
+        // the sweeps leave out what lies outside the mask
+        FM_CK(cudaMemsetAsync(p, 0, (size_t)c->nv * c->ts, c->stream), "clear");
         e = c->o.precision == FM_FP64 ? run_ic<double>(c, nullptr, g, p, nullptr, nullptr)
                                       : run_ic<float>(c, nullptr, g, p, nullptr, nullptr);
     }

@@ -20,20 +20,18 @@
 //
 // Schedule.  The fill offsets d, e, f link voxels of one x + y + z hyperplane, so the IC(0)
 // wavefront does not apply.  With level t = x + 2y + 3z every offset in P points to a strictly
-// lower level (t(a) = t(d) = t(f) = -1, t(b) = t(e) = -2, t(c) = -3), so one persistent kernel
-// sweeps the levels in order -- thread <-> (y, z) column, voxel x = t - 2y - 3z -- with a
-// barrier between levels; the back substitution sweeps them in reverse.  A level's work is
-// FP64 arithmetic on the active columns, so the blocks are sized to spread the columns over
-// every SM (a volume with few columns runs one-warp blocks), and the barrier is the bounded
-// grid barrier of a cooperative launch -- or a block barrier when one block holds every
-// column.  The factor stores 1 / L_ii, so every entry costs a multiply, and each row issues
-// all of its loads from the earlier rows before the dependency chain starts.
+// lower level (t(a) = t(d) = t(f) = -1, t(b) = t(e) = -2, t(c) = -3).  Groups of 32 rows walk along x, a
+// lane two steps behind the lane below, and hand their records on as they go ("row wavefront"
+// below); the back substitution is the walk mirrored.  The factor stores 1 / L_ii, so every entry
+// costs a multiply.
 //
 // Deeper fill.  When the tolerance keeps entries beyond level 1, the pattern P grows: the host
 // holds any set of offsets (up to kIctMaxOffsets), builds the correction pairs of each offset
 // by the same offset arithmetic (pairs (p1, p2) with o_p1 - o_p2 = o) and a level function
 // t = x + B y + C z under which every held offset points to a lower level, and the
-// table-driven kernels k_ictg_fwd / k_ictg_bwd sweep it.
+// table-driven kernels k_ictg_fwd / k_ictg_bwd sweep it: one persistent kernel, thread <-> (y, z)
+// column, voxel x = t - B y - C z, with a barrier between levels (the bounded grid barrier of a
+// cooperative launch, or a block barrier when one block holds every column).
 //
 // Exactness.  The held factor is the exact drop-tolerance factor as long as no entry outside
 // the held pattern survives.  With the factor in hand, k_ict_check forms every would-be entry
@@ -139,139 +137,499 @@ __device__ __forceinline__ bool level_sync(const IctArgs& a) {
     return grid_barrier(a.istate, a.spin_limit);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kIctThreads) k_ict_fwd(IctArgs a) {
-    const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
-    const long long nxy = (long long)nx * ny, nv = a.geo.nv;
-    double* Lp = a.L;
-    auto P = [&](int k, long long j) -> double* { return Lp + (size_t)k * nv + j; };
+// ------------------------------------------------------------------ row wavefront (base pattern)
+//
+// The two substitutions of the base pattern without level barriers.  A one-warp block holds 32
+// consecutive rows (lane = y) of one plane z and walks them along x, each lane two steps behind the
+// lane below: row y's voxel x is computed at step s = x + 2 lane, so that the -y neighbours b = (x, y-1)
+// and d = (x+1, y-1) are the lower lane's values of two steps and one step ago (shuffles) and
+// a = (x-1, y) is the lane's own.  The rows c = (x, y), e = (x+1, y), f = (x, y+1) of plane z-1 come
+// from the block that holds that plane: e is one record per lane and step, c is the e of the step
+// before, f the upper lane's e of the next step.  Records of a step go to an exchange buffer as they
+// are computed and are their own ready signal, as the IC(0) sweeps' face entries are: an entry
+// holds an all-ones pattern that is never stored until its value arrives, its one reader polls it
+// (bounded), and sets it back.  Two more kinds of record cross between the row groups of a plane:
+// the last lane's to the next group (its b and d), the first lane's to the group below in plane
+// z+1 (the last lane's f).  Blocks claim their rows through a ticket in (z, y) order, so whom a
+// block waits for has claimed before it.  Only steps that reach a mask voxel are walked and handed
+// over.  The back substitution is the same walk mirrored.
+//
+// A step is a chain of FP64 operations (one warp per SM: 16 cycles an operation), a block runs as
+// far behind plane z-1 as the hand-off takes, and no barrier is left: 74 x 74 x 10 voxels, 32 coils,
+// factor + forward 1012 -> 606 us, back substitution 904 -> 254; the level sweeps pay about 4 us on
+// each of 247 levels.  They stay for grown patterns (table-driven), whose offsets reach further.
+
+constexpr int kRec = 6;  // doubles of a record: R, Y, A, B, D, F (1/L_ii, y and the entries others use)
+
+struct IctwGeo {
+    int nyb, nsteps;  // row groups per plane, steps of a group (nx + 62)
+};
+__device__ __forceinline__ IctwGeo ictw_geo(const Geo& g) { return {(g.ny + 31) / 32, g.nx + 62}; }
+
+__device__ __forceinline__ double2 ldx(const double* p) {
+    double2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double keep_clear(double x) {  // a value that is never the unset pattern
+    return __double_as_longlong(x) == -1LL ? __longlong_as_double(0x7fffffffffffffffLL) : x;
+}
+__device__ __forceinline__ void stx(double* p, double a, double b) {
+    asm volatile("st.relaxed.gpu.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(keep_clear(a)), "d"(keep_clear(b)) : "memory");
+}
+__device__ __forceinline__ void stx_unset(double* p) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %1};" ::"l"(p), "l"(-1LL) : "memory");
+}
+__device__ __forceinline__ bool is_unset(double2 v) {
+    return __double_as_longlong(v.x) == -1LL || __double_as_longlong(v.y) == -1LL;
+}
+
+// A record's N double2 at p, wanted or 0.  issue() starts the loads, take() waits for the values
+// (bounded), hands the entry back and returns them.
+template <int N>
+struct Pending {
+    double2 v[N];
+    double* p;  // null: nothing wanted
+    __device__ __forceinline__ void issue(double* at, bool want) {
+        p = want ? at : nullptr;
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = want ? ldx(at + 2 * k) : double2{0.0, 0.0};
+    }
+    __device__ __forceinline__ bool missing() const {
+        bool m = false;
+#pragma unroll
+        for (int k = 0; k < N; ++k) m |= is_unset(v[k]);
+        return p && m;
+    }
+    __device__ __forceinline__ void take(const IctArgs& a, bool& ok) {
+        long long n = 0;
+        while (__any_sync(0xffffffffu, missing())) {
+            if (!ok || ++n > a.spin_limit) {
+                ok = false;
+                if (missing()) {
+                    p = nullptr;
+#pragma unroll
+                    for (int k = 0; k < N; ++k) v[k] = double2{0.0, 0.0};
+                }
+                continue;
+            }
+            if (missing()) {
+                __nanosleep(20);
+#pragma unroll
+                for (int k = 0; k < N; ++k) v[k] = ldx(p + 2 * k);
+            }
+        }
+        if (p) {
+#pragma unroll
+            for (int k = 0; k < N; ++k) stx_unset(p + 2 * k);
+        }
+    }
+};
+
+// Steps of a row group that reach a mask voxel (first > last: none).
+struct Span {
+    int lo, hi;
+    __device__ __forceinline__ bool has(int s) const { return s >= lo && s <= hi; }
+};
+__device__ __forceinline__ Span ictw_span(const int4* rows, bool there, int u, bool fwd) {
+    if (!there) return {1 << 30, -(1 << 30)};
+    const int4 r = rows[u];
+    return fwd ? Span{r.x, r.y} : Span{r.z, r.w};
+}
+
+// First and last step of every row group, forward (x + 2 lane) and mirrored (nx - 1 - x + 2 (31 - lane)).
+__global__ void __launch_bounds__(32) k_ictw_rows(Geo geo, const uint8_t* nb, int4* rows) {
+    const IctwGeo w = ictw_geo(geo);
+    const int u = blockIdx.x, z = u / w.nyb, y = (u % w.nyb) * 32 + threadIdx.x, l = threadIdx.x;
+    int lo = 1 << 30, hi = -(1 << 30), lo2 = lo, hi2 = hi;
+    if (y < geo.ny) {
+        const uint8_t* row = nb + ((long long)z * geo.ny + y) * geo.nx;
+        for (int x = 0; x < geo.nx; ++x)
+            if (row[x] & NB_IN) {
+                lo = min(lo, x + 2 * l);
+                hi = x + 2 * l;
+                hi2 = max(hi2, geo.nx - 1 - x + 2 * (31 - l));
+                lo2 = geo.nx - 1 - x + 2 * (31 - l);
+            }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo2 = __reduce_min_sync(0xffffffffu, lo2);
+    hi2 = __reduce_max_sync(0xffffffffu, hi2);
+    if (l == 0) rows[u] = make_int4(lo, hi, lo2, hi2);
+}
+
+// Exchange buffer: plane records [unit][step][lane] of kRec doubles, then edge records
+// [unit][step][2] (0: the first lane's for the group below in the next plane, 1: the last lane's for
+// the next group) of kRec doubles.  The substitution-only walks use the first two doubles.
+__device__ __forceinline__ double* plane_rec(const IctArgs& a, const IctwGeo& w, int u, int s, int lane) {
+    return a.xch + (((long long)u * w.nsteps + s) * 32 + lane) * kRec;
+}
+__device__ __forceinline__ double* edge_rec(const IctArgs& a, const IctwGeo& w, int u, int s, int which) {
+    const long long units = (long long)w.nyb * a.geo.nz;
+    return a.xch + units * w.nsteps * 32 * kRec + (((long long)u * w.nsteps + s) * 2 + which) * kRec;
+}
+
+__device__ __forceinline__ double up1(double v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ double down1(double v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+
+// Factor (FACTOR) or apply, with the forward substitution.
+template <typename T, bool FACTOR>
+__global__ void __launch_bounds__(32) k_ictw_fwd(IctArgs a) {
+    constexpr int C = 2;               // steps whose incoming records are in flight ahead
+    constexpr int N = FACTOR ? 3 : 1;  // double2 of a record that are used
+    const Geo geo = a.geo;
+    const IctwGeo w = ictw_geo(geo);
+    const int nx = geo.nx, ny = geo.ny, lane = threadIdx.x;
+    const long long nv = geo.nv;
+    const int units = w.nyb * geo.nz;
     const T* d = (const T*)a.d;
     const T* g = (const T*)a.g;
     T* ipo = (T*)a.ip_out;
-    const bool factor = d != nullptr;
-    const double beta = a.beta;
-    const double tau = factor ? a.scal[S_ICT_TAU] : 0.0;
-    const int npair = ny * nz;
-    const int tmax = (nx - 1) + 2 * (ny - 1) + 3 * (nz - 1);
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
-    bool bad = false;
-    for (int t = 0; t <= tmax; ++t) {
-        for (int pr = gtid; pr < npair; pr += nthr) {
-            const int y = pr % ny, z = pr / ny, x = t - 2 * y - 3 * z;
-            if (x < 0 || x >= nx) continue;
-            const long long i = x + (long long)nx * y + nxy * z;
-            const uint8_t b = a.nb[i];
-            if (!(b & NB_IN)) continue;
-            const long long ja = i - 1, jb = i - nx, jc = i - nxy, jd = i + 1 - nx, je = i + 1 - nxy, jf = i + nx - nxy;
-            const bool ha = b & NB_XM, hb = b & NB_YM, hc = b & NB_ZM;
-            const bool hd = x + 1 < nx && y > 0 && (a.nb[jd] & NB_IN);
-            const bool he = x + 1 < nx && z > 0 && (a.nb[je] & NB_IN);
-            const bool hf = y + 1 < ny && z > 0 && (a.nb[jf] & NB_IN);
-            auto ld = [&](bool h, int k, long long j) { return h ? ld_level(P(k, j)) : 0.0; };
-            // every value from the earlier rows first (independent loads), then the chain
-            const double yc = ld(hc, PL_Y, jc), ye = ld(he, PL_Y, je), yf = ld(hf, PL_Y, jf),
-                         yb = ld(hb, PL_Y, jb), yd = ld(hd, PL_Y, jd), ya = ld(ha, PL_Y, ja);
-            double la, lb, lc, l_d, le, lf, rii;
-            if (factor) {
-                const double rc = ld(hc, PL_R, jc), re = ld(he, PL_R, je), rf = ld(hf, PL_R, jf),
-                             rb = ld(hb, PL_R, jb), rd = ld(hd, PL_R, jd), ra = ld(ha, PL_R, ja);
-                const double e_a = ld(he, PL_A, je), f_b = ld(hf, PL_B, jf), f_d = ld(hf, PL_D1, jf),
-                             b_f = ld(hb, PL_F, jb), d_a = ld(hd, PL_A, jd), d_f = ld(hd, PL_F, jd),
-                             a_d = ld(ha, PL_D1, ja), a_e = ld(ha, PL_E, ja);
-                auto keep = [&](bool h, double v) { return h && fabs(v) >= tau ? v : 0.0; };
-                lc = keep(hc, -beta * rc);
-                le = keep(he, -(lc * e_a) * re);
-                lf = keep(hf, -(lc * f_b + le * f_d) * rf);
-                lb = keep(hb, (-beta - lc * b_f) * rb);
-                l_d = keep(hd, -(lb * d_a + le * d_f) * rd);
-                la = keep(ha, (-beta - lb * a_d - lc * a_e) * ra);
-                const double h = (double)d[i] + beta * (double)__popc((unsigned)(b >> 1) & 0x3fu);
-                const double s = h - (((la * la + lb * lb) + (lc * lc + l_d * l_d)) + (le * le + lf * lf));
-                if (!(s > 0.0)) bad = true;
-                rii = s > 0.0 ? rsqrt_nr(s) : 1.0;  // the error is reported; keep the arithmetic finite
-                *P(PL_R, i) = rii;
-                *P(PL_A, i) = la;
-                *P(PL_B, i) = lb;
-                *P(PL_C, i) = lc;
-                *P(PL_D1, i) = l_d;
-                *P(PL_E, i) = le;
-                *P(PL_F, i) = lf;
-                if (ipo) ipo[i] = (T)(rii * rii);
-            } else {
-                rii = *P(PL_R, i);
-                la = *P(PL_A, i);
-                lb = *P(PL_B, i);
-                lc = *P(PL_C, i);
-                l_d = *P(PL_D1, i);
-                le = *P(PL_E, i);
-                lf = *P(PL_F, i);
-            }
-            const double acc = (double)g[i] - ((lc * yc + le * ye) + (lf * yf + lb * yb) + (l_d * yd + la * ya));
-            *P(PL_Y, i) = acc * rii;
+    const double beta = a.beta, tau = FACTOR ? a.scal[S_ICT_TAU] : 0.0;
+    double* L = a.L;
+    bool bad = false, ok = true;
+    for (;;) {
+        int u = lane == 0 ? atomicAdd(a.ticket, 1) : 0;
+        u = __shfl_sync(0xffffffffu, u, 0);
+        if (u >= units) break;
+        const int z = u / w.nyb, yb = u % w.nyb, y = yb * 32 + lane;
+        const Span me = ictw_span(a.rows, true, u, true);
+        if (me.lo > me.hi) continue;
+        // whom this group reads, and who reads it
+        const Span rz = ictw_span(a.rows, z > 0, u - w.nyb, true), rf = ictw_span(a.rows, z > 0 && yb + 1 < w.nyb, u - w.nyb + 1, true),
+                   ry = ictw_span(a.rows, yb > 0, u - 1, true);
+        const Span uz = ictw_span(a.rows, z + 1 < geo.nz, u + w.nyb, true), uf = ictw_span(a.rows, z + 1 < geo.nz && yb > 0, u + w.nyb - 1, true),
+                   uy = ictw_span(a.rows, yb + 1 < w.nyb, u + 1, true);
+        const long long row = ((long long)z * ny + y) * nx;
+        const bool row_in = y < ny;
+        // plane record of producer step sp; edge record of this lane (lane 31: f at step s; lane 0: d at s)
+        auto want_z = [&](int sp) { return sp <= me.hi + 2 && rz.has(sp); };
+        auto issue_e = [&](Pending<N>& q, int sp) { q.issue(want_z(sp) ? plane_rec(a, w, u - w.nyb, sp, lane) : nullptr, want_z(sp)); };
+        auto issue_x = [&](Pending<N>& q, int s) {
+            const bool wf = lane == 31 && s <= me.hi && s >= me.lo && rf.has(s - 62), wy = lane == 0 && s <= me.hi && ry.has(s + 63);
+            q.issue(wf ? edge_rec(a, w, u - w.nyb + 1, s - 62, 0) : wy ? edge_rec(a, w, u - 1, s + 63, 1) : nullptr, wf | wy);
+        };
+        double oR = 0, oY = 0, oA = 0, oD = 0, oE = 0, oF = 0;      // this lane's row of the step before
+        double dR = 0, dY = 0, dF = 0;                              // the lower lane's, last step's d: now b
+        double cR, cY, eR, eY, eA;                                  // plane z-1: c, e of this step
+        {
+            Pending<N> p0, p1, x0;
+            issue_e(p0, me.lo);
+            issue_e(p1, me.lo + 1);
+            issue_x(x0, me.lo - 1);
+            p0.take(a, ok);
+            p1.take(a, ok);
+            x0.take(a, ok);
+            cR = p0.v[0].x; cY = p0.v[0].y;
+            eR = p1.v[0].x; eY = p1.v[0].y; eA = N > 1 ? p1.v[N > 1 ? 1 : 0].x : 0.0;
+            if (lane == 0) { dR = x0.v[0].x; dY = x0.v[0].y; dF = N > 2 ? x0.v[N - 1].y : 0.0; }
         }
-        if (t < tmax && !level_sync(a)) return;
+        Pending<N> e[C], xr[C];
+        T gv[C], dv[C];
+        uint8_t nbv[C];
+        double lp[C][FACTOR ? 1 : 7];  // apply: the stored row
+        auto issue_own = [&](int s0) {
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                const int x = s0 + q - 2 * lane;
+                const bool in = row_in && (unsigned)x < (unsigned)nx;
+                const long long i = row + x;
+                nbv[q] = in ? a.nb[i] : (uint8_t)0;
+                gv[q] = in ? g[i] : T(0);
+                dv[q] = FACTOR && in ? d[i] : T(0);
+                if (!FACTOR)
+#pragma unroll
+                    for (int k = 0; k < (FACTOR ? 1 : 7); ++k) lp[q][k] = in ? L[(size_t)k * nv + i] : 0.0;
+            }
+        };
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+            issue_e(e[q], me.lo + q + 2);
+            issue_x(xr[q], me.lo + q);
+        }
+        issue_own(me.lo);
+        for (int s0 = me.lo; s0 <= me.hi; s0 += C) {
+            // this chunk's incoming records and inputs; the next chunk's loads start
+            double nR[C], nY[C], nA[C], nB[C], nD[C], xR[C], xY[C], xA[C], xB[C], xD[C], xF[C];
+            T gg[C], dd[C];
+            uint8_t bb[C];
+            double ll[C][FACTOR ? 1 : 7];
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                e[q].take(a, ok);
+                xr[q].take(a, ok);
+                nR[q] = e[q].v[0].x; nY[q] = e[q].v[0].y;
+                xR[q] = xr[q].v[0].x; xY[q] = xr[q].v[0].y;
+                if constexpr (FACTOR) {
+                    nA[q] = e[q].v[1].x; nB[q] = e[q].v[1].y; nD[q] = e[q].v[2].x;
+                    xA[q] = xr[q].v[1].x; xB[q] = xr[q].v[1].y; xD[q] = xr[q].v[2].x; xF[q] = xr[q].v[2].y;
+                }
+                gg[q] = gv[q]; dd[q] = dv[q]; bb[q] = nbv[q];
+#pragma unroll
+                for (int k = 0; k < (FACTOR ? 1 : 7); ++k) ll[q][k] = lp[q][k];
+            }
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                issue_e(e[q], s0 + C + q + 2);
+                issue_x(xr[q], s0 + C + q);
+            }
+            issue_own(s0 + C);
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                const int s = s0 + q, x = s - 2 * lane;
+                const long long i = row + x;
+                const bool in = bb[q] & NB_IN;
+                // roles: a own, d / b the lower lane's of one and two steps ago, c, e, f plane z-1
+                const double aR = oR, aY = oY, bR = dR, bY = dY;
+                double uR = up1(oR), uY = up1(oY), fR = down1(nR[q]), fY = down1(nY[q]);
+                dR = lane == 0 ? xR[q] : uR;
+                dY = lane == 0 ? xY[q] : uY;
+                if (lane == 31) { fR = xR[q]; fY = xY[q]; }
+                double la, lb, lc, l_d, le, lf, rii;
+                if constexpr (FACTOR) {
+                    const double a_d = oD, a_e = oE, b_f = dF, e_a = eA;
+                    const double uA = up1(oA), uF = up1(oF);
+                    double f_b = down1(nB[q]), f_d = down1(nD[q]);
+                    const double d_a = lane == 0 ? xA[q] : uA;
+                    dF = lane == 0 ? xF[q] : uF;
+                    const double d_f = dF;
+                    if (lane == 31) { f_b = xB[q]; f_d = xD[q]; }
+                    auto kp = [&](double v) { return fabs(v) >= tau ? v : 0.0; };
+                    lc = cR != 0.0 ? kp(-beta * cR) : 0.0;
+                    le = kp(-(lc * e_a) * eR);
+                    lf = kp(-(lc * f_b + le * f_d) * fR);
+                    lb = bR != 0.0 ? kp((-beta - lc * b_f) * bR) : 0.0;
+                    l_d = kp(-(lb * d_a + le * d_f) * dR);
+                    la = aR != 0.0 ? kp((-beta - lb * a_d - lc * a_e) * aR) : 0.0;
+                    const double h = (double)dd[q] + beta * (double)__popc((unsigned)(bb[q] >> 1) & 0x3fu);
+                    const double sq = h - (((la * la + lb * lb) + (lc * lc + l_d * l_d)) + (le * le + lf * lf));
+                    if (in && !(sq > 0.0)) bad = true;
+                    rii = sq > 0.0 ? rsqrt_nr(sq) : 1.0;  // the error is reported; keep the arithmetic finite
+                } else {
+                    rii = ll[q][PL_R];
+                    la = ll[q][FACTOR ? 0 : PL_A];
+                    lb = ll[q][FACTOR ? 0 : PL_B];
+                    lc = ll[q][FACTOR ? 0 : PL_C];
+                    l_d = ll[q][FACTOR ? 0 : PL_D1];
+                    le = ll[q][FACTOR ? 0 : PL_E];
+                    lf = ll[q][FACTOR ? 0 : PL_F];
+                }
+                const double acc = (double)gg[q] - ((lc * cY + le * eY) + (lf * fY + lb * bY) + (l_d * dY + la * aY));
+                // a row outside the mask reads as 0 everywhere
+                oR = in ? rii : 0.0;
+                oY = in ? acc * rii : 0.0;
+                if constexpr (FACTOR) {
+                    oA = in ? la : 0.0;
+                    oD = in ? l_d : 0.0;
+                    oE = in ? le : 0.0;
+                    oF = in ? lf : 0.0;
+                    lb = in ? lb : 0.0;
+                }
+                if (in) {
+                    if (FACTOR) {
+                        L[(size_t)PL_R * nv + i] = rii;
+                        L[(size_t)PL_A * nv + i] = la;
+                        L[(size_t)PL_B * nv + i] = lb;
+                        L[(size_t)PL_C * nv + i] = lc;
+                        L[(size_t)PL_D1 * nv + i] = l_d;
+                        L[(size_t)PL_E * nv + i] = le;
+                        L[(size_t)PL_F * nv + i] = lf;
+                        if (ipo) ipo[i] = (T)(rii * rii);
+                    }
+                    L[(size_t)PL_Y * nv + i] = oY;
+                }
+                // hand over what is read: consumer steps s - 2 .. (plane), s + 62 and s - 63 (edges)
+                if (s <= me.hi) {
+                    if (s >= uz.lo && s <= uz.hi + 2) {
+                        double* r = plane_rec(a, w, u, s, lane);
+                        stx(r, oR, oY);
+                        if constexpr (FACTOR) {
+                            stx(r + 2, oA, lb);
+                            stx(r + 4, oD, oF);
+                        }
+                    }
+                    const bool gf = lane == 0 && uf.has(s + 62), gy = lane == 31 && s - 63 >= uy.lo - 1 && s - 63 <= uy.hi;
+                    if (gf | gy) {
+                        double* r = edge_rec(a, w, u, s, gf ? 0 : 1);
+                        stx(r, oR, oY);
+                        if constexpr (FACTOR) {
+                            stx(r + 2, oA, lb);
+                            stx(r + 4, oD, oF);
+                        }
+                    }
+                }
+                cR = eR; cY = eY;
+                eR = nR[q]; eY = nY[q];
+                if constexpr (FACTOR) eA = nA[q];
+            }
+        }
     }
-    // reported by the back sweep, after k_ict_check: fill beyond the held pattern (which can
-    // itself make a pivot of the restricted factor non-positive) takes precedence
     if (bad) atomicExch(a.istate + I_ICT_BAD, 1);
+    if (!ok) set_err(a.istate, FM_ERR_TIMEOUT);
 }
 
+// The mirrored walk: lane l holds row y = 32 yb + 31 - l and walks x = nx - 1 - (s - 2 l), solving
+// L' x = y with the entries of the later rows a = (x+1, y), b = (x, y+1), d = (x-1, y+1) of this plane and
+// c, e, f of plane z+1; then p and its dot products, summed per row group and added in order.
 template <typename T>
-__global__ void __launch_bounds__(kIctThreads) k_ict_bwd(IctArgs a) {
-    __shared__ double sbuf[2 * 32];
-    const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
-    const long long nxy = (long long)nx * ny, nv = a.geo.nv;
-    double* Lp = a.L;
-    auto P = [&](int k, long long j) -> double* { return Lp + (size_t)k * nv + j; };
+__global__ void __launch_bounds__(32) k_ictw_bwd(IctArgs a) {
+    constexpr int C = 2;
+    const Geo geo = a.geo;
+    const IctwGeo w = ictw_geo(geo);
+    const int nx = geo.nx, ny = geo.ny, lane = threadIdx.x;
+    const long long nv = geo.nv, nxy = (long long)nx * ny;
+    const int units = w.nyb * geo.nz;
+    const double* L = a.L;
     T* p = (T*)a.p;
     const T* gd = (const T*)a.gdot;
     const T* gpd = (const T*)a.gpdot;
-    const int npair = ny * nz;
-    const int tmax = (nx - 1) + 2 * (ny - 1) + 3 * (nz - 1);
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
-    double acc2[2] = {0.0, 0.0};
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.istate[I_ICT_BAD]) {
+    bool ok = true;
+    if (blockIdx.x == 0 && lane == 0 && a.istate[I_ICT_BAD]) {
         set_err(a.istate, FM_ERR_NOT_PD);
         a.istate[I_ICT_BAD] = 0;
     }
-    for (int t = tmax; t >= 0; --t) {
-        for (int pr = gtid; pr < npair; pr += nthr) {
-            const int y = pr % ny, z = pr / ny, x = t - 2 * y - 3 * z;
-            if (x < 0 || x >= nx) continue;
-            const long long i = x + (long long)nx * y + nxy * z;
-            const uint8_t b = a.nb[i];
-            if (!(b & NB_IN)) {
-                p[i] = T(0);
-                continue;
+    for (;;) {
+        int u = lane == 0 ? atomicAdd(a.ticket, 1) : 0;
+        u = units - 1 - __shfl_sync(0xffffffffu, u, 0);
+        if (u < 0) break;
+        const int z = u / w.nyb, yb = u % w.nyb, y = yb * 32 + 31 - lane;
+        const Span me = ictw_span(a.rows, true, u, false);
+        double acc0 = 0.0, acc1 = 0.0;
+        if (me.lo <= me.hi) {
+            const bool zp = z + 1 < geo.nz, zm = z > 0;
+            const Span rz = ictw_span(a.rows, zp, u + w.nyb, false), rf = ictw_span(a.rows, zp && yb > 0, u + w.nyb - 1, false),
+                       ry = ictw_span(a.rows, yb + 1 < w.nyb, u + 1, false);
+            const Span uz = ictw_span(a.rows, zm, u - w.nyb, false), uf = ictw_span(a.rows, zm && yb + 1 < w.nyb, u - w.nyb + 1, false),
+                       uy = ictw_span(a.rows, yb > 0, u - 1, false);
+            const long long row = ((long long)z * ny + y) * nx;
+            const bool row_in = y < ny;
+            auto want_z = [&](int sp) { return sp <= me.hi + 2 && rz.has(sp); };
+            auto issue_e = [&](Pending<1>& q, int sp) { q.issue(want_z(sp) ? plane_rec(a, w, u + w.nyb, sp, lane) : nullptr, want_z(sp)); };
+            auto issue_x = [&](Pending<1>& q, int s) {
+                const bool wf = lane == 31 && s <= me.hi && s >= me.lo && rf.has(s - 62), wy = lane == 0 && s <= me.hi && ry.has(s + 63);
+                q.issue(wf ? edge_rec(a, w, u + w.nyb - 1, s - 62, 0) : wy ? edge_rec(a, w, u + 1, s + 63, 1) : nullptr, wf | wy);
+            };
+            double o = 0.0, dv = 0.0, cv, ev;
+            {
+                Pending<1> p0, p1, x0;
+                issue_e(p0, me.lo);
+                issue_e(p1, me.lo + 1);
+                issue_x(x0, me.lo - 1);
+                p0.take(a, ok);
+                p1.take(a, ok);
+                x0.take(a, ok);
+                cv = p0.v[0].x;
+                ev = p1.v[0].x;
+                if (lane == 0) dv = x0.v[0].x;
             }
-            // the later rows r = i - o that hold an entry in column i: L_{r,i} = plane o of row r
-            const long long ra = i + 1, rb = i + nx, rc = i + nxy, rd = i - 1 + nx, re = i - 1 + nxy, rf = i - nx + nxy;
-            const bool ha = b & NB_XP, hb = b & NB_YP, hc = b & NB_ZP;
-            const bool hd = x > 0 && y + 1 < ny && (a.nb[rd] & NB_IN);
-            const bool he = x > 0 && z + 1 < nz && (a.nb[re] & NB_IN);
-            const bool hf = y > 0 && z + 1 < nz && (a.nb[rf] & NB_IN);
-            auto ld = [&](bool h, int k, long long j) { return h ? ld_level(P(k, j)) : 0.0; };
-            const double s = *P(PL_Y, i) - ((ld(ha, PL_A, ra) * ld(ha, PL_Y, ra) + ld(hd, PL_D1, rd) * ld(hd, PL_Y, rd)) +
-                                            (ld(hf, PL_F, rf) * ld(hf, PL_Y, rf) + ld(hb, PL_B, rb) * ld(hb, PL_Y, rb)) +
-                                            (ld(he, PL_E, re) * ld(he, PL_Y, re) + ld(hc, PL_C, rc) * ld(hc, PL_Y, rc)));
-            const double xi = s * *P(PL_R, i);
-            *P(PL_Y, i) = xi;  // y_i becomes x_i: every row that still needs y_i is this one
-            p[i] = (T)xi;
-            if (gd) acc2[0] += (double)gd[i] * (double)(T)xi;
-            if (gpd) acc2[1] += (double)gpd[i] * (double)(T)xi;
+            Pending<1> e[C], xr[C];
+            // the entries that multiply the neighbours' values, this row's y and 1/L_ii, g and g_prev
+            double lp[C][8];
+            T gv[C], gpv[C];
+            bool inq[C];
+            auto issue_own = [&](int s0) {
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int x = nx - 1 - (s0 + q - 2 * lane);
+                    const bool in = row_in && (unsigned)x < (unsigned)nx;
+                    const long long i = row + x;
+                    const bool ym = y > 0, yp = y + 1 < ny, xm = x > 0, xp = x + 1 < nx;
+                    auto ld = [&](bool h, int pl, long long j) { return in && h ? L[(size_t)pl * nv + j] : 0.0; };
+                    inq[q] = in && (a.nb[i] & NB_IN);
+                    lp[q][0] = ld(xp, PL_A, i + 1);
+                    lp[q][1] = ld(yp, PL_B, i + nx);
+                    lp[q][2] = ld(zp, PL_C, i + nxy);
+                    lp[q][3] = ld(yp && xm, PL_D1, i + nx - 1);
+                    lp[q][4] = ld(zp && xm, PL_E, i + nxy - 1);
+                    lp[q][5] = ld(zp && ym, PL_F, i + nxy - nx);
+                    lp[q][6] = ld(true, PL_Y, i);
+                    lp[q][7] = ld(true, PL_R, i);
+                    gv[q] = gd && in ? gd[i] : T(0);
+                    gpv[q] = gpd && in ? gpd[i] : T(0);
+                }
+            };
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+                issue_e(e[q], me.lo + q + 2);
+                issue_x(xr[q], me.lo + q);
+            }
+            issue_own(me.lo);
+            for (int s0 = me.lo; s0 <= me.hi; s0 += C) {
+                double nv_[C], xv[C], ll[C][8];
+                T gg[C], gp[C];
+                bool in_[C];
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    e[q].take(a, ok);
+                    xr[q].take(a, ok);
+                    nv_[q] = e[q].v[0].x;
+                    xv[q] = xr[q].v[0].x;
+                    gg[q] = gv[q];
+                    gp[q] = gpv[q];
+                    in_[q] = inq[q];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) ll[q][k] = lp[q][k];
+                }
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    issue_e(e[q], s0 + C + q + 2);
+                    issue_x(xr[q], s0 + C + q);
+                }
+                issue_own(s0 + C);
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int s = s0 + q;
+                    const double av = o, bv = dv, uv = up1(o), fdn = down1(nv_[q]);
+                    dv = lane == 0 ? xv[q] : uv;
+                    const double fv = lane == 31 ? xv[q] : fdn;
+                    const double t = ll[q][6] - ((ll[q][0] * av + ll[q][3] * dv) + (ll[q][5] * fv + ll[q][1] * bv) +
+                                                 (ll[q][4] * ev + ll[q][2] * cv));
+                    const double xi = t * ll[q][7];
+                    o = in_[q] ? xi : 0.0;
+                    if (in_[q]) {
+                        p[row + nx - 1 - (s - 2 * lane)] = (T)xi;
+                        acc0 += (double)gg[q] * (double)(T)xi;
+                        acc1 += (double)gp[q] * (double)(T)xi;
+                    }
+                    if (s <= me.hi) {
+                        if (s >= uz.lo && s <= uz.hi + 2) stx(plane_rec(a, w, u, s, lane), o, 0.0);
+                        const bool gf = lane == 0 && uf.has(s + 62), gy = lane == 31 && s - 63 >= uy.lo - 1 && s - 63 <= uy.hi;
+                        if (gf | gy) stx(edge_rec(a, w, u, s, gf ? 0 : 1), o, 0.0);
+                    }
+                    cv = ev;
+                    ev = nv_[q];
+                }
+            }
         }
-        if (t > 0 && !level_sync(a)) return;
-    }
-    if (gd || gpd) {
-        double out[2];
-        if (last_block_reduce<2>(acc2, a.partials, (unsigned*)(a.istate + I_DONE0), out, sbuf)) {
-            if (threadIdx.x == 0) {
-                a.scal[S_GP] = out[0];
-                a.scal[S_GPREVP] = out[1];
-                if (!isfinite(out[0]) || !isfinite(out[1])) set_err(a.istate, FM_ERR_NONFINITE);
+        if (gd || gpd) {
+            acc0 = warp_sum(acc0);
+            acc1 = warp_sum(acc1);
+            int last = 0;
+            if (lane == 0) {
+                a.part[u] = acc0;
+                a.part[units + u] = acc1;
+                __threadfence();
+                last = atomicAdd(a.done, 1) == units - 1;
+                if (last) __threadfence();
+            }
+            if (__shfl_sync(0xffffffffu, last, 0)) {
+                double t0 = 0.0, t1 = 0.0;
+                for (int k = lane; k < units; k += 32) {
+                    t0 += __ldcg(a.part + k);
+                    t1 += __ldcg(a.part + units + k);
+                }
+                t0 = warp_sum(t0);
+                t1 = warp_sum(t1);
+                if (lane == 0) {
+                    a.scal[S_GP] = t0;
+                    a.scal[S_GPREVP] = t1;
+                    if (!isfinite(t0) || !isfinite(t1)) set_err(a.istate, FM_ERR_NONFINITE);
+                }
             }
         }
     }
+    if (!ok) set_err(a.istate, FM_ERR_TIMEOUT);
 }
 
 // ------------------------------------------------------------------ table-driven sweeps
@@ -285,8 +643,8 @@ __device__ __forceinline__ long long ict_nbr(const IctArgs& a, int x, int y, int
     return (a.nb[j] & NB_IN) ? j : -1;
 }
 
-// The same factorisation and substitutions as k_ict_fwd / k_ict_bwd for any held pattern
-// (a.tb): row i's entries in increasing column order, L_{i,j} = (H_ij - sum over the pairs
+// The factorisation and substitutions for any held pattern (a.tb) -- grown ones, and the base
+// pattern of volumes whose rows make the wavefront's exchange buffer too large (fm_create): row i's entries in increasing column order, L_{i,j} = (H_ij - sum over the pairs
 // (p1, p2) of o of L_{i,i+o_p1} L_{j,j+o_p2}) / L_jj, dropped below tau, then L_ii and y_i.
 // Level t = x + B y + C z, with B and C chosen by the host so that every held offset points
 // to a strictly lower level.
@@ -467,33 +825,32 @@ int ictg_max_blocks_per_sm(int block) {
 }
 
 template <typename T>
-int ict_max_blocks_per_sm(int block) {
-    int f = 0, b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f, k_ict_fwd<T>, block, 0) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ict_bwd<T>, block, 0) != cudaSuccess) return 0;
-    return f < b ? f : b;
-}
-
-template <typename T>
 cudaError_t launch_ict_tau(const DataArgs& a, double droptol, int grid, cudaStream_t s) {
     k_ict_tau<T><<<grid, kThreads, 0, s>>>(a, droptol);
     return cudaGetLastError();
 }
+template <typename T>
+cudaError_t launch_ictw_fwd(const IctArgs& a, int grid, cudaStream_t s) {
+    if (a.d) k_ictw_fwd<T, true><<<grid, 32, 0, s>>>(a);
+    else k_ictw_fwd<T, false><<<grid, 32, 0, s>>>(a);
+    return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_ictw_bwd(const IctArgs& a, int grid, cudaStream_t s) {
+    k_ictw_bwd<T><<<grid, 32, 0, s>>>(a);
+    return cudaGetLastError();
+}
+cudaError_t launch_ictw_rows(const Geo& geo, const uint8_t* nb, int4* rows, cudaStream_t s) {
+    k_ictw_rows<<<ictw_units(geo), 32, 0, s>>>(geo, nb, rows);
+    return cudaGetLastError();
+}
+int ictw_units(const Geo& geo) { return (geo.ny + 31) / 32 * geo.nz; }
+size_t ictw_exchange_bytes(const Geo& geo) {
+    return (size_t)ictw_units(geo) * (geo.nx + 62) * (32 + 2) * kRec * sizeof(double);
+}
 // The level sweeps wait at a grid barrier, so every block must be resident at once.  A
 // cooperative launch guarantees that (or refuses the launch) even when other kernels run
 // beside the sweep, e.g. the other volumes' branches of a batched graph.
-template <typename T>
-cudaError_t launch_ict_fwd(const IctArgs& a, int grid, int block, cudaStream_t s) {
-    IctArgs copy = a;
-    void* args[] = {&copy};
-    return cudaLaunchCooperativeKernel((const void*)k_ict_fwd<T>, dim3(grid), dim3(block), args, 0, s);
-}
-template <typename T>
-cudaError_t launch_ict_bwd(const IctArgs& a, int grid, int block, cudaStream_t s) {
-    IctArgs copy = a;
-    void* args[] = {&copy};
-    return cudaLaunchCooperativeKernel((const void*)k_ict_bwd<T>, dim3(grid), dim3(block), args, 0, s);
-}
 template <typename T>
 cudaError_t launch_ictg_fwd(const IctArgs& a, int grid, int block, cudaStream_t s) {
     IctArgs copy = a;
@@ -514,12 +871,11 @@ cudaError_t launch_ict_check(const IctArgs& a, int grid, cudaStream_t s) {
 
 #define FM_ICT_INST(T)                                                                   \
     template cudaError_t launch_ict_tau<T>(const DataArgs&, double, int, cudaStream_t); \
-    template cudaError_t launch_ict_fwd<T>(const IctArgs&, int, int, cudaStream_t);     \
-    template cudaError_t launch_ict_bwd<T>(const IctArgs&, int, int, cudaStream_t);     \
+    template cudaError_t launch_ictw_fwd<T>(const IctArgs&, int, cudaStream_t);         \
+    template cudaError_t launch_ictw_bwd<T>(const IctArgs&, int, cudaStream_t);         \
     template cudaError_t launch_ict_check<T>(const IctArgs&, int, cudaStream_t);        \
     template cudaError_t launch_ictg_fwd<T>(const IctArgs&, int, int, cudaStream_t);    \
     template cudaError_t launch_ictg_bwd<T>(const IctArgs&, int, int, cudaStream_t);    \
-    template int ict_max_blocks_per_sm<T>(int);                                         \
     template int ictg_max_blocks_per_sm<T>(int);
 FM_ICT_INST(float)
 FM_ICT_INST(double)
