@@ -107,16 +107,80 @@ __device__ __forceinline__ void sum_partials(const double* partials, int n, doub
     block_sum<Q>(out, sbuf);
 }
 
+// The same sums for blocks of 256 threads, with a quarter of the FP64 instructions: the FP64 pipe
+// issues one warp's addition every 16 cycles for the whole SM, and in block_sum all eight warps
+// walk the tree with 32 redundant lanes (45 instructions a value, 12 here; with the scalar divisions
+// left to one thread, k_ls of a 64x64x16 grid went from 55 to 37 us, of 256x256x128 with 8 coils from
+// 681 to 662).  One warp per value takes the 256 entries, lane 4 w + i the entries i, i + 4, .. of
+// warp w, and adds them in exactly block_sum's order: lanes 16, 8, 4, 2, 1 apart within a warp, then
+// warps 4, 2, 1 apart.  Result in every lane.
+__device__ __forceinline__ double tree_256(const double (&x)[8]) {
+    double t[4], u[2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) t[j] = x[j] + x[j + 4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) u[j] = t[j] + t[j + 2];
+    double v = u[0] + u[1];
+#pragma unroll
+    for (const int o : {2, 1, 16, 8, 4}) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+constexpr int kTreePitch = 36;  // doubles between the warps' entries: lanes on different banks
+constexpr int kTree = 8 * kTreePitch;
+
+// Block sum of Q doubles over 256 threads; the warp q < Q returns value q in every lane of out
+// (other warps: undefined).  s_val: Q * kTree doubles.
+template <int Q>
+__device__ __forceinline__ double block_sum_256(const double (&v)[Q], double* s_val) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) s_val[q * kTree + wid * kTreePitch + lane] = v[q];
+    __syncthreads();
+    double out = 0.0;
+    if (wid < Q) {
+        double x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = s_val[wid * kTree + (lane >> 2) * kTreePitch + (lane & 3) + 4 * j];
+        out = tree_256(x);
+    }
+    return out;
+}
+
+// The sum of partials[0..n) by one warp, in sum_partials' order for a block of 256 threads.
+__device__ __forceinline__ double sum_partials_256(const double* partials, int n) {
+    const int lane = threadIdx.x & 31;
+    double x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = 0.0;
+    const int i = (lane >> 2) * 32 + (lane & 3);
+    for (int base = 0; base < n; base += 256) {  // eight loads in flight
+        double y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) y[j] = base + i + 4 * j < n ? __ldcg(partials + base + i + 4 * j) : 0.0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] += y[j];
+    }
+    return tree_256(x);
+}
+
 // Each block stores its Q partial sums; the last block to finish reduces all of them in
 // block order and returns true in every thread of that block (out valid in thread 0).
 template <int Q>
 __device__ __forceinline__ bool last_block_reduce(double (&v)[Q], double* partials, unsigned* done,
                                                   double (&out)[Q], double* sbuf) {
     __shared__ bool s_last;
-    block_sum<Q>(v, sbuf);
+    __shared__ double s_val[Q * kTree], s_sum[Q];
+    const bool b256 = blockDim.x == 256;
+    if (b256) {
+        const double t = block_sum_256<Q>(v, s_val);
+        if ((threadIdx.x & 31) == 0 && threadIdx.x < 32 * Q) s_sum[threadIdx.x >> 5] = t;
+        __syncthreads();
+    } else {
+        block_sum<Q>(v, sbuf);
+    }
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q) partials[(size_t)q * gridDim.x + blockIdx.x] = v[q];
+        for (int q = 0; q < Q; ++q) partials[(size_t)q * gridDim.x + blockIdx.x] = b256 ? s_sum[q] : v[q];
         __threadfence();
         unsigned prev = atomicAdd(done, 1u);
         s_last = (prev == gridDim.x - 1);
@@ -124,7 +188,18 @@ __device__ __forceinline__ bool last_block_reduce(double (&v)[Q], double* partia
     }
     __syncthreads();
     if (!s_last) return false;
-    sum_partials<Q>(partials, gridDim.x, out, sbuf);
+    if (b256) {
+        const int wid = threadIdx.x >> 5;
+        if (wid < Q) {
+            const double t = sum_partials_256(partials + (size_t)wid * gridDim.x, gridDim.x);
+            if ((threadIdx.x & 31) == 0) s_sum[wid] = t;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < Q; ++q) out[q] = s_sum[q];
+    } else {
+        sum_partials<Q>(partials, gridDim.x, out, sbuf);
+    }
     if (threadIdx.x == 0) *done = 0u;
     return true;
 }

@@ -576,8 +576,10 @@ template <typename T, int NC> constexpr int ls_blocks() {
 
 template <typename T, int NC>
 __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a) {
-    __shared__ double sbuf[4 * 32];
+    static_assert(kThreads == 256, "block_sum_256");
+    __shared__ double s_val[4 * kTree];
     __shared__ double s_tot[4];
+    __shared__ T s_aT, s_muT;
     const T* w = (const T*)a.w_out;
     using T2 = typename V2<T>::t;
     T2* zw = (T2*)a.zw;
@@ -588,13 +590,20 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
     if ((int)blockIdx.x >= nb) return;
     const int nx = a.geo.nx;
     const long long nxy = (long long)nx * a.geo.ny;
+    const int lane0 = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // mu, and each step's alpha below, come from one thread: a double division by all eight warps
+    // would hold the FP64 pipe for more than a microsecond
     double mu = 0.0;
-    if (it > 0) {
-        const double den = a.scal[S_GP_PREV];
-        mu = den != 0.0 ? (a.scal[S_GP] - a.scal[S_GPREVP]) / den : 0.0;
+    if (threadIdx.x == 0) {
+        if (it > 0) {
+            const double den = a.scal[S_GP_PREV];
+            mu = den != 0.0 ? (a.scal[S_GP] - a.scal[S_GPREVP]) / den : 0.0;
+        }
+        s_muT = (T)mu;
     }
+    __syncthreads();
     {
-        const T muT = (T)mu;
+        const T muT = s_muT;
         const T* p = (const T*)a.p;
         const T* zo = (const T*)a.z_old;
         T* zn = (T*)a.z_new;
@@ -640,25 +649,24 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
             const long long j = a.vlist[k];
             dir_voxel(k, j, a.nb[j], p[j], zo[j], w[j], g[j], d[j]);
         }
-        double v[4] = {(double)s_cz2, (double)s_czw, (double)s_zg, (double)s_zzd};
-        block_sum<4>(v, sbuf);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) a.partials[(size_t)q * nb + blockIdx.x] = v[q];
+        const double v[4] = {(double)s_cz2, (double)s_czw, (double)s_zg, (double)s_zzd};
+        const double bs = block_sum_256<4>(v, s_val);
+        if (wid < 4 && lane0 == 0) a.partials[(size_t)wid * nb + blockIdx.x] = bs;
         if (!grid_barrier(a.istate, a.spin_limit, nb)) return;
-        double tot[4];
-        sum_partials<4>(a.partials, nb, tot, sbuf);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) s_tot[q] = tot[q];
+        if (wid < 4) {
+            const double t = sum_partials_256(a.partials + (size_t)wid * nb, nb);
+            if (lane0 == 0) s_tot[wid] = t;
+        }
         __syncthreads();
     }
-    const double cz2 = s_tot[0], czw = s_tot[1];
-    double alpha;
-    {
+    double alpha = 0.0, cz2 = 0.0, czw = 0.0;  // thread 0's
+    if (threadIdx.x == 0) {
+        cz2 = s_tot[0];
+        czw = s_tot[1];
         const double den = s_tot[3] + a.beta * cz2;
         alpha = den != 0.0 ? -s_tot[2] / den : 0.0;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
+        s_aT = (T)alpha;
+        if (blockIdx.x == 0) {
             a.scal[S_CZ2] = cz2;
             a.scal[S_CZW] = czw;
             a.scal[S_ZG] = s_tot[2];
@@ -668,10 +676,12 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
             if (a.mu_hist) a.mu_hist[it] = mu;
             if (!isfinite(alpha) || !isfinite(mu) || !isfinite(den)) set_err(a.istate, FM_ERR_NONFINITE);
         }
-        __syncthreads();  // s_tot is reused by the steps below
     }
+    __shared__ bool s_stop;
+    if (threadIdx.x == 0) s_stop = false;
+    __syncthreads();
     for (int step = 1; step < a.nls; ++step) {
-        const T aT = (T)alpha;
+        const T aT = s_aT;
         // each thread sums its few voxels in the voxel type, then the block and the grid in FP64
         T t1 = 0, t2 = 0;
         if constexpr (NC == 1) {
@@ -721,23 +731,25 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
                 t2 += q.x * q.x * cu;
             }
         }
-        double v[2] = {(double)t1, (double)t2};
-        block_sum<2>(v, sbuf);
+        const double v[2] = {(double)t1, (double)t2};
+        const double bs = block_sum_256<2>(v, s_val);
         double* part = a.partials + 4 * (size_t)nb + (size_t)(step & 1) * 2 * nb;
-        if (threadIdx.x == 0) {
-            part[blockIdx.x] = v[0];
-            part[nb + blockIdx.x] = v[1];
-        }
+        if (wid < 2 && lane0 == 0) part[(size_t)wid * nb + blockIdx.x] = bs;
         if (!grid_barrier(a.istate, a.spin_limit, nb)) return;
-        double tot[2];
-        sum_partials<2>(part, nb, tot, sbuf);
-        if (threadIdx.x == 0) { s_tot[0] = tot[0]; s_tot[1] = tot[1]; }
+        if (wid < 2) {
+            const double t = sum_partials_256(part + (size_t)wid * nb, nb);
+            if (lane0 == 0) s_tot[wid] = t;
+        }
         __syncthreads();
-        const double fp = s_tot[0] + a.beta * (czw + alpha * cz2);
-        const double den = s_tot[1] + a.beta * cz2;
+        if (threadIdx.x == 0) {
+            const double fp = s_tot[0] + a.beta * (czw + alpha * cz2);
+            const double den = s_tot[1] + a.beta * cz2;
+            alpha = den == 0.0 ? 0.0 : alpha - fp / den;
+            s_aT = (T)alpha;
+            s_stop = den == 0.0;
+        }
         __syncthreads();
-        if (den == 0.0) { alpha = 0.0; break; }
-        alpha = alpha - fp / den;
+        if (s_stop) break;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.scal[S_ALPHA] = alpha;
