@@ -150,7 +150,7 @@ void free_all(fm_ctx* c) {
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
 }
 
-// The grid barrier's arrival count.  A block that gives up in grid_barrier (FM_ERR_TIMEOUT)
+// The grid barriers' arrival counts.  A block that gives up in grid_barrier (FM_ERR_TIMEOUT)
 // leaves its arrival counted; if the count survived into the next launch sequence, a later
 // barrier would open before every block had arrived.  So every launch sequence starts from
 // a zero count (stream-ordered after the launch that timed out has finished), and an error
@@ -158,7 +158,7 @@ void free_all(fm_ctx* c) {
 // when it is read: an error of an earlier asynchronous call is reported by the next call
 // that synchronises.
 cudaError_t reset_barrier(fm_ctx* c) {
-    return cudaMemsetAsync(c->istate + I_BAR_COUNT, 0, sizeof(int), c->stream);
+    return cudaMemsetAsync(c->istate + I_BAR_COUNT, 0, 4 * sizeof(int), c->stream);
 }
 // After a device error the IC forward sweep's face entries may hold values that no reader
 // consumed (a fetch that gave up), so they are set back to the unset pattern too.

@@ -580,6 +580,8 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
     __shared__ double s_val[4 * kTree];
     __shared__ double s_tot[4];
     __shared__ T s_aT, s_muT;
+    __shared__ double s_mu, s_alpha, s_cz2, s_czw;  // thread 0's, kept out of the other threads' registers
+    __shared__ int s_bar;                           // number of the next grid barrier
     const T* w = (const T*)a.w_out;
     using T2 = typename V2<T>::t;
     T2* zw = (T2*)a.zw;
@@ -593,12 +595,14 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
     const int lane0 = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // mu, and each step's alpha below, come from one thread: a double division by all eight warps
     // would hold the FP64 pipe for more than a microsecond
-    double mu = 0.0;
     if (threadIdx.x == 0) {
+        double mu = 0.0;
+        s_bar = a.istate[I_LS_PH];
         if (it > 0) {
             const double den = a.scal[S_GP_PREV];
             mu = den != 0.0 ? (a.scal[S_GP] - a.scal[S_GPREVP]) / den : 0.0;
         }
+        s_mu = mu;
         s_muT = (T)mu;
     }
     __syncthreads();
@@ -610,17 +614,17 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
         const T* g = (const T*)a.g;
         const T* d = (const T*)a.d;
         auto zval = [&](long long k) -> T { return -p[k] + muT * zo[k]; };
-        T s_cz2 = 0, s_czw = 0, s_zg = 0, s_zzd = 0;
+        T t_cz2 = 0, t_czw = 0, t_zg = 0, t_zzd = 0;
         // one voxel's direction entry and its terms of the four sums (the +x, +y, +z edges)
         auto dir_voxel = [&](long long k, long long j, uint8_t b, T pj, T zoj, T wj, T gj, T dj) {
             const T zj = -pj + muT * zoj;
             zn[j] = zj;
             zw[k] = T2{zj, wj};
-            if (b & NB_XP) { const T e = zj - zval(j + 1), f = wj - w[j + 1]; s_cz2 += e * e; s_czw += e * f; }
-            if (b & NB_YP) { const T e = zj - zval(j + nx), f = wj - w[j + nx]; s_cz2 += e * e; s_czw += e * f; }
-            if (b & NB_ZP) { const T e = zj - zval(j + nxy), f = wj - w[j + nxy]; s_cz2 += e * e; s_czw += e * f; }
-            s_zg += zj * gj;
-            s_zzd += zj * zj * dj;
+            if (b & NB_XP) { const T e = zj - zval(j + 1), f = wj - w[j + 1]; t_cz2 += e * e; t_czw += e * f; }
+            if (b & NB_YP) { const T e = zj - zval(j + nx), f = wj - w[j + nx]; t_cz2 += e * e; t_czw += e * f; }
+            if (b & NB_ZP) { const T e = zj - zval(j + nxy), f = wj - w[j + nxy]; t_cz2 += e * e; t_czw += e * f; }
+            t_zg += zj * gj;
+            t_zzd += zj * zj * dj;
         };
         // four voxels per pass with their own loads issued first (the gathers of a voxel
         // depend on its list entry), then the rest one by one, in the same voxel order
@@ -649,22 +653,23 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
             const long long j = a.vlist[k];
             dir_voxel(k, j, a.nb[j], p[j], zo[j], w[j], g[j], d[j]);
         }
-        const double v[4] = {(double)s_cz2, (double)s_czw, (double)s_zg, (double)s_zzd};
+        const double v[4] = {(double)t_cz2, (double)t_czw, (double)t_zg, (double)t_zzd};
         const double bs = block_sum_256<4>(v, s_val);
         if (wid < 4 && lane0 == 0) a.partials[(size_t)wid * nb + blockIdx.x] = bs;
-        if (!grid_barrier(a.istate, a.spin_limit, nb)) return;
+        if (!ls_barrier(a.istate, a.spin_limit, nb, &s_bar)) return;
         if (wid < 4) {
             const double t = sum_partials_256(a.partials + (size_t)wid * nb, nb);
             if (lane0 == 0) s_tot[wid] = t;
         }
         __syncthreads();
     }
-    double alpha = 0.0, cz2 = 0.0, czw = 0.0;  // thread 0's
     if (threadIdx.x == 0) {
-        cz2 = s_tot[0];
-        czw = s_tot[1];
+        const double mu = s_mu, cz2 = s_tot[0], czw = s_tot[1];
         const double den = s_tot[3] + a.beta * cz2;
-        alpha = den != 0.0 ? -s_tot[2] / den : 0.0;
+        const double alpha = den != 0.0 ? -s_tot[2] / den : 0.0;
+        s_cz2 = cz2;
+        s_czw = czw;
+        s_alpha = alpha;
         s_aT = (T)alpha;
         if (blockIdx.x == 0) {
             a.scal[S_CZ2] = cz2;
@@ -735,16 +740,18 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
         const double bs = block_sum_256<2>(v, s_val);
         double* part = a.partials + 4 * (size_t)nb + (size_t)(step & 1) * 2 * nb;
         if (wid < 2 && lane0 == 0) part[(size_t)wid * nb + blockIdx.x] = bs;
-        if (!grid_barrier(a.istate, a.spin_limit, nb)) return;
+        if (!ls_barrier(a.istate, a.spin_limit, nb, &s_bar)) return;
         if (wid < 2) {
             const double t = sum_partials_256(part + (size_t)wid * nb, nb);
             if (lane0 == 0) s_tot[wid] = t;
         }
         __syncthreads();
         if (threadIdx.x == 0) {
-            const double fp = s_tot[0] + a.beta * (czw + alpha * cz2);
-            const double den = s_tot[1] + a.beta * cz2;
+            double alpha = s_alpha;
+            const double fp = s_tot[0] + a.beta * (s_czw + alpha * s_cz2);
+            const double den = s_tot[1] + a.beta * s_cz2;
             alpha = den == 0.0 ? 0.0 : alpha - fp / den;
+            s_alpha = alpha;
             s_aT = (T)alpha;
             s_stop = den == 0.0;
         }
@@ -752,10 +759,12 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
         if (s_stop) break;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const double alpha = s_alpha;
         a.scal[S_ALPHA] = alpha;
         if (a.alpha_hist) a.alpha_hist[it] = alpha;
         if (!isfinite(alpha)) set_err(a.istate, FM_ERR_NONFINITE);
         a.istate[I_ITER] = it + 1;
+        a.istate[I_LS_PH] = s_bar;
     }
 }
 
