@@ -1060,12 +1060,6 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     A(&c->order, 2 * (size_t)c->ntiles * sizeof(int));
     A(&c->order_act, 3 * (size_t)c->ntiles * sizeof(int));  // and the dot-product units
     A(&c->tile_rng, (size_t)c->ntiles * sizeof(unsigned));
-    if (c->ict_xch_bytes) {
-        const int units = ictw_units(Geo{nx, ny, nz, c->nv});
-        A(&c->ict_xch, c->ict_xch_bytes);
-        A(&c->ict_part, 2 * (size_t)units * sizeof(double));
-        A(&c->ict_rows, (size_t)units * sizeof(int4));
-    }
 
     if (!ok) { cudaGetLastError(); return bail(FM_ERR_OOM); }
 #ifndef FM_IC_WXY
@@ -1077,6 +1071,22 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     if (o.precond == FM_PC_ICT) {  // IC(0)'s offsets and the level-1 fill offsets, in plane order
         c->ict_off = {-1, 0, 0, 0, -1, 0, 0, 0, -1, 1, -1, 0, 1, 0, -1, 0, 1, -1};
         if (ict_build(c) != FM_OK) return bail(FM_ERR_OOM);
+    }
+    // last, so that a volume that only fits without it still opens: it takes the table-driven sweeps
+    if (c->ict_xch_bytes) {
+        const size_t units = (size_t)ictw_units(Geo{nx, ny, nz, c->nv});
+        if (dalloc(&c->ict_xch, c->ict_xch_bytes) != cudaSuccess ||
+            dalloc(&c->ict_part, 2 * units * sizeof(double)) != cudaSuccess ||
+            dalloc(&c->ict_rows, units * sizeof(int4)) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(c->ict_xch);
+            cudaFree(c->ict_part);
+            cudaFree(c->ict_rows);
+            c->ict_xch = c->ict_part = nullptr;
+            c->ict_rows = nullptr;
+            c->ict_xch_bytes = 0;
+            c->grid_ict = c->base_ict = 0;
+        }
     }
     if (!set_ic_order(c, FM_IC_WXY, FM_IC_WZ) ||
         cudaMemset(c->scal, 0, S_NSCAL * sizeof(double)) != cudaSuccess ||
