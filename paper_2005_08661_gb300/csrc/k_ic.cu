@@ -802,10 +802,12 @@ __device__ __forceinline__ void kahan_add(double& s, double& c, double x, double
 // plane: each lane sums a column of 32 voxels along y in order, in T with Kahan compensation, and
 // converts it to double once (per-product FP64 additions would queue on GB300's narrow FP64 pipe,
 // about 1/64 of the FP32 rate); the columns are added in double.  All of a column's loads are in
-// flight together.  p comes from other blocks of this launch.
+// flight together.  p comes from other blocks of this launch, and only where they swept: of the
+// unit's two tiles one may hold no mask voxel, and nothing has written p there.  Its rows (outside
+// y in [ylo, yhi)) count as the zeros they stand for.
 template <typename T>
-__device__ __forceinline__ void unit_dots(const T* p, const T* g, const T* gp, int x0, int y0, int z0, const Geo& geo,
-                                          double (&acc)[2]) {
+__device__ __forceinline__ void unit_dots(const T* p, const T* g, const T* gp, int x0, int y0, int z0, int ylo, int yhi,
+                                          const Geo& geo, double (&acc)[2]) {
     constexpr int B = sizeof(T) == 4 ? 32 : 16;  // voxels in flight
     static_assert(kThreadsB == 32 * kTZ, "one column per thread");
     const int x = x0 + (threadIdx.x & 31), z = z0 + (threadIdx.x >> 5);
@@ -818,7 +820,7 @@ __device__ __forceinline__ void unit_dots(const T* p, const T* g, const T* gp, i
             for (int k = 0; k < B; ++k) {
                 const int y = y0 + r0 + k;
                 const long long j = ((long long)z * geo.ny + y) * geo.nx + x;
-                const bool in = y < geo.ny;
+                const bool in = y >= ylo && y < yhi;
                 pv[k] = in ? __ldcg(p + j) : T(0);
                 gv[k] = in && g ? g[j] : T(0);
                 qv[k] = in && gp ? gp[j] : T(0);
@@ -848,7 +850,7 @@ __global__ void __launch_bounds__(kThreadsB, sizeof(T) == 4 ? 2 : 1) k_ic_bwd(Ic
     T* sip = sv + kVox;          // 1/pi
     T* f_in = sip + kVox;        // incoming faces
     T* ring = f_in + FN::n;      // step records [2][C][kRows]
-    __shared__ int s_tile;
+    __shared__ int s_tile, s_yhi;
     __shared__ __align__(8) unsigned long long s_mbar[Steps<C>::chunks];
     __shared__ bool s_last;
     __shared__ double sbuf[2 * 32];
@@ -972,9 +974,10 @@ __global__ void __launch_bounds__(kThreadsB, sizeof(T) == 4 ? 2 : 1) k_ic_bwd(Ic
             s_tile = u < nhalf ? u : -1;
             if (u < nhalf) {
                 const int t = a.unit[nhalf / 2 - 1 - u / 2], Y = (t / a.ntx) % a.nty;
+                const bool both = !(Y & 1) && Y + 1 < a.nty && (a.range[t + a.ntx] & 255u) != 255u;
+                s_yhi = min(ny, (Y + (both ? 2 : 1)) * kTY);
                 bool ok = wait_written(a.written + t, a.spin_limit);
-                if (!(Y & 1) && Y + 1 < a.nty && (a.range[t + a.ntx] & 255u) != 255u)
-                    ok = wait_written(a.written + t + a.ntx, a.spin_limit) && ok;
+                if (both) ok = wait_written(a.written + t + a.ntx, a.spin_limit) && ok;
                 if (!ok) set_err(a.istate, FM_ERR_TIMEOUT);
             }
         }
@@ -983,7 +986,7 @@ __global__ void __launch_bounds__(kThreadsB, sizeof(T) == 4 ? 2 : 1) k_ic_bwd(Ic
         if (u < 0) break;
         const int t = a.unit[nhalf / 2 - 1 - u / 2], X = t % a.ntx, Y = (t / a.ntx) % a.nty, Z = t / (a.ntx * a.nty);
         double acc[2] = {0.0, 0.0};
-        unit_dots<T>(p, gd, gpd, X * kTX + 32 * (u & 1), (Y & ~1) * kTY, Z * kTZ, geo, acc);
+        unit_dots<T>(p, gd, gpd, X * kTX + 32 * (u & 1), (Y & ~1) * kTY, Z * kTZ, Y * kTY, s_yhi, geo, acc);
         block_sum<2>(acc, sbuf);
         if (tid == 0) {
             // by place, in blocks of 32 x 32 x 8 voxels (blocks outside the mask stay 0)
