@@ -70,11 +70,12 @@ __device__ __forceinline__ unsigned phase_fixed(float w, float dtt) {
     return (unsigned)(unsigned long long)__float2ll_rn(hi) + (unsigned)__float2int_rn(lo);
 }
 
-// w (t_m - t_n) as a fixed-point angle, reduced by turns in float before the conversion (the 64-bit
-// conversion of phase_fixed runs on the narrow FP64 pipe).
+// The same reduced by turns in float before the conversion (the 64-bit conversion of phase_fixed
+// runs on the narrow FP64 pipe).  Both hold to 2^24 turns, where lo leaves 32 bits; rintf and not the
+// addition of 1.5 * 2^23, which finds whole turns below 2^22 only.
 __device__ __forceinline__ unsigned phase_fixed_32(float w, float dtt) {
     const float hi = w * dtt, lo = fmaf(w, dtt, -hi);
-    const float k = fmaf(hi, 2.3283064365386963e-10f, 12582912.0f) - 12582912.0f;  // whole turns
+    const float k = rintf(hi * 2.3283064365386963e-10f);  // whole turns
     return (unsigned)__float2int_rn(fmaf(k, -4294967296.0f, hi)) + (unsigned)__float2int_rn(lo);
 }
 
