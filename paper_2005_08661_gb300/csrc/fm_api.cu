@@ -1049,7 +1049,10 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     for (int k = 0; k < 2; ++k) { A(&c->w[k], vb); A(&c->z[k], vb); A(&c->g[k], vb); }
     A(&c->d, vb); A(&c->p, vb); A(&c->v, vb); A(&c->ip, vb); A(&c->rho, vb); A(&c->zw, 2 * vb);
     A(&c->scal, S_NSCAL * sizeof(double));
-    A(&c->partials, std::max<size_t>(8 * (size_t)std::max(c->grid_data, c->grid_ls), nchunks) * sizeof(double));
+    // 8 values a block for every line search the context may come to (fm_set_fat_model changes the
+    // evaluator), 2 a block of the level sweeps, whose blocks follow the (y, z) columns and not the voxels
+    A(&c->partials, std::max({8 * (size_t)std::max(c->grid_data, kLsMaxBlocks * c->nsm), 2 * (size_t)c->base_ictg,
+                              (size_t)nchunks}) * sizeof(double));
     c->face_bytes = (size_t)c->ntiles *
                     (o.precision == FM_FP64 ? ic_face_bytes_per_tile<double>() : ic_face_bytes_per_tile<float>());
     A(&c->face, c->face_bytes);

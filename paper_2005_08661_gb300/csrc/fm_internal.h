@@ -533,6 +533,7 @@ template <typename T> size_t ic_face_bytes_per_tile();
 template <typename T> int ic_max_blocks_per_sm(bool bwd);  // resident IC sweep blocks per SM
 
 constexpr int kThreads = 256;     // data-term / stencil kernels
+constexpr int kLsMaxBlocks = 4;   // line-search blocks per SM, of any evaluator
 constexpr int kTileX = 64, kTileY = 16;  // IC sweep tiles (k_ic.cu)
 
 }  // namespace fm

@@ -15,6 +15,7 @@
 // FP32 mode evaluates the voxel arithmetic in float and sums in double; FP64 mode is double
 // throughout.  Global sums are block partials reduced in a fixed order (bitwise
 // reproducible).
+#include <algorithm>
 #include <type_traits>
 
 #include "fm_internal.h"
@@ -567,12 +568,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && NC == 1 ? 4 : 2) k
 // the first nb blocks take part -- one mask voxel per thread at most (fewer threads with
 // several voxels each measured slower: each voxel is a chain of dependent gathers) -- and the
 // rest leave before the first grid barrier, which then counts the nb participants only.
-// Resident blocks per SM the line search is compiled for.  The grid follows from it, and with the
-// grid each thread's voxels and the order of every sum, so it is stated rather than left to the
-// compiler's register count: 128 registers for eight coils in registers and the lane-shared form
+// Resident blocks per SM of the line search: compiled for, and the most that its grid takes
+// (ls_max_blocks_per_sm), as each thread's voxels and the order of every sum follow from the grid and
+// should not from the compiler's register count.  128 registers for eight coils in registers and the lane-shared form
 // (whose polynomial constants otherwise do not stay in registers), 64 to 80 for the others.
 template <typename T, int NC> constexpr int ls_blocks() {
-    return sizeof(T) == 8 ? (NC == 0 ? 3 : 2) : NC == 8 || NC < 0 || NC > kPadded + 4 ? 2 : NC > kPadded ? 3 : 4;
+    constexpr int n = sizeof(T) == 8 ? (NC == 0 ? 3 : 2) : NC == 8 || NC < 0 || NC > kPadded + 4 ? 2 : NC > kPadded ? 3 : 4;
+    static_assert(n <= kLsMaxBlocks, "a context's partials buffer holds kLsMaxBlocks blocks per SM");
+    return n;
 }
 
 template <typename T, int NC>
@@ -860,7 +863,7 @@ int ls_max_blocks_per_sm(const DataArgs& a) {
         int n = 0;
         const cudaError_t e =
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ls<T, decltype(nc)::value>, kThreads, 0);
-        return e == cudaSuccess ? n : 0;
+        return e == cudaSuccess ? std::min(n, ls_blocks<T, decltype(nc)::value>()) : 0;
     });
 }
 
