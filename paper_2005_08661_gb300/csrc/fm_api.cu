@@ -44,7 +44,7 @@ struct fm_ctx {
     size_t face_bytes = 0;  // per-tile IC face buffers (the forward part starts unset: all bits set)
     double *hist_cost = nullptr, *hist_alpha = nullptr, *hist_mu = nullptr;
     int hist_cap = 0;
-    int hist_gen = 0;      // bumped when the history buffers move (captured graphs hold them)
+    int hist_gen = 0;      // bumped when the history or factor buffers move (a batch's graph holds them)
     int* istate = nullptr;
     int* icint = nullptr;  // IC sweeps: [0] forward ticket, [1] back-substitution ticket, [2] its done count,
                            // [3] its unit ticket, [4 ..] its written flags, one per tile
@@ -308,6 +308,36 @@ bool lex_less(const int* a, const int* b) {
     return a[0] < b[0];
 }
 
+// Gives the row wavefront's buffers back; the context takes the table-driven sweeps from then on.
+// False where it holds none.
+bool ict_drop_rows(fm_ctx* c) {
+    if (!c->ict_xch) return false;
+    cudaStreamSynchronize(c->stream);
+    cudaFree(c->ict_xch);
+    cudaFree(c->ict_part);
+    cudaFree(c->ict_rows);
+    c->ict_xch = c->ict_part = nullptr;
+    c->ict_rows = nullptr;
+    c->ict_xch_bytes = 0;
+    c->grid_ict = c->base_ict = 0;
+    if (c->gexec) { cudaGraphExecDestroy(c->gexec); c->gexec = nullptr; }
+    if (c->cg_gexec) { cudaGraphExecDestroy(c->cg_gexec); c->cg_gexec = nullptr; }
+    c->hist_gen++;
+    return true;
+}
+
+// dalloc for what a context allocates after fm_create: where memory is short the wavefront's buffers,
+// which are there for speed alone, give way.
+template <typename P>
+cudaError_t dalloc_late(fm_ctx* c, P** ptr, size_t bytes) {
+    cudaError_t e = dalloc(ptr, bytes);
+    if (e == cudaErrorMemoryAllocation && ict_drop_rows(c)) {
+        cudaGetLastError();
+        e = dalloc(ptr, bytes);
+    }
+    return e;
+}
+
 int ceil_div_pos(long long num, long long den) {  // ceil(num / den), den > 0
     return (int)(num >= 0 ? (num + den - 1) / den : -((-num) / den));
 }
@@ -371,6 +401,7 @@ int ict_build(fm_ctx* c) {
     auto put = [&](const std::vector<int>& v) { const size_t at = tab.size(); tab.insert(tab.end(), v.begin(), v.end()); return at; };
     const size_t a_off = put(c->ict_off), a_ord = put(ord), a_hs = put(hs), a_pp = put(pp), a_pr = put(pr),
                  a_qoff = put(qoff), a_qp = put(qp), a_qpr = put(qpr);
+    if (nh > kIctBaseOffsets) ict_drop_rows(c);  // it holds the base pattern only, and patterns never shrink
     if (c->ict_tab) { cudaFree(c->ict_tab); c->ict_tab = nullptr; }
     if (c->ict_qflags) { cudaFree(c->ict_qflags); c->ict_qflags = nullptr; }
     const int nflag = std::max(1, (nq + 31) / 32);
@@ -409,6 +440,7 @@ int ict_build(fm_ctx* c) {
         c->have_factor = false;
     }
     FM_CK(cudaMemset(c->ict_L, 0, (size_t)c->ict_nplanes * c->nv * sizeof(double)), "clear factor");
+    c->hist_gen++;
     if (c->gexec) { cudaGraphExecDestroy(c->gexec); c->gexec = nullptr; }  // the tables are kernel arguments
     if (c->cg_gexec) { cudaGraphExecDestroy(c->cg_gexec); c->cg_gexec = nullptr; }
     return FM_OK;
@@ -584,9 +616,9 @@ int solve_begin(fm_ctx* c, void* omega, int init, int niter, bool host_io = fals
         c->hist_cost = c->hist_alpha = c->hist_mu = nullptr;
         c->hist_cap = 0;
         const int cap = std::max(niter + 1, 128);
-        FM_CK(dalloc(&c->hist_cost, cap * sizeof(double)), "allocate history");
-        FM_CK(dalloc(&c->hist_alpha, cap * sizeof(double)), "allocate history");
-        FM_CK(dalloc(&c->hist_mu, cap * sizeof(double)), "allocate history");
+        FM_CK(dalloc_late(c, &c->hist_cost, cap * sizeof(double)), "allocate history");
+        FM_CK(dalloc_late(c, &c->hist_alpha, cap * sizeof(double)), "allocate history");
+        FM_CK(dalloc_late(c, &c->hist_mu, cap * sizeof(double)), "allocate history");
         c->hist_cap = cap;
         c->hist_gen++;
     }
@@ -656,7 +688,7 @@ int solve_t(fm_ctx* c, void* omega, int init, int niter, double* cost_hist, bool
     bool in_host = host_io;
     if (!init) {  // keep the start map: the output overwrites omega
         const size_t vb = (size_t)c->nv * c->ts;
-        if (!c->ict_w0 && dalloc(&c->ict_w0, vb) != cudaSuccess) {
+        if (!c->ict_w0 && dalloc_late(c, &c->ict_w0, vb) != cudaSuccess) {
             cudaGetLastError();
             return fail(c, FM_ERR_OOM, "allocate start map");
         }
@@ -1082,13 +1114,10 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
             dalloc(&c->ict_part, 2 * units * sizeof(double)) != cudaSuccess ||
             dalloc(&c->ict_rows, units * sizeof(int4)) != cudaSuccess) {
             cudaGetLastError();
-            cudaFree(c->ict_xch);
-            cudaFree(c->ict_part);
-            cudaFree(c->ict_rows);
-            c->ict_xch = c->ict_part = nullptr;
-            c->ict_rows = nullptr;
-            c->ict_xch_bytes = 0;
-            c->grid_ict = c->base_ict = 0;
+            if (!ict_drop_rows(c)) {
+                c->ict_xch_bytes = 0;
+                c->grid_ict = c->base_ict = 0;
+            }
         }
     }
     if (!set_ic_order(c, FM_IC_WXY, FM_IC_WZ) ||
@@ -1413,8 +1442,8 @@ int fm_set_data_host(fm_ctx* c, const void* y, const void* smap, const double* t
     }
     const int k = c->st_next;
     if (!c->st_y[k]) {
-        bool ok = dalloc(&c->st_y[k], yb) == cudaSuccess && dalloc(&c->st_s[k], sb) == cudaSuccess &&
-                  dalloc(&c->st_m[k], mb) == cudaSuccess;
+        bool ok = dalloc_late(c, &c->st_y[k], yb) == cudaSuccess && dalloc_late(c, &c->st_s[k], sb) == cudaSuccess &&
+                  dalloc_late(c, &c->st_m[k], mb) == cudaSuccess;
         if (!ok) { cudaGetLastError(); return fail(c, FM_ERR_OOM, "allocate staging buffers"); }
     }
     c->st_next ^= 1;
@@ -1847,7 +1876,7 @@ int fm_batch_solve(fm_batch* b, void* const* omega, int init_from_data, int nite
         for (size_t k = 0; k < b->v.size(); ++k) {
             fm_ctx* c = b->v[k];
             const size_t vb = (size_t)c->nv * c->ts;
-            if (!c->ict_w0 && dalloc(&c->ict_w0, vb) != cudaSuccess) { cudaGetLastError(); return FM_ERR_OOM; }
+            if (!c->ict_w0 && dalloc_late(c, &c->ict_w0, vb) != cudaSuccess) { cudaGetLastError(); return FM_ERR_OOM; }
             if (cudaMemcpyAsync(c->ict_w0, omega[k], vb, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
                 return FM_ERR_CUDA;
             in[k] = c->ict_w0;
