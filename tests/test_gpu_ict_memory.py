@@ -80,3 +80,45 @@ def test_the_exchange_buffer_makes_room_for_the_start_map():
         w = to_np(inout)
     # the two routes of the factor differ by the order of their sums
     np.testing.assert_allclose(w, ref, rtol=0, atol=1e-9)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_without_room_for_the_exchange_buffer_the_level_sweeps_hold_the_base_pattern(prec):
+    """A context that opens with too little memory for the exchange buffer gives the factor and the
+    substitutions of one that has it, alone and in a solve.  Tolerances as in test_gpu_ict_rows.py."""
+    nx, ny, nz, beta, drop = 160, 128, 64, 0.3, 0.007  # level-1 fill kept, none deeper
+    vol = make_volume(nx, ny, nz, ncoil=1, snr_db=20.0, seed=4, fmax_hz=120.0, nblobs=3)
+    y, s, m = dev_inputs(vol, prec)
+    rng = np.random.default_rng(13)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    d = torch.from_numpy(rng.uniform(0.3, 3.0, size=vol.mask.shape)).cuda().to(dt)
+    g = torch.from_numpy(rng.standard_normal(vol.mask.shape)).cuda().to(dt)
+
+    def run(fm):
+        fm.set_data(y, s, vol.te, m, beta)
+        ip = to_np(fm.ic_factor_curv(d))
+        p = to_np(fm.ic_apply(g))
+        assert len(fm.ict_pattern(planes=False)[0]) == 6
+        return ip, p, to_np(fm.solve(niter=2)[0])
+
+    _grow_a_pattern()
+    before = _free()
+    with FieldMap(nx, ny, nz, precision=prec, precond="ict", droptol=drop) as fm:
+        whole = before - _free()
+        ref = run(fm)
+    short = whole - 40 * vol.mask.size  # the exchange buffer has at least 48 bytes a voxel
+    with _left(short):
+        fm = FieldMap(nx, ny, nz, precision=prec, precond="ict", droptol=drop)
+    got = run(fm)
+    fm.close()
+    tol = 1e-11 if prec == "fp64" else 2e-4
+    for a, b in zip(got[:2], ref[:2]):
+        assert np.max(np.abs(a - b)) <= tol * np.max(np.abs(b))
+    move = np.abs(ref[2] - to_np(_start(vol, y, s, m, beta, prec))).max()
+    assert np.max(np.abs(got[2] - ref[2])) <= (1e-9 if prec == "fp64" else 1e-4 * move)
+
+
+def _start(vol, y, s, m, beta, prec):
+    with FieldMap(vol.nx, vol.ny, vol.nz, precision=prec) as fm:
+        fm.set_data(y, s, vol.te, m, beta)
+        return fm.init_omega()
