@@ -53,7 +53,7 @@ struct fm_ctx {
     unsigned* tile_rng = nullptr;  // per tile: steps of the sweeps that reach a mask voxel
     int ntx = 0, nty = 0, ntz = 0, ntiles = 0, npart = 0;
     int ic_wxy = 2, ic_wz = 1;  // forward tile claim order weights
-    int lanes = 1;  // lanes that share a voxel in the data-term kernels
+    int lanes = 1;  // most lanes that share a voxel in the data-term kernels
     int nsm = 0, grid_data = 0, grid_ls = 0, grid_ic = 0, grid_icb = 0;  // grid_icb: backward IC sweep
     int base_data = 0, base_ls = 0, base_ic = 0, base_icb = 0;
     int occ_icb = 0;  // resident back-substitution blocks per SM the kernel allows

@@ -498,7 +498,7 @@ template <typename T> cudaError_t launch_grad(const DataArgs& a, int grid, cudaS
 template <typename T> cudaError_t launch_ls(const DataArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_pdiag(const DataArgs& a, int mode, int grid, cudaStream_t s);
 template <typename T> int ls_max_blocks_per_sm(const DataArgs& a);
-int data_lanes(const DataArgs& a);  // FP32: lanes that share a voxel in the data-term kernels
+int data_lanes(const DataArgs& a);  // FP32: most lanes that share a voxel in the data-term kernels
 template <typename T> cudaError_t launch_rb_black(const DataArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_rb_red(const DataArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, unsigned* range,

@@ -350,36 +350,19 @@ __device__ __forceinline__ void eval_padded(const DataArgs& a, long long j, floa
     curv = 2.f * d_acc;
 }
 
-// Evaluator codes of the kernels below (with_evaluator): kPadded + NR is eval_padded.
-constexpr int kPadded = 100;
-
-// The three-echo path in registers, the padded one, or the general one.
-template <typename T, int NC, bool COST, bool CURV>
-__device__ __forceinline__ void eval_any(const DataArgs& a, long long j, T w, T& cost, T& grad, T& curv) {
-    if constexpr (NC > kPadded) {
-        eval_padded<NC - kPadded, COST, CURV>(a, j, w, cost, grad, curv);
-    } else if constexpr (sizeof(T) == 4 && NC > 1) {
-        eval_fixed<T, NC, 3, COST, CURV>(a, j, w, cost, grad, curv);
-    } else {
-        if (NC != 0 && a.L == 3) eval_fixed<T, (NC == 0 ? 1 : NC), 3, COST, CURV>(a, j, w, cost, grad, curv);
-        else eval_voxel<T, NC, COST, CURV>(a, j, w, cost, grad, curv);
-    }
-}
-
 // ------------------------------------------------------------------ voxels shared by lanes
 
-// FP32 literal curvature of more than eight coils, any echo count: SP = 8 lanes share a voxel.
-// Lane slice sl takes the rows c = sl, sl + 8, .. of every pair's sum over (c, d), and the pairs
-// sl, sl + 8, .. of the cost and gradient; the slices' results add up to the voxel's.
+// FP32 literal curvature of more than eight coils, any echo count: SP lanes share a voxel, eight or
+// one (slice_lanes).  Lane slice sl takes the rows c = sl, sl + SP, .. of every pair's sum over (c, d),
+// and the pairs sl, sl + SP, .. of the cost and gradient; the slices' results add up to the voxel's.
 //
-// Bound by FP32 issue: a pair has N_c^2 terms of about 6 slots.  One thread per voxel left the
-// chip idle where coils are many and voxels few (74 x 74 x 10 voxels with 32 coils: 14,000 mask
-// voxels for 152 SMs, each thread 3072 terms in sequence, one coil load per term and no reuse): the
-// line search took 630 us, with 8 lanes per voxel 228 (gradient 108, 47).  Below nine coils the
-// padded form is the faster one (four coils: line search 129 us, with four lanes per voxel 205).  A lane holds eight
-// d in registers for all of its rows, two terms per instruction as in coil_pair_sum_x2; the lanes
-// of a slice are neighbouring voxels, so that a load fetches whole 32-byte sectors of each coil's
-// plane.
+// Bound by FP32 issue: a pair has N_c^2 terms of about 6 slots.  A lane holds eight d in registers for
+// all of its rows, two terms per instruction as in coil_pair_sum_x2 (with one coil load per term and no
+// reuse, 11 to 15 slots a term).  One lane per voxel leaves the chip idle where coils are many and
+// voxels few: 74 x 74 x 10 voxels with 32 coils are 14,000 mask voxels for 152 SMs, 3072 terms each, and
+// their line search took 630 us, with eight lanes per voxel 205 (gradient 108, 47).  The lanes of a slice
+// are neighbouring voxels, so that a load fetches whole 32-byte sectors of each coil's plane.  Up to
+// eight coils are eval_padded's, which holds both sides of a pair in registers.
 
 // sum over the rows c = sl, sl + SP, .. of |W_cm| sum_{d < DB} |W_dn| sinc(..), entries past the last
 // of nd coils counting as |W_dn| = 0.
@@ -464,6 +447,37 @@ __device__ __forceinline__ float slice_sum(float v) {
     return v;
 }
 
+// Lanes that share a voxel of a mask of nm voxels: kShared while the chip holds them in few rounds (9728
+// voxels with eight lanes each, two blocks per SM), else one, as a lane of its own keeps a voxel's rows
+// even and its loads whole (eight lanes have 16 rows' time for nine coils).  The more coils, the later:
+// line search / gradient in us with one and with eight lanes, three echoes, 9216 voxels: 9 coils 74 / 18
+// and 55 / 16, 32 coils 390 / 53 and 96 / 25; 20,480: 9 coils 76 / 20 and 95 / 31, 16 coils 127 / 26 and
+// 92 / 28, 32 coils 392 / 57 and 210 / 47; 82,944: 16 coils 227 / 45 and 212 / 63, 32 coils 759 / 127 and
+// 561 / 133; 393,216: 9 coils 332 / 77 and 1005 / 315.  With two echoes the pair's work is a third, and the
+// line lies at half as many voxels (12 coils, 10,240: 47 / 14 and 52 / 19).
+constexpr int kShared = 8;
+__device__ __forceinline__ int slice_lanes(const DataArgs& a, long long nm) {
+    return nm <= 2432LL * (a.nc - 5) / (a.pr.P < 3 ? 2 : 1) ? kShared : 1;
+}
+
+// Evaluator codes of the kernels below (with_evaluator): kPadded + NR is eval_padded.
+constexpr int kPadded = 100;
+
+// The three-echo path in registers, the padded one, or the general one.
+template <typename T, int NC, bool COST, bool CURV>
+__device__ __forceinline__ void eval_any(const DataArgs& a, long long j, T w, T& cost, T& grad, T& curv) {
+    if constexpr (NC < 0) {
+        eval_slice<1, COST>(a, j, 0, w, cost, grad, curv);
+    } else if constexpr (NC > kPadded) {
+        eval_padded<NC - kPadded, COST, CURV>(a, j, w, cost, grad, curv);
+    } else if constexpr (sizeof(T) == 4 && NC > 1) {
+        eval_fixed<T, NC, 3, COST, CURV>(a, j, w, cost, grad, curv);
+    } else {
+        if (NC != 0 && a.L == 3) eval_fixed<T, (NC == 0 ? 1 : NC), 3, COST, CURV>(a, j, w, cost, grad, curv);
+        else eval_voxel<T, NC, COST, CURV>(a, j, w, cost, grad, curv);
+    }
+}
+
 // ------------------------------------------------------------------ gradient pass
 
 // w_out = w_in + alpha z (the previous iteration's update, Algorithm box), then at w_out:
@@ -487,52 +501,56 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && NC == 1 ? 4 : 2) k
     // the thread's cost and penalty sums in T with Kahan compensation, converted to double
     // once (per-voxel FP64 additions would queue on GB300's narrow FP64 pipe)
     T cs = 0, cc = 0, rs = 0, rc = 0;
-    constexpr int SP = NC < 0 ? -NC : 1, VW = 32 / SP;  // lanes per voxel, voxels per warp
-    const int lane = threadIdx.x & 31, sl = lane / VW;
-    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long first = SP == 1 ? tid : tid / 32 * VW, stride = (long long)gridDim.x * blockDim.x / SP;
-    for (long long kb = first; kb < nm; kb += stride) {  // SP > 1: the same trips for a whole warp
-        const long long k = SP == 1 ? kb : min(kb + lane % VW, nm - 1);
-        const bool mine = SP == 1 || (sl == 0 && kb + lane % VW < nm);
-        constexpr bool kRegs = sizeof(T) == 4 && NC > 1 && NC < kPadded;  // three echoes, dispatched by coil count
-        VoxelData<T, kRegs ? NC : 1, 3, kRegs> data;
-        if constexpr (kRegs) data.load(a, k);  // in flight under the stencil's gathers
-        const long long j = a.vlist[k];
-        const T wj = upd(j);
-        T lap = 0, reg = 0;
-        if (mine) {
-            const uint8_t b = a.nb[j];
-            w_out[j] = wj;
-            if (b & NB_XM) lap += wj - upd(j - 1);
-            if (b & NB_YM) lap += wj - upd(j - nx);
-            if (b & NB_ZM) lap += wj - upd(j - nxy);
-            if (b & NB_XP) { const T e = wj - upd(j + 1); lap += e; reg += e * e; }
-            if (b & NB_YP) { const T e = wj - upd(j + nx); lap += e; reg += e * e; }
-            if (b & NB_ZP) { const T e = wj - upd(j + nxy); lap += e; reg += e * e; }
+    auto pass = [&](auto lanes) {
+        constexpr int SP = decltype(lanes)::value, VW = 32 / SP;  // lanes per voxel, voxels per warp
+        const int lane = threadIdx.x & 31, sl = lane / VW;
+        const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+        const long long first = SP == 1 ? tid : tid / 32 * VW, stride = (long long)gridDim.x * blockDim.x / SP;
+        for (long long kb = first; kb < nm; kb += stride) {  // SP > 1: the same trips for a whole warp
+            const long long k = SP == 1 ? kb : min(kb + lane % VW, nm - 1);
+            const bool mine = SP == 1 || (sl == 0 && kb + lane % VW < nm);
+            constexpr bool kRegs = sizeof(T) == 4 && NC > 1 && NC < kPadded;  // three echoes, dispatched by coil count
+            VoxelData<T, kRegs ? NC : 1, 3, kRegs> data;
+            if constexpr (kRegs) data.load(a, k);  // in flight under the stencil's gathers
+            const long long j = a.vlist[k];
+            const T wj = upd(j);
+            T lap = 0, reg = 0;
+            if (mine) {
+                const uint8_t b = a.nb[j];
+                w_out[j] = wj;
+                if (b & NB_XM) lap += wj - upd(j - 1);
+                if (b & NB_YM) lap += wj - upd(j - nx);
+                if (b & NB_ZM) lap += wj - upd(j - nxy);
+                if (b & NB_XP) { const T e = wj - upd(j + 1); lap += e; reg += e * e; }
+                if (b & NB_YP) { const T e = wj - upd(j + nx); lap += e; reg += e * e; }
+                if (b & NB_ZP) { const T e = wj - upd(j + nxy); lap += e; reg += e * e; }
+            }
+            T cst, gr, cu;
+            if constexpr (SP > 1) {
+                eval_slice<SP, true>(a, k, sl, wj, cst, gr, cu);
+                cst = slice_sum<SP>(cst);
+                gr = slice_sum<SP>(gr);
+                cu = slice_sum<SP>(cu);
+                if (!mine) continue;
+            } else if constexpr (kRegs) {
+                data.template eval<true>(a, wj, cst, gr, cu);
+            } else {
+                eval_any<T, NC, true, true>(a, k, wj, cst, gr, cu);
+            }
+            if (g) g[j] = gr + beta * lap;
+            if (d) d[j] = cu;
+            {
+                const T y1 = cst - cc, t1 = cs + y1;
+                cc = (t1 - cs) - y1;
+                cs = t1;
+                const T y2 = reg - rc, t2 = rs + y2;
+                rc = (t2 - rs) - y2;
+                rs = t2;
+            }
         }
-        T cst, gr, cu;
-        if constexpr (SP > 1) {
-            eval_slice<SP, true>(a, k, sl, wj, cst, gr, cu);
-            cst = slice_sum<SP>(cst);
-            gr = slice_sum<SP>(gr);
-            cu = slice_sum<SP>(cu);
-            if (!mine) continue;
-        } else if constexpr (kRegs) {
-            data.template eval<true>(a, wj, cst, gr, cu);
-        } else {
-            eval_any<T, NC, true, true>(a, k, wj, cst, gr, cu);
-        }
-        if (g) g[j] = gr + beta * lap;
-        if (d) d[j] = cu;
-        {
-            const T y1 = cst - cc, t1 = cs + y1;
-            cc = (t1 - cs) - y1;
-            cs = t1;
-            const T y2 = reg - rc, t2 = rs + y2;
-            rc = (t2 - rs) - y2;
-            rs = t2;
-        }
-    }
+    };
+    if (NC < 0 && slice_lanes(a, nm) > 1) pass(std::integral_constant<int, NC < 0 ? kShared : 1>());
+    else pass(std::integral_constant<int, 1>());
     double v[1] = {((double)cs - (double)cc) + 0.5 * a.beta * ((double)rs - (double)rc)}, out[1];
     if (last_block_reduce<1>(v, a.partials, (unsigned*)(a.istate + I_DONE0), out, sbuf)) {
         if (threadIdx.x == 0) {
@@ -591,8 +609,8 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
     T2* zw = (T2*)a.zw;
     const int it = a.istate[I_ITER];
     const long long nm = a.istate[I_NMASK];
-    constexpr int SP = NC < 0 ? -NC : 1, VW = 32 / SP;  // lanes per voxel, voxels per warp
-    const int nb = (int)max(1LL, min((long long)gridDim.x, (nm * SP + kThreads - 1) / kThreads));
+    const int sp = NC < 0 ? slice_lanes(a, nm) : 1;  // lanes per voxel
+    const int nb = (int)max(1LL, min((long long)gridDim.x, (nm * sp + kThreads - 1) / kThreads));
     if ((int)blockIdx.x >= nb) return;
     const int nx = a.geo.nx;
     const long long nxy = (long long)nx * a.geo.ny;
@@ -718,20 +736,26 @@ __global__ void __launch_bounds__(kThreads, ls_blocks<T, NC>()) k_ls(DataArgs a)
                 t1 += q.x * gr;
                 t2 += q.x * q.x * cu;
             }
-        } else if constexpr (SP > 1) {
-            // each slice adds its own share: the sums run over all lanes anyway
-            const int lane = threadIdx.x & 31;
-            const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
-            for (long long k = warp * VW + lane % VW; k < nm; k += (long long)nb * blockDim.x / SP) {
-                const T2 q = __ldcg(zw + k);  // written by another thread before the grid barrier
-                T cst, gr, cu;
-                eval_slice<SP, false>(a, k, lane / VW, q.y + aT * q.x, cst, gr, cu);
-                t1 += q.x * gr;
-                t2 += q.x * q.x * cu;
-            }
         } else {
+            bool shared = false;
+            if constexpr (NC < 0) {
+                if (sp > 1) {
+                    // each slice adds its own share: the sums run over all lanes anyway
+                    constexpr int SP = kShared, VW = 32 / SP;  // voxels per warp
+                    const int lane = threadIdx.x & 31;
+                    const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
+                    for (long long k = warp * VW + lane % VW; k < nm; k += (long long)nb * blockDim.x / SP) {
+                        const T2 q = __ldcg(zw + k);  // written by another thread before the grid barrier
+                        T cst, gr, cu;
+                        eval_slice<SP, false>(a, k, lane / VW, q.y + aT * q.x, cst, gr, cu);
+                        t1 += q.x * gr;
+                        t2 += q.x * q.x * cu;
+                    }
+                    shared = true;
+                }
+            }
             // a voxel with z = 0 adds exactly 0
-            for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nm;
+            for (long long k = shared ? nm : blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nm;
                  k += (long long)nb * blockDim.x) {
                 const T2 q = zw[k];
                 T cst, gr, cu;
@@ -812,7 +836,7 @@ __global__ void __launch_bounds__(kThreads) k_pdiag(DataArgs a, int mode) {
 
 // Calls f(integral constant NC) with the evaluator of a context: 1 coil-combined curvature (or one
 // coil); 2, 4, 8 that many coils and three echoes in registers; kPadded + NR (FP32) other literal
-// curvatures of up to NR coils; -8 (FP32) more than eight coils, eight lanes per voxel; 0 a runtime
+// curvatures of up to NR coils; -8 (FP32) more than eight coils, eight lanes per voxel or one; 0 a runtime
 // coil count with one thread per voxel (FP64, and the water-fat model).
 template <typename T, typename F>
 static auto with_evaluator(const DataArgs& a, F f) {
