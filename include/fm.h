@@ -396,7 +396,7 @@ FM_API int fm_batch_solve(fm_batch *b, void *const *omega, int init_from_data, i
  * use (candidates 1, 1/2, 1/4, 1/8), the order in which the IC(0) forward wavefront claims
  * its tiles (weights (X + Y) : Z of 2 : 1, 1 : 1, 3 : 2; any positive weights keep the
  * dependency order), and then, at the best of those, the back-substitution wavefront's blocks
- * per SM (1, 2 or 3, as its occupancy allows).  best_ms (host, nullable) receives the winning
+ * per SM (1 to 3, as far as they fit on an SM).  best_ms (host, nullable) receives the winning
  * probe time.  Requires fm_batch_set_data on every volume.  The schedule stays in effect
  * until changed (fm_batch_schedule and fm_batch_bwd_blocks report it). */
 FM_API int fm_batch_autotune(fm_batch *b, int niter_probe, double *best_fraction, double *best_ms);

@@ -1030,8 +1030,8 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     {
         // the two sweeps claim tiles from their own tickets, so each sizes its own grid: one block
         // per SM, as a second slows the other's steps (256x256x128 volume: forward 122 / 149 us per
-        // sweep at 1 / 2; back substitution on 192x192x96 71 / 77); a batch may take more
-        // (fm_batch_autotune)
+        // sweep at 1 / 2; back substitution on 192x192x96 71 / 77); a batch may take more for the
+        // back substitution (batch_icb, fm_batch_autotune)
         const bool f64 = o.precision == FM_FP64;
         const int occ_f = f64 ? ic_max_blocks_per_sm<double>(false) : ic_max_blocks_per_sm<float>(false);
         const int occ_b = f64 ? ic_max_blocks_per_sm<double>(true) : ic_max_blocks_per_sm<float>(true);
@@ -1689,7 +1689,7 @@ struct fm_batch {
     cudaGraphExec_t gexec = nullptr;
     std::vector<int> gen;  // history generations the captured graph was built with
     double fraction = 1.0;
-    int icb_per_sm = 2;  // back-substitution blocks per SM (before the fraction)
+    int icb_per_sm = 0;  // back-substitution blocks per SM (before the fraction) that the autotuner chose, or 0
     std::string err;
 };
 
@@ -1704,12 +1704,23 @@ void batch_free(fm_batch* b) {
     if (b->own_origin && b->origin) cudaStreamDestroy(b->origin);
 }
 
+// The back substitution's blocks per SM (before the fraction) as they run: no more than the kernel
+// allows on any volume, and until the autotuner has chosen, one from half of the grid on and two below,
+// where one would leave SMs to no volume.  One / two, 10 iterations in ms: eight uneven volumes at 1
+// 17.3 / 18.0, at 1/2 14.1 / 14.6, at 1/4 14.3 / 14.4, at 1/8 20.1 / 19.6; three volumes at 1 5.07 / 5.26, at 1/2
+// 3.62 / 3.79, at 1/4 4.45 / 4.07, at 1/8 6.86 / 6.01.
+int batch_icb(const fm_batch* b) {
+    int occ = 1;
+    for (const fm_ctx* c : b->v) occ = std::max(occ, c->occ_icb);
+    return std::min(b->icb_per_sm ? b->icb_per_sm : b->fraction >= 0.5 ? 1 : 2, occ);
+}
+
 void batch_apply_fraction(fm_batch* b) {
     for (fm_ctx* c : b->v) {
         c->grid_data = std::max(1, (int)std::lround(c->base_data * b->fraction));
         c->grid_ls = std::max(1, (int)std::lround(c->base_ls * b->fraction));
         c->grid_ic = std::max(1, (int)std::lround(c->base_ic * b->fraction));
-        const int icb = std::max(1, std::min(c->ntiles, std::min(c->occ_icb, b->icb_per_sm) * c->nsm));
+        const int icb = std::max(1, std::min(c->ntiles, std::min(c->occ_icb, batch_icb(b)) * c->nsm));
         c->grid_icb = std::max(1, (int)std::lround(icb * b->fraction));
         if (c->base_ict) c->grid_ict = std::max(1, (int)std::lround(c->base_ict * b->fraction));
         if (c->base_ictg) c->grid_ictg = std::max(1, (int)std::lround(c->base_ictg * b->fraction));
@@ -1850,6 +1861,7 @@ int fm_batch_create(fm_batch** out, int n, const int* dims, const fm_opts* opts,
         delete b;
         return FM_ERR_CUDA;
     }
+    batch_apply_fraction(b);  // the schedule that fm_batch_schedule and fm_batch_bwd_blocks report
     *out = b;
     return FM_OK;
 }
@@ -1916,7 +1928,9 @@ int fm_batch_autotune(fm_batch* b, int niter_probe, double* best_fraction, doubl
     ok = ok && cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
     const double cand[4] = {1.0, 0.5, 0.25, 0.125};
     const int wcand[3][2] = {{2, 1}, {1, 1}, {3, 2}};  // forward tile claim order weights (X + Y, Z)
-    const int bcand[3] = {1, 2, 3};                    // back-substitution blocks per SM
+    const int bcand[3] = {1, 2, 3};                    // back-substitution blocks per SM, as far as they fit
+    int occ = 1;
+    for (const fm_ctx* c : b->v) occ = std::max(occ, c->occ_icb);
     double bestf = b->fraction, bestt = 1e300;
     int bestw = 0, bestb = b->icb_per_sm;
     int rc = ok ? FM_OK : FM_ERR_OOM;
@@ -1936,7 +1950,7 @@ int fm_batch_autotune(fm_batch* b, int niter_probe, double* best_fraction, doubl
             bestt = ms;
             bestf = f;
             bestw = wq;
-            bestb = bcand[bq];
+            bestb = batch_icb(b);
         }
     };
     // grid fraction x forward claim order at two back-substitution blocks per SM, then the
@@ -1949,7 +1963,7 @@ int fm_batch_autotune(fm_batch* b, int niter_probe, double* best_fraction, doubl
     for (fm_ctx* c : b->v)
         if (rc == FM_OK && !set_ic_order(c, wcand[bestw][0], wcand[bestw][1])) rc = FM_ERR_CUDA;
     for (int bq = 0; bq < 3 && rc == FM_OK; ++bq)
-        if (bcand[bq] != 2) probe(bestf, bestw, bq);
+        if (bcand[bq] != 2 && bcand[bq] <= occ) probe(bestf, bestw, bq);
     for (void* p : w)
         if (p) cudaFree(p);
     if (e0) cudaEventDestroy(e0);
@@ -1974,7 +1988,7 @@ int fm_batch_schedule(const fm_batch* b, double* fraction, int* order_wxy, int* 
 
 int fm_batch_bwd_blocks(const fm_batch* b, int* blocks_per_sm) {
     if (!b || !blocks_per_sm) return FM_ERR_ARG;
-    *blocks_per_sm = b->icb_per_sm;
+    *blocks_per_sm = batch_icb(b);
     return FM_OK;
 }
 
