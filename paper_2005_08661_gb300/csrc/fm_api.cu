@@ -58,7 +58,9 @@ struct fm_ctx {
     int base_data = 0, base_ls = 0, base_ic = 0, base_icb = 0;
     int occ_icb = 0;  // resident back-substitution blocks per SM the kernel allows
     int grid_ict = 0, base_ict = 0;  // drop-tolerance IC: row wavefront (0: volume takes the level sweeps)
-    int grid_ictg = 0, base_ictg = 0, block_ict = 0;  // its table-driven sweeps (persistent, level barriers)
+    bool ict_level_factor = false;   // the factor takes the level sweeps all the same
+    int grid_ictl = 0, base_ictl = 0;                 // level sweeps of the base pattern (persistent, level barriers)
+    int grid_ictg = 0, base_ictg = 0, block_ict = 0;  // table-driven level sweeps of a grown one
     double *ict_xch = nullptr, *ict_part = nullptr;   // row wavefront: exchange buffer, dot products
     size_t ict_xch_bytes = 0;
     int4* ict_rows = nullptr;
@@ -308,7 +310,22 @@ bool lex_less(const int* a, const int* b) {
     return a[0] < b[0];
 }
 
-// Gives the row wavefront's buffers back; the context takes the table-driven sweeps from then on.
+// Form of the drop-tolerance IC's base pattern: which sweeps take rows, which levels (k_ict.cu).  A plane
+// of the row wavefront follows the one below by a group of 32 rows (64 steps) where planes have several
+// groups, by a few steps where they have one; by levels it follows after three, which cost a barrier each.
+// The ratio of the two chains, in steps per level, decides; the factor pays the most per step.  ms of
+// ic_factor / ic_apply by levels and by rows (droptol 0.02, no mask, FP32): 256x256x128 (ratio 8) 16.3 / 12.4
+// and 12.1 / 6.8; 96x96x96 (11) 6.5 / 4.8 and 6.3 / 3.6; 64x64x96 (13) 5.0 / 3.8 and 5.5 / 3.1; 64x64x128 (15) 6.1 /
+// 4.7 and 7.1 / 4.0; 64x64x256 (17) 10.6 / 7.8 and 13.6 / 8.0; 32x33x256 (19) 8.7 / 6.6 and 12.1 / 7.1; with one group
+// to a plane, 256x32x256 (2) 14.1 / 10.9 and 8.4 / 4.1.
+enum IctForm { kIctRows, kIctLevelFactor /* factor by levels, the rest by rows */, kIctLevels };
+IctForm ict_form(int nx, int ny, int nz) {
+    const long long nyb = (ny + 31) / 32;
+    const long long steps = nyb > 1 ? 64 * (nz + nyb) + nx : 6LL * nz + nx, levels = nx + 2LL * ny + 3LL * nz;
+    return steps < 12 * levels ? kIctRows : steps < 17 * levels ? kIctLevelFactor : kIctLevels;
+}
+
+// Gives the row wavefront's buffers back; the context takes the level sweeps from then on.
 // False where it holds none.
 bool ict_drop_rows(fm_ctx* c) {
     if (!c->ict_xch) return false;
@@ -497,9 +514,10 @@ cudaError_t run_ict(fm_ctx* c, const void* d, const void* g, void* p, const void
         e = launch_ict_tau<T>(t, c->o.droptol, c->grid_data, c->stream);
         if (e != cudaSuccess) return e;
     }
-    // the row wavefront holds exactly the base pattern
-    const bool base = c->ict_tb.nh == kIctBaseOffsets && c->grid_ict > 0;
-    if (base) {
+    // the row wavefront and the unrolled level sweeps hold exactly the base pattern
+    const bool base = c->ict_tb.nh == kIctBaseOffsets, rows = base && c->grid_ict > 0;
+    const bool fwd_rows = rows && !(d && c->ict_level_factor);
+    if (rows) {
         e = cudaMemsetAsync(c->icint, 0, 4 * sizeof(int), c->stream);
         if (e != cudaSuccess) return e;
         a.rows = c->ict_rows;
@@ -509,8 +527,9 @@ cudaError_t run_ict(fm_ctx* c, const void* d, const void* g, void* p, const void
         a.done = c->icint + 2;
     }
     if (prof) prof_record(c->ev[slot][FM_K_IC_FWD][0], c->stream);
-    e = base ? launch_ictw_fwd<T>(a, c->grid_ict, c->stream)
-             : launch_ictg_fwd<T>(a, c->grid_ictg, c->block_ict, c->stream);
+    e = fwd_rows ? launch_ictw_fwd<T>(a, c->grid_ict, c->stream)
+        : base   ? launch_ict_fwd<T>(a, c->grid_ictl, c->block_ict, c->stream)
+                 : launch_ictg_fwd<T>(a, c->grid_ictg, c->block_ict, c->stream);
     if (prof) {
         prof_record(c->ev[slot][FM_K_IC_FWD][1], c->stream);
         c->ev_rec[slot][FM_K_IC_FWD] = true;
@@ -522,8 +541,9 @@ cudaError_t run_ict(fm_ctx* c, const void* d, const void* g, void* p, const void
     }
     if (prof) prof_record(c->ev[slot][FM_K_IC_BWD][0], c->stream);
     a.ticket = c->icint + 1;
-    e = base ? launch_ictw_bwd<T>(a, c->grid_ict, c->stream)
-             : launch_ictg_bwd<T>(a, c->grid_ictg, c->block_ict, c->stream);
+    e = rows   ? launch_ictw_bwd<T>(a, c->grid_ict, c->stream)
+        : base ? launch_ict_bwd<T>(a, c->grid_ictl, c->block_ict, c->stream)
+               : launch_ictg_bwd<T>(a, c->grid_ictg, c->block_ict, c->stream);
     if (prof) {
         prof_record(c->ev[slot][FM_K_IC_BWD][1], c->stream);
         c->ev_rec[slot][FM_K_IC_BWD] = true;
@@ -1056,12 +1076,20 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
         c->grid_ictg = (int)std::max(1LL, std::min<long long>((cols + c->block_ict - 1) / c->block_ict,
                                                               (long long)occg * c->nsm));
         c->base_ictg = c->grid_ictg;
+        const int occl = o.precision == FM_FP64 ? ict_max_blocks_per_sm<double>(c->block_ict)
+                                                : ict_max_blocks_per_sm<float>(c->block_ict);
+        if (occl < 1) return bail(FM_ERR_CUDA);
+        c->grid_ictl = (int)std::max(1LL, std::min<long long>((cols + c->block_ict - 1) / c->block_ict,
+                                                              (long long)occl * c->nsm));
+        c->base_ictl = c->grid_ictl;
         // row wavefront: blocks claim row groups, eight one-warp blocks per SM at most.  Its exchange
         // buffer holds 32 lanes per row group, so thin volumes (few rows per plane) of large size
-        // would need many times their factor; they take the table-driven sweeps.
+        // would need many times their factor; they take the level sweeps.
         const Geo geo{nx, ny, nz, c->nv};
         const size_t xb = ictw_exchange_bytes(geo), limit = std::max<size_t>((size_t)1 << 30, 4 * kIctPlanes * sizeof(double) * (size_t)c->nv);
-        if (xb <= limit) {
+        const IctForm form = ict_form(nx, ny, nz);
+        c->ict_level_factor = form == kIctLevelFactor;
+        if (xb <= limit && form != kIctLevels) {
             c->ict_xch_bytes = xb;
             c->grid_ict = std::min(ictw_units(geo), 8 * c->nsm);
             c->base_ict = c->grid_ict;
@@ -1083,7 +1111,7 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
     A(&c->scal, S_NSCAL * sizeof(double));
     // 8 values a block for every line search the context may come to (fm_set_fat_model changes the
     // evaluator), 2 a block of the level sweeps, whose blocks follow the (y, z) columns and not the voxels
-    A(&c->partials, std::max({8 * (size_t)std::max(c->grid_data, kLsMaxBlocks * c->nsm), 2 * (size_t)c->base_ictg,
+    A(&c->partials, std::max({8 * (size_t)std::max(c->grid_data, kLsMaxBlocks * c->nsm), 2 * (size_t)std::max(c->base_ictg, c->base_ictl),
                               (size_t)nchunks}) * sizeof(double));
     c->face_bytes = (size_t)c->ntiles *
                     (o.precision == FM_FP64 ? ic_face_bytes_per_tile<double>() : ic_face_bytes_per_tile<float>());
@@ -1107,7 +1135,7 @@ int fm_create(fm_ctx** out, int nx, int ny, int nz, int ncoil, int necho, const 
         c->ict_off = {-1, 0, 0, 0, -1, 0, 0, 0, -1, 1, -1, 0, 1, 0, -1, 0, 1, -1};
         if (ict_build(c) != FM_OK) return bail(FM_ERR_OOM);
     }
-    // last, so that a volume that only fits without it still opens: it takes the table-driven sweeps
+    // last, so that a volume that only fits without it still opens: it takes the level sweeps
     if (c->ict_xch_bytes) {
         const size_t units = (size_t)ictw_units(Geo{nx, ny, nz, c->nv});
         if (dalloc(&c->ict_xch, c->ict_xch_bytes) != cudaSuccess ||
@@ -1723,6 +1751,7 @@ void batch_apply_fraction(fm_batch* b) {
         const int icb = std::max(1, std::min(c->ntiles, std::min(c->occ_icb, batch_icb(b)) * c->nsm));
         c->grid_icb = std::max(1, (int)std::lround(icb * b->fraction));
         if (c->base_ict) c->grid_ict = std::max(1, (int)std::lround(c->base_ict * b->fraction));
+        if (c->base_ictl) c->grid_ictl = std::max(1, (int)std::lround(c->base_ictl * b->fraction));
         if (c->base_ictg) c->grid_ictg = std::max(1, (int)std::lround(c->base_ictg * b->fraction));
         if (c->gexec) { cudaGraphExecDestroy(c->gexec); c->gexec = nullptr; }
     }

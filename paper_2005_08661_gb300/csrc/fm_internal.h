@@ -409,8 +409,8 @@ struct IcArgs {
 // (each pointing to an earlier voxel in natural order): factor planes, each [nv] double:
 // plane 0 = 1 / L_ii, plane 1 + h = L_{i,i+o_h}, plane 1 + nh = the substitution vector.
 // The first six offsets are always IC(0)'s (-1,0,0), (0,-1,0), (0,0,-1) and the level-1 fill
-// offsets (1,-1,0), (1,0,-1), (0,1,-1); with exactly those the sweeps take the row wavefront,
-// with more (fill the tolerance keeps beyond level 1) the table-driven level sweeps.
+// offsets (1,-1,0), (1,0,-1), (0,1,-1); with exactly those the sweeps take the row wavefront or the
+// unrolled level sweeps, with more (fill the tolerance keeps beyond level 1) the table-driven level sweeps.
 constexpr int kIctBaseOffsets = 6;
 constexpr int kIctPlanes = kIctBaseOffsets + 2;
 constexpr int kIctMaxOffsets = 64;  // largest held pattern; beyond it the call reports FM_ERR_FILL
@@ -519,6 +519,8 @@ template <typename T> cudaError_t launch_wf_sweep(const AdjArgs& a, int nsweep, 
                                                   cudaStream_t s);
 template <typename T> cudaError_t launch_wf_amp(const AdjArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_ict_tau(const DataArgs& a, double droptol, int grid, cudaStream_t s);
+template <typename T> cudaError_t launch_ict_fwd(const IctArgs& a, int grid, int block, cudaStream_t s);
+template <typename T> cudaError_t launch_ict_bwd(const IctArgs& a, int grid, int block, cudaStream_t s);
 template <typename T> cudaError_t launch_ictw_fwd(const IctArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_ictw_bwd(const IctArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_ictw_rows(const Geo& geo, const uint8_t* nb, int4* rows, cudaStream_t s);
@@ -527,6 +529,7 @@ size_t ictw_exchange_bytes(const Geo& geo);  // its exchange buffer
 template <typename T> cudaError_t launch_ict_check(const IctArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_ictg_fwd(const IctArgs& a, int grid, int block, cudaStream_t s);
 template <typename T> cudaError_t launch_ictg_bwd(const IctArgs& a, int grid, int block, cudaStream_t s);
+template <typename T> int ict_max_blocks_per_sm(int block);
 template <typename T> int ictg_max_blocks_per_sm(int block);
 template <typename T> int ic_tz();
 template <typename T> size_t ic_face_bytes_per_tile();

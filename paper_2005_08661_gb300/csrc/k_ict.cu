@@ -22,7 +22,8 @@
 // wavefront does not apply.  With level t = x + 2y + 3z every offset in P points to a strictly
 // lower level (t(a) = t(d) = t(f) = -1, t(b) = t(e) = -2, t(c) = -3).  Groups of 32 rows walk along x, a
 // lane two steps behind the lane below, and hand their records on as they go ("row wavefront"
-// below); the back substitution is the walk mirrored.  The factor stores 1 / L_ii, so every entry
+// below), or, where planes follow each other faster that way, a grid barrier separates the levels
+// ("level sweeps"); the back substitution is the walk mirrored.  The factor stores 1 / L_ii, so every entry
 // costs a multiply.
 //
 // Deeper fill.  When the tolerance keeps entries beyond level 1, the pattern P grows: the host
@@ -137,6 +138,149 @@ __device__ __forceinline__ bool level_sync(const IctArgs& a) {
     return grid_barrier(a.istate, a.spin_limit);
 }
 
+// ------------------------------------------------------------------ level sweeps (base pattern)
+//
+// For volumes whose planes follow each other faster by levels than by rows (ict_form), and those without
+// the row wavefront's buffer: thread <-> (y, z) column, voxel x = t - 2y - 3z, a barrier between the levels
+// t = x + 2y + 3z.  A level is FP64 arithmetic on the active columns, so the blocks are sized to spread the
+// columns over every SM (a volume with few columns runs one-warp blocks).  Each row issues all of its
+// loads from the earlier rows before the dependency chain starts.
+
+template <typename T>
+__global__ void __launch_bounds__(kIctThreads) k_ict_fwd(IctArgs a) {
+    const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
+    const long long nxy = (long long)nx * ny, nv = a.geo.nv;
+    double* Lp = a.L;
+    auto P = [&](int k, long long j) -> double* { return Lp + (size_t)k * nv + j; };
+    const T* d = (const T*)a.d;
+    const T* g = (const T*)a.g;
+    T* ipo = (T*)a.ip_out;
+    const bool factor = d != nullptr;
+    const double beta = a.beta;
+    const double tau = factor ? a.scal[S_ICT_TAU] : 0.0;
+    const int npair = ny * nz;
+    const int tmax = (nx - 1) + 2 * (ny - 1) + 3 * (nz - 1);
+    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
+    bool bad = false;
+    for (int t = 0; t <= tmax; ++t) {
+        for (int pr = gtid; pr < npair; pr += nthr) {
+            const int y = pr % ny, z = pr / ny, x = t - 2 * y - 3 * z;
+            if (x < 0 || x >= nx) continue;
+            const long long i = x + (long long)nx * y + nxy * z;
+            const uint8_t b = a.nb[i];
+            if (!(b & NB_IN)) continue;
+            const long long ja = i - 1, jb = i - nx, jc = i - nxy, jd = i + 1 - nx, je = i + 1 - nxy, jf = i + nx - nxy;
+            const bool ha = b & NB_XM, hb = b & NB_YM, hc = b & NB_ZM;
+            const bool hd = x + 1 < nx && y > 0 && (a.nb[jd] & NB_IN);
+            const bool he = x + 1 < nx && z > 0 && (a.nb[je] & NB_IN);
+            const bool hf = y + 1 < ny && z > 0 && (a.nb[jf] & NB_IN);
+            auto ld = [&](bool h, int k, long long j) { return h ? ld_level(P(k, j)) : 0.0; };
+            // every value from the earlier rows first (independent loads), then the chain
+            const double yc = ld(hc, PL_Y, jc), ye = ld(he, PL_Y, je), yf = ld(hf, PL_Y, jf),
+                         yb = ld(hb, PL_Y, jb), yd = ld(hd, PL_Y, jd), ya = ld(ha, PL_Y, ja);
+            double la, lb, lc, l_d, le, lf, rii;
+            if (factor) {
+                const double rc = ld(hc, PL_R, jc), re = ld(he, PL_R, je), rf = ld(hf, PL_R, jf),
+                             rb = ld(hb, PL_R, jb), rd = ld(hd, PL_R, jd), ra = ld(ha, PL_R, ja);
+                const double e_a = ld(he, PL_A, je), f_b = ld(hf, PL_B, jf), f_d = ld(hf, PL_D1, jf),
+                             b_f = ld(hb, PL_F, jb), d_a = ld(hd, PL_A, jd), d_f = ld(hd, PL_F, jd),
+                             a_d = ld(ha, PL_D1, ja), a_e = ld(ha, PL_E, ja);
+                auto keep = [&](bool h, double v) { return h && fabs(v) >= tau ? v : 0.0; };
+                lc = keep(hc, -beta * rc);
+                le = keep(he, -(lc * e_a) * re);
+                lf = keep(hf, -(lc * f_b + le * f_d) * rf);
+                lb = keep(hb, (-beta - lc * b_f) * rb);
+                l_d = keep(hd, -(lb * d_a + le * d_f) * rd);
+                la = keep(ha, (-beta - lb * a_d - lc * a_e) * ra);
+                const double h = (double)d[i] + beta * (double)__popc((unsigned)(b >> 1) & 0x3fu);
+                const double s = h - (((la * la + lb * lb) + (lc * lc + l_d * l_d)) + (le * le + lf * lf));
+                if (!(s > 0.0)) bad = true;
+                rii = s > 0.0 ? rsqrt_nr(s) : 1.0;  // the error is reported; keep the arithmetic finite
+                *P(PL_R, i) = rii;
+                *P(PL_A, i) = la;
+                *P(PL_B, i) = lb;
+                *P(PL_C, i) = lc;
+                *P(PL_D1, i) = l_d;
+                *P(PL_E, i) = le;
+                *P(PL_F, i) = lf;
+                if (ipo) ipo[i] = (T)(rii * rii);
+            } else {
+                rii = *P(PL_R, i);
+                la = *P(PL_A, i);
+                lb = *P(PL_B, i);
+                lc = *P(PL_C, i);
+                l_d = *P(PL_D1, i);
+                le = *P(PL_E, i);
+                lf = *P(PL_F, i);
+            }
+            const double acc = (double)g[i] - ((lc * yc + le * ye) + (lf * yf + lb * yb) + (l_d * yd + la * ya));
+            *P(PL_Y, i) = acc * rii;
+        }
+        if (t < tmax && !level_sync(a)) return;
+    }
+    // reported by the back sweep, after k_ict_check: fill beyond the held pattern (which can
+    // itself make a pivot of the restricted factor non-positive) takes precedence
+    if (bad) atomicExch(a.istate + I_ICT_BAD, 1);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kIctThreads) k_ict_bwd(IctArgs a) {
+    __shared__ double sbuf[2 * 32];
+    const int nx = a.geo.nx, ny = a.geo.ny, nz = a.geo.nz;
+    const long long nxy = (long long)nx * ny, nv = a.geo.nv;
+    double* Lp = a.L;
+    auto P = [&](int k, long long j) -> double* { return Lp + (size_t)k * nv + j; };
+    T* p = (T*)a.p;
+    const T* gd = (const T*)a.gdot;
+    const T* gpd = (const T*)a.gpdot;
+    const int npair = ny * nz;
+    const int tmax = (nx - 1) + 2 * (ny - 1) + 3 * (nz - 1);
+    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
+    double acc2[2] = {0.0, 0.0};
+    if (blockIdx.x == 0 && threadIdx.x == 0 && a.istate[I_ICT_BAD]) {
+        set_err(a.istate, FM_ERR_NOT_PD);
+        a.istate[I_ICT_BAD] = 0;
+    }
+    for (int t = tmax; t >= 0; --t) {
+        for (int pr = gtid; pr < npair; pr += nthr) {
+            const int y = pr % ny, z = pr / ny, x = t - 2 * y - 3 * z;
+            if (x < 0 || x >= nx) continue;
+            const long long i = x + (long long)nx * y + nxy * z;
+            const uint8_t b = a.nb[i];
+            if (!(b & NB_IN)) {
+                p[i] = T(0);
+                continue;
+            }
+            // the later rows r = i - o that hold an entry in column i: L_{r,i} = plane o of row r
+            const long long ra = i + 1, rb = i + nx, rc = i + nxy, rd = i - 1 + nx, re = i - 1 + nxy, rf = i - nx + nxy;
+            const bool ha = b & NB_XP, hb = b & NB_YP, hc = b & NB_ZP;
+            const bool hd = x > 0 && y + 1 < ny && (a.nb[rd] & NB_IN);
+            const bool he = x > 0 && z + 1 < nz && (a.nb[re] & NB_IN);
+            const bool hf = y > 0 && z + 1 < nz && (a.nb[rf] & NB_IN);
+            auto ld = [&](bool h, int k, long long j) { return h ? ld_level(P(k, j)) : 0.0; };
+            const double s = *P(PL_Y, i) - ((ld(ha, PL_A, ra) * ld(ha, PL_Y, ra) + ld(hd, PL_D1, rd) * ld(hd, PL_Y, rd)) +
+                                            (ld(hf, PL_F, rf) * ld(hf, PL_Y, rf) + ld(hb, PL_B, rb) * ld(hb, PL_Y, rb)) +
+                                            (ld(he, PL_E, re) * ld(he, PL_Y, re) + ld(hc, PL_C, rc) * ld(hc, PL_Y, rc)));
+            const double xi = s * *P(PL_R, i);
+            *P(PL_Y, i) = xi;  // y_i becomes x_i: every row that still needs y_i is this one
+            p[i] = (T)xi;
+            if (gd) acc2[0] += (double)gd[i] * (double)(T)xi;
+            if (gpd) acc2[1] += (double)gpd[i] * (double)(T)xi;
+        }
+        if (t > 0 && !level_sync(a)) return;
+    }
+    if (gd || gpd) {
+        double out[2];
+        if (last_block_reduce<2>(acc2, a.partials, (unsigned*)(a.istate + I_DONE0), out, sbuf)) {
+            if (threadIdx.x == 0) {
+                a.scal[S_GP] = out[0];
+                a.scal[S_GPREVP] = out[1];
+                if (!isfinite(out[0]) || !isfinite(out[1])) set_err(a.istate, FM_ERR_NONFINITE);
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------ row wavefront (base pattern)
 //
 // The two substitutions of the base pattern without level barriers.  A one-warp block holds 32
@@ -157,7 +301,7 @@ __device__ __forceinline__ bool level_sync(const IctArgs& a) {
 // A step is a chain of FP64 operations (one warp per SM: 16 cycles an operation), a block runs as
 // far behind plane z-1 as the hand-off takes, and no barrier is left: 74 x 74 x 10 voxels, 32 coils,
 // factor + forward 1012 -> 606 us, back substitution 904 -> 254; the level sweeps pay about 4 us on
-// each of 247 levels.  They stay for grown patterns (table-driven), whose offsets reach further.
+// each of 247 levels.
 
 constexpr int kRec = 6;  // doubles of a record: R, Y, A, B, D, F (1/L_ii, y and the entries others use)
 
@@ -643,9 +787,8 @@ __device__ __forceinline__ long long ict_nbr(const IctArgs& a, int x, int y, int
     return (a.nb[j] & NB_IN) ? j : -1;
 }
 
-// The factorisation and substitutions for any held pattern (a.tb) -- grown ones, and the base
-// pattern of volumes whose rows make the wavefront's exchange buffer too large (fm_create): row i's entries in increasing column order, L_{i,j} = (H_ij - sum over the pairs
-// (p1, p2) of o of L_{i,i+o_p1} L_{j,j+o_p2}) / L_jj, dropped below tau, then L_ii and y_i.
+// The factorisation and substitutions for any held pattern (a.tb), used for the grown ones: row i's
+// entries in increasing column order, L_{i,j} = (H_ij - sum over the pairs (p1, p2) of o of L_{i,i+o_p1} L_{j,j+o_p2}) / L_jj, dropped below tau, then L_ii and y_i.
 // Level t = x + B y + C z, with B and C chosen by the host so that every held offset points
 // to a strictly lower level.
 template <typename T>
@@ -825,6 +968,14 @@ int ictg_max_blocks_per_sm(int block) {
 }
 
 template <typename T>
+int ict_max_blocks_per_sm(int block) {
+    int f = 0, b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f, k_ict_fwd<T>, block, 0) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_ict_bwd<T>, block, 0) != cudaSuccess) return 0;
+    return f < b ? f : b;
+}
+
+template <typename T>
 cudaError_t launch_ict_tau(const DataArgs& a, double droptol, int grid, cudaStream_t s) {
     k_ict_tau<T><<<grid, kThreads, 0, s>>>(a, droptol);
     return cudaGetLastError();
@@ -852,6 +1003,18 @@ size_t ictw_exchange_bytes(const Geo& geo) {
 // cooperative launch guarantees that (or refuses the launch) even when other kernels run
 // beside the sweep, e.g. the other volumes' branches of a batched graph.
 template <typename T>
+cudaError_t launch_ict_fwd(const IctArgs& a, int grid, int block, cudaStream_t s) {
+    IctArgs copy = a;
+    void* args[] = {&copy};
+    return cudaLaunchCooperativeKernel((const void*)k_ict_fwd<T>, dim3(grid), dim3(block), args, 0, s);
+}
+template <typename T>
+cudaError_t launch_ict_bwd(const IctArgs& a, int grid, int block, cudaStream_t s) {
+    IctArgs copy = a;
+    void* args[] = {&copy};
+    return cudaLaunchCooperativeKernel((const void*)k_ict_bwd<T>, dim3(grid), dim3(block), args, 0, s);
+}
+template <typename T>
 cudaError_t launch_ictg_fwd(const IctArgs& a, int grid, int block, cudaStream_t s) {
     IctArgs copy = a;
     void* args[] = {&copy};
@@ -874,8 +1037,11 @@ cudaError_t launch_ict_check(const IctArgs& a, int grid, cudaStream_t s) {
     template cudaError_t launch_ictw_fwd<T>(const IctArgs&, int, cudaStream_t);         \
     template cudaError_t launch_ictw_bwd<T>(const IctArgs&, int, cudaStream_t);         \
     template cudaError_t launch_ict_check<T>(const IctArgs&, int, cudaStream_t);        \
+    template cudaError_t launch_ict_fwd<T>(const IctArgs&, int, int, cudaStream_t);     \
+    template cudaError_t launch_ict_bwd<T>(const IctArgs&, int, int, cudaStream_t);     \
     template cudaError_t launch_ictg_fwd<T>(const IctArgs&, int, int, cudaStream_t);    \
     template cudaError_t launch_ictg_bwd<T>(const IctArgs&, int, int, cudaStream_t);    \
+    template int ict_max_blocks_per_sm<T>(int);                                         \
     template int ictg_max_blocks_per_sm<T>(int);
 FM_ICT_INST(float)
 FM_ICT_INST(double)
