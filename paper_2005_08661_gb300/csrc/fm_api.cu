@@ -897,6 +897,20 @@ int implicit_t(fm_ctx* c, const void* y, const void* smap, const void* w_hat, co
 #define FM_IC_BZ 1
 #endif
 
+TileLists tile_lists(fm_ctx* c) {
+    TileLists t;
+    t.ntx = c->ntx;
+    t.nty = c->nty;
+    t.ntiles = c->ntiles;
+    t.order = c->order;
+    t.range = c->tile_rng;
+    t.out = c->order_act;
+    t.istate = c->istate;
+    t.tile_part = c->tile_part;
+    t.npart = c->npart;
+    return t;
+}
+
 // Tile claim orders: a weighted tile hyperplane wxy (4 X + Y) + 2 wz Z (ties: z, y, x), for tiles of
 // 64 x 16 x 8.  Every weight is positive, so a tile's -x, -y, -z neighbours always come first.  Both
 // sweeps stream faces, and a tile starts 63, 15 and 16 steps plus one hand-off behind its x, y and
@@ -920,7 +934,7 @@ bool set_ic_order(fm_ctx* c, int wxy, int wz) {
     c->ic_wz = wz;
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;  // launches that read the order are done
     if (cudaMemcpy(c->order, ord.data(), ord.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return false;
-    return !c->have_data || launch_ic_order(c->order, c->tile_rng, c->ntx, c->nty, c->ntiles, c->order_act, c->istate, c->stream) == cudaSuccess;
+    return !c->have_data || c->o.precond == FM_PC_ICT || launch_ic_order(tile_lists(c), c->stream) == cudaSuccess;
 }
 
 // Cooperative line-search grid: every block must be co-resident, so the grid follows the
@@ -1265,16 +1279,12 @@ int fm_set_data(fm_ctx* c, const void* y, const void* smap, const double* te, co
     a.partials = c->partials;
     a.scal = c->scal;
     a.istate = c->istate;
+    if (c->o.precond != FM_PC_ICT) a.tiles = tile_lists(c);
+    a.ict_rows = c->ict_rows;
+    a.ict_units = c->ict_rows ? ictw_units(a.geo) : 0;
     cudaError_t e = c->o.precision == FM_FP64 ? launch_setup<double>(a, c->stream)
                                               : launch_setup<float>(a, c->stream);
-    if (e == cudaSuccess) e = launch_ic_ranges(a.geo, c->ntx, c->nty, c->ntiles, c->nb, c->tile_rng, c->stream);
-    if (e == cudaSuccess) e = launch_ic_order(c->order, c->tile_rng, c->ntx, c->nty, c->ntiles, c->order_act, c->istate, c->stream);
-    if (e == cudaSuccess && c->ict_rows) e = launch_ictw_rows(a.geo, c->nb, c->ict_rows, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "setup kernel");
-    // the IC sweeps leave out tiles outside the mask: their inverse pivots and their part of the dot
-    // products are 0
-    FM_CK(cudaMemsetAsync(c->tile_part, 0, 2 * (size_t)c->npart * sizeof(double), c->stream), "clear sums");
-    FM_CK(cudaMemsetAsync(c->ip, 0, (size_t)c->nv * c->ts, c->stream), "clear pivots");
     // rows outside the new mask must read as empty in the drop-tolerance factor
     if (c->ict_L)
         FM_CK(cudaMemsetAsync(c->ict_L, 0, (size_t)c->ict_nplanes * c->nv * sizeof(double), c->stream), "clear factor");
@@ -1344,8 +1354,9 @@ int ic_factor_from_d(fm_ctx* c, void* inv_pivot) {
             if (e != cudaSuccess) return cuda_fail(c, e, "IC kernels");
         }
     }
-    if (inv_pivot)
-        FM_CK(cudaMemcpyAsync(inv_pivot, c->ip, (size_t)c->nv * c->ts, cudaMemcpyDeviceToDevice, c->stream), "copy");
+    if (inv_pivot)  // the sweeps leave out what lies outside the mask
+        FM_CK(f64 ? launch_masked_copy<double>(c->ip, inv_pivot, c->nb, c->nv, c->grid_data, c->stream)
+                  : launch_masked_copy<float>(c->ip, inv_pivot, c->nb, c->nv, c->grid_data, c->stream), "copy");
     c->have_factor = true;
     return FM_OK;
 }
@@ -1406,7 +1417,7 @@ int fm_ic_factor64(fm_ctx* c, const void* omega, double* inv_pivot) {
     FM_CK(run_grad<float>(c, omega, nullptr, c->w[0], c->g[0], c->d, nullptr), "gradient kernel");
     FM_CK(cudaMemsetAsync(c->ip_lo, 0, (size_t)c->nv * sizeof(float), c->stream), "clear");
     FM_CK(run_ic0<float>(c, c->d, c->g[0], c->p, nullptr, nullptr, -1, c->ip_lo), "IC(0) kernels");
-    FM_CK(launch_inv_pivot64((const float*)c->ip, c->ip_lo, inv_pivot, c->nv, c->grid_data, c->stream), "combine");
+    FM_CK(launch_inv_pivot64((const float*)c->ip, c->ip_lo, inv_pivot, c->nb, c->nv, c->grid_data, c->stream), "combine");
     c->have_factor = true;
     return FM_OK;
 }

@@ -314,6 +314,19 @@ struct Geo {
     long long nv;
 };
 
+// Tiles of the IC(0) sweeps: their steps that reach a mask voxel, a byte each (first and last of the forward
+// sweep, first and last of the back substitution; an empty tile has first 255, last 0), and the lists of the
+// tiles that hold any (ic_tiles.h).
+struct TileLists {
+    int ntx, nty, ntiles;  // ntiles 0: none kept (a context that runs no IC(0) sweeps)
+    const int* order;      // [2][ntiles] claim orders of all tiles: forward, back substitution
+    unsigned* range;       // [ntiles]
+    int* out;              // [3][ntiles]
+    int* istate;
+    double* tile_part;     // [2][npart] dot products by place, 0 where no tile stands for them
+    int npart;
+};
+
 struct SetupArgs {
     Geo geo;
     int nc, L;
@@ -331,6 +344,9 @@ struct SetupArgs {
     void* w0;           // T [nv] initial field map (Eq. 6)
     int* vlist;         // [nv] voxel index of each mask voxel, ascending (compact order)
     int* chunk_off;     // [nchunks] mask voxels before each chunk (exclusive scan)
+    TileLists tiles;
+    int4* ict_rows;     // [ict_units] row groups of the drop-tolerance wavefront, or null
+    int ict_units;
     double* partials;   // [nchunks]
     double* scal;
     int* istate;
@@ -501,13 +517,11 @@ template <typename T> int ls_max_blocks_per_sm(const DataArgs& a);
 int data_lanes(const DataArgs& a);  // FP32: most lanes that share a voxel in the data-term kernels
 template <typename T> cudaError_t launch_rb_black(const DataArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_rb_red(const DataArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, unsigned* range,
-                             cudaStream_t s);
-cudaError_t launch_ic_order(const int* order, const unsigned* range, int ntx, int nty, int ntiles, int* out, int* istate,
-                            cudaStream_t s);
+cudaError_t launch_ic_order(const TileLists& a, cudaStream_t s);
 template <typename T> cudaError_t launch_ic_fwd(const IcArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_ic_bwd(const IcArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_inv_pivot64(const float* hi, const float* lo, double* out, long long nv, int grid, cudaStream_t s);
+cudaError_t launch_inv_pivot64(const float* hi, const float* lo, double* out, const uint8_t* nb, long long nv, int grid,
+                               cudaStream_t s);
 template <typename T> cudaError_t launch_true_curv(const AdjArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_cg_init(const AdjArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_cg_dir(const AdjArgs& a, int grid, cudaStream_t s);
@@ -523,7 +537,6 @@ template <typename T> cudaError_t launch_ict_fwd(const IctArgs& a, int grid, int
 template <typename T> cudaError_t launch_ict_bwd(const IctArgs& a, int grid, int block, cudaStream_t s);
 template <typename T> cudaError_t launch_ictw_fwd(const IctArgs& a, int grid, cudaStream_t s);
 template <typename T> cudaError_t launch_ictw_bwd(const IctArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_ictw_rows(const Geo& geo, const uint8_t* nb, int4* rows, cudaStream_t s);
 int ictw_units(const Geo& geo);               // row groups of the drop-tolerance wavefront
 size_t ictw_exchange_bytes(const Geo& geo);  // its exchange buffer
 template <typename T> cudaError_t launch_ict_check(const IctArgs& a, int grid, cudaStream_t s);

@@ -42,8 +42,8 @@
 //
 // Support mask.  A voxel outside the mask has 1/pi = v = p = 0 whatever its neighbours hold, so
 // the sweeps leave out what the mask leaves empty.  fm_set_data records, per tile, the first
-// and last step of each sweep that reaches a mask voxel (k_ic_range) and lists the tiles that hold
-// any (k_ic_order).  Only listed tiles are claimed, a tile sweeps its own steps only, and
+// and last step of each sweep that reaches a mask voxel and lists the tiles that hold any
+// (ic_tiles.h).  Only listed tiles are claimed, a tile sweeps its own steps only, and
 // a face entry is handed over only where the producer's and the consumer's steps both
 // reach it (both sides evaluate the same test); every other incoming entry is 0.  An ellipsoid
 // mask fills a quarter of its grid, and the chain through it is about half as long as the
@@ -63,6 +63,7 @@
 #include <type_traits>
 
 #include "fm_internal.h"
+#include "ic_tiles.h"
 
 namespace fm {
 
@@ -158,38 +159,6 @@ __device__ __forceinline__ void cp_wait_all() {
 
 // ------------------------------------------------------------------ tile geometry
 
-#ifndef FM_IC_CSF
-#define FM_IC_CSF 4
-#endif
-#ifndef FM_IC_CSB
-#define FM_IC_CSB 4
-#endif
-#ifndef FM_IC_FWF
-#define FM_IC_FWF 2
-#endif
-#ifndef FM_IC_FWB
-#define FM_IC_FWB 3
-#endif
-constexpr int kTX = kTileX, kTY = kTileY, kTZ = 8;  // 64 x 16 x 8 voxels
-constexpr int kRows = kTY * kTZ;                     // rows along x: one per compute thread
-constexpr int kWarps = kRows / 32;                   // compute warps, two z planes each
-constexpr int kVox = kTX * kRows;
-static_assert(kTX == 64 && kTY == 16 && kWarps == 4, "lane = (y, plane of the warp's pair)");
-// Steps per chunk (the unit of the face hand-off, of the barrier between the warps and of
-// their lag), and the warps that fetch incoming faces, taking the chunks in turn, so that the
-// polls for consecutive chunks are in flight together (a poll round trip is about 0.7 us, a chunk
-// 0.2 to 0.4).  Forward / back substitution on 256 x 256 x 128 (us): chunks of 4 with 2 fetch warps
-// 122 / 97, with 3 125 / 98, with 4 127 / 103; chunks of 3 with 3 130 / 95, of 2 with 4 146 / 101,
-// of 6 with 2 126 / 104.
-constexpr int kCSF = FM_IC_CSF, kCSB = FM_IC_CSB;
-constexpr int kFetchF = FM_IC_FWF, kFetchB = FM_IC_FWB;
-// compute warps, one warp that publishes the outgoing faces, fetch warps
-constexpr int kThreadsF = kRows + 32 + 32 * kFetchF, kThreadsB = kRows + 32 + 32 * kFetchB;
-constexpr int kSweep = kRows + 32;  // threads that meet at the end of a chunk: compute and publishing warps
-
-// First step of plane lz with chunks of C steps: the two planes of a warp follow each other by
-// one step, and each warp starts C + 1 steps after the warp below.
-template <int C> __host__ __device__ constexpr int tz(int lz) { return (C + 1) * (lz >> 1) + (lz & 1); }
 template <int C> struct Steps {
     static constexpr int n = kTX + kTY - 1 + tz<C>(kTZ - 1), chunks = (n + C - 1) / C;
     static_assert(n < 255 && chunks <= 64, "steps in a byte, chunks in a mask");
@@ -273,69 +242,8 @@ __device__ __forceinline__ Range tile_range(const unsigned* range, int tile) {
     return {(int)(r & 255u), (int)(r >> 8 & 255u)};
 }
 
-// One block per tile, one thread per row.
-__global__ void __launch_bounds__(kRows) k_ic_range(Geo geo, int ntx, int nty, const uint8_t* nb, unsigned* range) {
-    __shared__ int s_lim[4];
-    const int tile = blockIdx.x, X = tile % ntx, Y = (tile / ntx) % nty, Z = tile / (ntx * nty);
-    const int ly = threadIdx.x % kTY, lz = threadIdx.x / kTY;
-    const int y = Y * kTY + ly, z = Z * kTZ + lz, x0 = X * kTX;
-    if (threadIdx.x < 4) s_lim[threadIdx.x] = (threadIdx.x & 1) ? 0 : 255;
-    __syncthreads();
-    if (y < geo.ny && z < geo.nz) {
-        const uint8_t* row = nb + ((long long)z * geo.ny + y) * geo.nx + x0;
-        const int n = min(kTX, geo.nx - x0);
-        int lo = 255, hi = -1;
-        for (int i = 0; i < n; ++i)
-            if (row[i] & NB_IN) {
-                lo = min(lo, i);
-                hi = i;
-            }
-        if (hi >= 0) {
-            const int f = ly + tz<kCSF>(lz), b = (kTY - 1 - ly) + tz<kCSB>(kTZ - 1 - lz);
-            atomicMin(&s_lim[0], lo + f);
-            atomicMax(&s_lim[1], hi + f);
-            atomicMin(&s_lim[2], kTX - 1 - hi + b);
-            atomicMax(&s_lim[3], kTX - 1 - lo + b);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        range[tile] = (unsigned)s_lim[0] | (unsigned)s_lim[1] << 8 | (unsigned)s_lim[2] << 16 | (unsigned)s_lim[3] << 24;
-}
-
-// Lists in claim order, one block each: block 0 the non-empty tiles of the forward order
-// (order[0..ntiles)), block 1 those of the back substitution's (order[ntiles..)), and block 2, in
-// the same order, the tiles that stand for a dot-product unit: a unit is a pair of tiles Y = 2k,
-// 2k + 1 and belongs to the lower one (the later of the two to be swept back) if that is not empty.
-__global__ void __launch_bounds__(1024) k_ic_order(const int* order, const unsigned* range, int ntx, int nty, int ntiles,
-                                                   int* out, int* istate) {
-    __shared__ int s_warp[32], s_base;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int* in = order + (blockIdx.x == 0 ? 0 : ntiles);
-    out += (size_t)blockIdx.x * ntiles;
-    auto empty = [&](int t) { return (range[t] & 255u) == 255u; };
-    if (threadIdx.x == 0) s_base = 0;
-    __syncthreads();
-    for (int b = 0; b < ntiles; b += 1024) {
-        const int i = b + threadIdx.x;
-        const int t = i < ntiles ? in[i] : -1;
-        bool keep = t >= 0 && !empty(t);
-        if (blockIdx.x == 2 && keep && ((t / ntx) % nty & 1)) keep = empty(t - ntx);
-        const unsigned bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) s_warp[wid] = __popc(bal);
-        __syncthreads();
-        int at = s_base, tot = 0;
-        for (int w = 0; w < 32; ++w) {
-            if (w < wid) at += s_warp[w];
-            tot += s_warp[w];
-        }
-        if (keep) out[at + __popc(bal & ((1u << lane) - 1u))] = t;
-        __syncthreads();
-        if (threadIdx.x == 0) s_base += tot;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && blockIdx.x != 1) istate[blockIdx.x == 0 ? I_NTILE : I_NUNIT] = s_base;
-}
+// The lists anew, for another claim order of the same mask.
+__global__ void __launch_bounds__(1024) k_ic_order(TileLists a) { list_tiles(a, blockIdx.x); }
 
 // ------------------------------------------------------------------ streamed faces
 //
@@ -1014,14 +922,8 @@ __global__ void __launch_bounds__(kThreadsB, sizeof(T) == 4 ? 2 : 1) k_ic_bwd(Ic
     }
 }
 
-cudaError_t launch_ic_ranges(const Geo& geo, int ntx, int nty, int ntiles, const uint8_t* nb, unsigned* range,
-                             cudaStream_t s) {
-    k_ic_range<<<ntiles, kRows, 0, s>>>(geo, ntx, nty, nb, range);
-    return cudaGetLastError();
-}
-cudaError_t launch_ic_order(const int* order, const unsigned* range, int ntx, int nty, int ntiles, int* out, int* istate,
-                            cudaStream_t s) {
-    k_ic_order<<<3, 1024, 0, s>>>(order, range, ntx, nty, ntiles, out, istate);
+cudaError_t launch_ic_order(const TileLists& a, cudaStream_t s) {
+    k_ic_order<<<3, 1024, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1086,14 +988,15 @@ cudaError_t launch_ic_bwd(const IcArgs& a, int grid, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// 1/pi = hi + lo as one double (FP32 mode's pivot pair, for inspection)
-__global__ void k_inv_pivot64(const float* hi, const float* lo, double* out, long long nv) {
+// 1/pi = hi + lo as one double (FP32 mode's pivot pair, for inspection), 0 outside the mask
+__global__ void k_inv_pivot64(const float* hi, const float* lo, double* out, const uint8_t* nb, long long nv) {
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < nv; j += (long long)gridDim.x * blockDim.x)
-        out[j] = (double)hi[j] + (double)lo[j];
+        out[j] = nb[j] & NB_IN ? (double)hi[j] + (double)lo[j] : 0.0;
 }
 
-cudaError_t launch_inv_pivot64(const float* hi, const float* lo, double* out, long long nv, int grid, cudaStream_t s) {
-    k_inv_pivot64<<<grid, kThreads, 0, s>>>(hi, lo, out, nv);
+cudaError_t launch_inv_pivot64(const float* hi, const float* lo, double* out, const uint8_t* nb, long long nv, int grid,
+                               cudaStream_t s) {
+    k_inv_pivot64<<<grid, kThreads, 0, s>>>(hi, lo, out, nb, nv);
     return cudaGetLastError();
 }
 

@@ -381,28 +381,6 @@ __device__ __forceinline__ Span ictw_span(const int4* rows, bool there, int u, b
     return fwd ? Span{r.x, r.y} : Span{r.z, r.w};
 }
 
-// First and last step of every row group, forward (x + 2 lane) and mirrored (nx - 1 - x + 2 (31 - lane)).
-__global__ void __launch_bounds__(32) k_ictw_rows(Geo geo, const uint8_t* nb, int4* rows) {
-    const IctwGeo w = ictw_geo(geo);
-    const int u = blockIdx.x, z = u / w.nyb, y = (u % w.nyb) * 32 + threadIdx.x, l = threadIdx.x;
-    int lo = 1 << 30, hi = -(1 << 30), lo2 = lo, hi2 = hi;
-    if (y < geo.ny) {
-        const uint8_t* row = nb + ((long long)z * geo.ny + y) * geo.nx;
-        for (int x = 0; x < geo.nx; ++x)
-            if (row[x] & NB_IN) {
-                lo = min(lo, x + 2 * l);
-                hi = x + 2 * l;
-                hi2 = max(hi2, geo.nx - 1 - x + 2 * (31 - l));
-                lo2 = geo.nx - 1 - x + 2 * (31 - l);
-            }
-    }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    lo2 = __reduce_min_sync(0xffffffffu, lo2);
-    hi2 = __reduce_max_sync(0xffffffffu, hi2);
-    if (l == 0) rows[u] = make_int4(lo, hi, lo2, hi2);
-}
-
 // Exchange buffer: plane records [unit][step][lane] of kRec doubles, then edge records
 // [unit][step][2] (0: the first lane's for the group below in the next plane, 1: the last lane's for
 // the next group) of kRec doubles.  The substitution-only walks use the first two doubles.
@@ -989,10 +967,6 @@ cudaError_t launch_ictw_fwd(const IctArgs& a, int grid, cudaStream_t s) {
 template <typename T>
 cudaError_t launch_ictw_bwd(const IctArgs& a, int grid, cudaStream_t s) {
     k_ictw_bwd<T><<<grid, 32, 0, s>>>(a);
-    return cudaGetLastError();
-}
-cudaError_t launch_ictw_rows(const Geo& geo, const uint8_t* nb, int4* rows, cudaStream_t s) {
-    k_ictw_rows<<<ictw_units(geo), 32, 0, s>>>(geo, nb, rows);
     return cudaGetLastError();
 }
 int ictw_units(const Geo& geo) { return (geo.ny + 31) / 32 * geo.nz; }

@@ -23,15 +23,24 @@
 // counts into exclusive offsets (single block, fixed order), and k_setup ranks each mask
 // voxel inside its chunk with warp ballots, so the compact order is the voxel order.
 #include "fm_internal.h"
+#include "ic_tiles.h"
 
 namespace fm {
 
 constexpr int kSetupThreads = 256;
 
-__device__ __forceinline__ bool in_mask(const uint8_t* mask, long long j) { return mask ? mask[j] != 0 : true; }
-
-__global__ void __launch_bounds__(kSetupThreads) k_mask_count(const uint8_t* mask, long long nv, int* counts) {
+// Mask voxels of a chunk; behind the chunks' blocks one for each IC(0) tile and each row group.
+__global__ void __launch_bounds__(kSetupThreads) k_mask_count(Geo geo, const uint8_t* mask, int* counts, int nchunks,
+                                                              TileLists tiles, int4* ict_rows) {
+    static_assert(kSetupThreads == 2 * kRows, "tile_steps, row_steps");
     __shared__ int warp_cnt[kSetupThreads / 32];
+    const long long nv = geo.nv;
+    if ((int)blockIdx.x >= nchunks) {
+        const int b = blockIdx.x - nchunks;
+        if (b < tiles.ntiles) tile_steps(geo, mask, tiles.ntx, tiles.nty, b, tiles.range);
+        else row_steps(geo, mask, b - tiles.ntiles, ict_rows);
+        return;
+    }
     const long long base = (long long)blockIdx.x * kChunk;
     int c = 0;
 #pragma unroll
@@ -51,10 +60,18 @@ __global__ void __launch_bounds__(kSetupThreads) k_mask_count(const uint8_t* mas
 }
 
 // Exclusive scan of counts[0..n) in place (one block of 1024 threads, tiles of 1024);
-// the total goes to *total.
-__global__ void __launch_bounds__(1024) k_chunk_scan(int* counts, int n, int* total) {
+// the total goes to *total.  Three more blocks list the IC(0) tiles, a fifth clears their dot products.
+__global__ void __launch_bounds__(1024) k_chunk_scan(int* counts, int n, int* total, TileLists tiles) {
     __shared__ int warp_sum[32];
     __shared__ int s_carry;
+    if (blockIdx.x == 4) {
+        for (int i = threadIdx.x; i < 2 * tiles.npart; i += blockDim.x) tiles.tile_part[i] = 0.0;
+        return;
+    }
+    if (blockIdx.x > 0) {
+        list_tiles(tiles, blockIdx.x - 1);
+        return;
+    }
     if (threadIdx.x == 0) s_carry = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -389,15 +406,30 @@ __global__ void __launch_bounds__(kSetupThreads) k_setup(SetupArgs a) {
 
 template <typename T>
 __global__ void __launch_bounds__(kSetupThreads) k_masked_copy(const T* in, T* out, const uint8_t* nb, long long nv) {
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < nv; j += (long long)gridDim.x * blockDim.x)
-        out[j] = (nb[j] & NB_IN) ? in[j] : T(0);
+    constexpr int U = 4;  // values in flight a thread, neither load behind the other
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long j0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; j0 < nv; j0 += U * stride) {
+        T v[U];
+        uint8_t b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long j = j0 + u * stride;
+            b[u] = j < nv ? nb[j] : (uint8_t)0;
+            v[u] = j < nv ? in[j] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long j = j0 + u * stride;
+            if (j < nv) out[j] = (b[u] & NB_IN) ? v[u] : T(0);
+        }
+    }
 }
 
 template <typename T>
 cudaError_t launch_setup(const SetupArgs& a, cudaStream_t s) {
     const int nchunks = (int)((a.geo.nv + kChunk - 1) / kChunk);
-    k_mask_count<<<nchunks, kSetupThreads, 0, s>>>(a.mask, a.geo.nv, a.chunk_off);
-    k_chunk_scan<<<1, 1024, 0, s>>>(a.chunk_off, nchunks, a.istate + I_NMASK);
+    k_mask_count<<<nchunks + a.tiles.ntiles + a.ict_units, kSetupThreads, 0, s>>>(a.geo, a.mask, a.chunk_off, nchunks, a.tiles, a.ict_rows);
+    k_chunk_scan<<<a.tiles.ntiles ? 5 : 1, 1024, 0, s>>>(a.chunk_off, nchunks, a.istate + I_NMASK, a.tiles);
     k_setup<T><<<nchunks, kSetupThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
