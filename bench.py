@@ -39,13 +39,14 @@ if ROOT not in sys.path:
 # kernel), from one ncu capture of the full workload (its summary sits with the committed
 # profiles), each with the hash of the kernel sources it was measured on: a figure whose
 # sources have changed since is reported as null.
-KERNEL_SOURCES = {"ls": ("k_data.cu",), "grad": ("k_data.cu",), "ic_fwd": ("k_ic.cu",), "ic_bwd": ("k_ic.cu",)}
+KERNEL_SOURCES = {"ls": ("k_data.cu",), "grad": ("k_data.cu",), "ic_fwd": ("k_ic.cu", "ic_tiles.h"),
+                  "ic_bwd": ("k_ic.cu", "ic_tiles.h")}
 NCU_TRAFFIC_BYTES = {  # (bytes per launch, kernel_src_hash of the sources measured)
-    ("full", "ls"): (2007300608 + 12793088, "4494fb0460a61f4d"),
-    ("full", "grad"): (506223872 + 27680256, "4494fb0460a61f4d"),
+    ("full", "ls"): (1964159232 + 31045888, "0aebc3b8267e27af"),
+    ("full", "grad"): (504923392 + 25731328, "0aebc3b8267e27af"),
     # the IC sweeps on the same 256x256x128 grid with one coil (their work does not depend on it)
-    ("full", "ic_fwd"): (79724800 + 37426688, "355df626ce512b8a"),
-    ("full", "ic_bwd"): (137366784 + 18694656, "355df626ce512b8a"),
+    ("full", "ic_fwd"): (40396544 + 2662912, "d4918ce19c2b3e74"),
+    ("full", "ic_bwd"): (64768768 + 2126080, "d4918ce19c2b3e74"),
 }
 
 

@@ -112,7 +112,7 @@ FM_API void fm_default_opts(fm_opts *opts);
  * (Sec. II: N_c >= 1, L >= 2).  opts may be NULL (defaults).  device is a CUDA
  * device ordinal; cuda_stream is a cudaStream_t of that device or NULL for the
  * legacy default stream.  Allocates every device buffer the solver needs (about
- * (8 N_c L + 80) bytes per voxel in FM_FP32 mode).  *out is NULL on failure.
+ * (8 N_c L + 90) bytes per voxel in FM_FP32 mode with three echoes).  *out is NULL on failure.
  * Errors: FM_ERR_ARG (sizes < 1, ncoil > FM_MAX_COIL, necho outside 2..FM_MAX_ECHO,
  * bad option), FM_ERR_CUDA, FM_ERR_OOM.
  */

@@ -311,13 +311,14 @@ bool lex_less(const int* a, const int* b) {
 }
 
 // Form of the drop-tolerance IC's base pattern: which sweeps take rows, which levels (k_ict.cu).  A plane
-// of the row wavefront follows the one below by a group of 32 rows (64 steps) where planes have several
-// groups, by a few steps where they have one; by levels it follows after three, which cost a barrier each.
-// The ratio of the two chains, in steps per level, decides; the factor pays the most per step.  ms of
-// ic_factor / ic_apply by levels and by rows (droptol 0.02, no mask, FP32): 256x256x128 (ratio 8) 16.3 / 12.4
-// and 12.1 / 6.8; 96x96x96 (11) 6.5 / 4.8 and 6.3 / 3.6; 64x64x96 (13) 5.0 / 3.8 and 5.5 / 3.1; 64x64x128 (15) 6.1 /
-// 4.7 and 7.1 / 4.0; 64x64x256 (17) 10.6 / 7.8 and 13.6 / 8.0; 32x33x256 (19) 8.7 / 6.6 and 12.1 / 7.1; with one group
-// to a plane, 256x32x256 (2) 14.1 / 10.9 and 8.4 / 4.1.
+// of the row wavefront starts about 8 steps behind the one below (one hand-off) where planes have one group
+// of 32 rows, 11 (two) where they have several, and a step takes about 2.5 us in the factor and 1.2 in the
+// back substitution; by levels a plane follows after three, at about 5 us each.  So many planes of several
+// groups go faster by levels, the factor first.  The weights of `steps` and the two lines are fitted to measurements.
+// ms of ic_factor / ic_apply by levels and by rows (droptol 0.02, no mask, FP32; steps / levels in brackets):
+// 256x256x128 (8) 16.3 / 12.4 and 12.1 / 6.8; 96x96x96 (11) 6.5 / 4.8 and 6.3 / 3.6; 64x64x96 (13) 5.0 / 3.8 and
+// 5.5 / 3.1; 64x64x128 (15) 6.1 / 4.7 and 7.1 / 4.0; 64x64x256 (17) 10.6 / 7.8 and 13.6 / 8.0; 32x33x256 (19) 8.7 / 6.6
+// and 12.1 / 7.1; with one group to a plane, 256x32x256 (2) 14.1 / 10.9 and 8.4 / 4.1.
 enum IctForm { kIctRows, kIctLevelFactor /* factor by levels, the rest by rows */, kIctLevels };
 IctForm ict_form(int nx, int ny, int nz) {
     const long long nyb = (ny + 31) / 32;

@@ -33,9 +33,9 @@ static_assert(kTX == 64 && kTY == 16 && kWarps == 4, "lane = (y, plane of the wa
 // Steps per chunk (the unit of the face hand-off, of the barrier between the warps and of
 // their lag), and the warps that fetch incoming faces, taking the chunks in turn, so that the
 // polls for consecutive chunks are in flight together (a poll round trip is about 0.7 us, a chunk
-// 0.2 to 0.4).  Forward / back substitution on 256 x 256 x 128 (us): chunks of 4 with 2 fetch warps
-// 122 / 97, with 3 125 / 98, with 4 127 / 103; chunks of 3 with 3 130 / 95, of 2 with 4 146 / 101,
-// of 6 with 2 126 / 104.
+// 0.2 to 0.4).  Forward / back substitution on 256 x 256 x 128 (us), measured before the dot products
+// moved behind the back substitution (which made it 109): chunks of 4 with 2 fetch warps 122 / 97, with 3
+// 125 / 98, with 4 127 / 103; chunks of 3 with 3 130 / 95, of 2 with 4 146 / 101, of 6 with 2 126 / 104.
 constexpr int kCSF = FM_IC_CSF, kCSB = FM_IC_CSB;
 constexpr int kFetchF = FM_IC_FWF, kFetchB = FM_IC_FWB;
 // compute warps, one warp that publishes the outgoing faces, fetch warps

@@ -316,7 +316,8 @@ __device__ __forceinline__ void eval_fixed(const DataArgs& a, long long j, T w, 
 // FP32 literal curvature of up to NR coils (two coils per instruction, so NR is even) and any
 // echo count: a pair's coil weights in registers, coils past a.nc counting as |W| = 0.  Bound by
 // FP32 issue at 6 slots per term of NR^2; the runtime-count form it replaces took 11 to 15 per
-// term.  133 x 117 x 45 voxels, four coils and echoes: line search 163 -> 129 us, gradient 32 -> 28.
+// term.  133 x 117 x 45 voxels, four coils and echoes: line search 163 -> 129 us, gradient 32 -> 28
+// (96 and 30 in the present build).
 template <int NR, bool COST, bool CURV>
 __device__ __forceinline__ void eval_padded(const DataArgs& a, long long j, float w, float& cost, float& grad,
                                             float& curv) {
@@ -578,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && NC == 1 ? 4 : 2) k
 // The direction phase leaves each voxel's (z, w) in compact order (a.zw), so that a step's loads
 // all follow from the loop index: with z and w behind the voxel list, and the data term's loads
 // behind a test of z, a voxel cost three dependent memory round trips before its arithmetic
-// (256 x 256 x 128, eight coils: 722 -> 684 us).  Every thread visits the same voxels in both
+// (256 x 256 x 128, eight coils: 722 -> 681 us).  Every thread visits the same voxels in both
 // phases (one grid-stride mapping), so it reads back only what it wrote itself -- but for the
 // lane-shared form, where the grid barrier between the phases orders the two.
 //
@@ -588,8 +589,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 && NC == 1 ? 4 : 2) k
 // rest leave before the first grid barrier, which then counts the nb participants only.
 // Resident blocks per SM of the line search: compiled for, and the most that its grid takes
 // (ls_max_blocks_per_sm), as each thread's voxels and the order of every sum follow from the grid and
-// should not from the compiler's register count.  128 registers for eight coils in registers and the lane-shared form
-// (whose polynomial constants otherwise do not stay in registers), 64 to 80 for the others.
+// should not from the compiler's register count.  128 registers for eight coils in registers and more than
+// eight coils (whose polynomial constants otherwise do not stay in registers), 64 to 80 for the others.
 template <typename T, int NC> constexpr int ls_blocks() {
     constexpr int n = sizeof(T) == 8 ? (NC == 0 ? 3 : 2) : NC == 8 || NC < 0 || NC > kPadded + 4 ? 2 : NC > kPadded ? 3 : 4;
     static_assert(n <= kLsMaxBlocks, "a context's partials buffer holds kLsMaxBlocks blocks per SM");

@@ -265,8 +265,8 @@ __global__ void __launch_bounds__(1024) k_ic_order(TileLists a) { list_tiles(a, 
 // the pattern when the context is created and after a device error.
 //
 // Extra warps per CTA fetch the faces: chunk by chunk (a few steps each), they poll the
-// entries the chunk needs (bounded, with a short sleep), copies them into shared memory and
-// signals the compute warps through a shared-memory counter.  The compute warps synchronise
+// entries the chunk needs (bounded, with a short sleep), copy them into shared memory and
+// hand the chunk to the compute warps through an mbarrier.  The compute warps synchronise
 // among themselves with a named barrier and never poll global memory.
 
 template <int NT>
@@ -345,8 +345,9 @@ __device__ __forceinline__ void st_rlx(double2* a, double2 v) {
 }
 
 // Chunk hand-off from the fetch warp to the compute warps: one mbarrier per chunk with an
-// arrival count of 1, completing one phase per tile (the wait parity is the CTA's tile count
-// & 1).  The fetch warp's lane 0 arrives (release) once the chunk's faces are in shared
+// arrival count of 1, completing one phase per tile that has the chunk.  Tiles sweep their own steps
+// only, so the chunks' barriers run on by themselves: the wait parity is bit c of `par`, flipped with
+// each tile that had chunk c.  The fetch warp's lane 0 arrives (release) once the chunk's faces are in shared
 // memory; the compute warps wait with try_wait (acquire), which suspends the warp instead of
 // spinning and, unlike an acquire load, does not wait for the warp's own outstanding global
 // stores to drain.

@@ -298,10 +298,12 @@ __global__ void __launch_bounds__(kIctThreads) k_ict_bwd(IctArgs a) {
 // block waits for has claimed before it.  Only steps that reach a mask voxel are walked and handed
 // over.  The back substitution is the same walk mirrored.
 //
-// A step is a chain of FP64 operations (one warp per SM: 16 cycles an operation), a block runs as
-// far behind plane z-1 as the hand-off takes, and no barrier is left: 74 x 74 x 10 voxels, 32 coils,
-// factor + forward 1012 -> 606 us, back substitution 904 -> 254; the level sweeps pay about 4 us on
-// each of 247 levels.
+// No barrier is left, and a block runs as far behind plane z-1 as the hand-off takes: 74 x 74 x 10 voxels,
+// 32 coils, factor + forward 1012 -> 606 us, back substitution 904 -> 254; the level sweeps pay about 4 us
+// on each of 247 levels.  A step of the factor takes about 2.5 us (512 x 512 x 1 voxels: 4.0 ms for a walk of
+// 1520 steps), of which its chain of FP64 operations (one warp per SM: 16 cycles an operation, 600 cycles)
+// is 0.3.  The rest is not taken apart; beside the chain a step loads its inputs two steps ahead and stores
+// seven planes, at addresses a row apart from lane to lane.
 
 constexpr int kRec = 6;  // doubles of a record: R, Y, A, B, D, F (1/L_ii, y and the entries others use)
 
